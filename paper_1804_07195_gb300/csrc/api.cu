@@ -405,6 +405,7 @@ hmc_status hmc_destroy(hmc_ctx* c) {
   if (c->tickets) cudaFree(c->tickets);
   if (c->sc) cudaFree(c->sc);
   if (c->gbar) cudaFree(c->gbar);
+  if (c->tile_sync) cudaFree(c->tile_sync);
   if (c->loop_trips) cudaFree(c->loop_trips);
   if (c->loop_trips_host) cudaFreeHost(c->loop_trips_host);
   for (int i = 0; i < hmc_ctx::kBatchSlots; ++i)

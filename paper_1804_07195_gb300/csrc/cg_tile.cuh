@@ -1,0 +1,862 @@
+// CG on resident tiles: a whole solve of (M M^dagger + sigma) x = b (Section 3;
+// the inner solver of Algorithm A.1) in one launch, every vector of the
+// iteration kept on the chip. One group of thread blocks holds one system: all
+// blocks of a cooperative launch (CL = false), or the blocks of one thread
+// block cluster (CL = true; many clusters of one launch solve many systems).
+//
+// Tiles. A block owns all n cells of J rows and T time slices. p and
+// u = M^dagger p of the tile live in shared memory, each of the four arrays
+// p_A, p_B, u_A, u_B padded by the one row and the one slice of neighbouring
+// tiles its stencil reads (Eq. ferm_op: the A rows of M^dagger read p_B at
+// (i, j), (i-1, j), (i, j-1) and p_A at t+1; the B rows read p_A at (i, j),
+// (i+1, j), (i, j+1) and p_B at t-1; M reads u the same way with the time hops
+// reversed); the i-neighbours wrap inside the tile. A thread owns a column:
+// CW neighbouring cells of one row over S time slices, whose r and x stay in
+// its registers, and walks up in time, so that a time neighbour it has just
+// read is carried instead of read again.
+//
+// Iteration:
+//   P  x += alpha p (the previous iteration's), p = r + beta p, on the tile and
+//      on the padding of p (from the neighbours' r at the padding's cells: the
+//      same operation on the same numbers as in the tile that owns them);
+//   U  u = M^dagger p (u_A kept with its sign changed, so that no own value is
+//      negated in either stencil); the tile's edges of u handed to the neighbours;
+//      <p, A p> = |u|^2 + sigma |p|^2 summed over the group;
+//   M  r -= alpha (M u + sigma p); the tile's edges of r handed to the
+//      neighbours; |r|^2 summed over the group.
+// Padding slices beyond t = nt - 1 or before t = 0 hold the anti-periodic
+// continuation (negated values), so the time hops carry no sign of their own.
+//
+// Between blocks of a cooperative launch edges go through global memory (r
+// itself and U), read with L2-only loads. A sum is one arrival word on which
+// every block adds (a reduction that returns nothing: the parity a block waits
+// for is its own count of exchanges) and polls, then warp 0 gathers the
+// blocks' partials while the other warps fetch the edges. Every wait is
+// bounded: a block that gives up marks the launch, and all leave.
+// Between blocks of a cluster edges and partials are stored straight into the
+// other blocks' shared memory, and a cluster barrier (arrive.release,
+// wait.acquire) publishes both.
+//
+// Every sum is formed in a fixed order that is the same in every block, so
+// all blocks of a group hold the same scalars and leave together. FP32 sums
+// are float-float pairs, FP64 sums doubles.
+//
+// What bounds an FP32 iteration of a cooperative launch (us, 2070 MHz; in
+// brackets the design before it, which read r, x and phi from L2 row by row in
+// both halves and published p as well):
+//   6x6x16 6.4 (9.0)   12x12x32 6.8 (8.6)   36x36x64 5.9 (7.5)
+//   51x51x64 7.9 (11.6)   72x72x64 8.2 (11.8)   102x102x64 14.1 (16.2)
+// The two exchanges take about 2 us each (arrival and poll of one L2 word 1.4,
+// the gather or the edges 0.5), whatever the lattice. The rest is, at
+// 102x102x64, shared memory (4.3 us of wavefronts), instruction issue (4.1) and
+// L2 (x streamed, phi twice, edges: 2.4 us at 64 B a cycle and SM), which the
+// phases overlap only in part. Tried and not kept: every block polling every
+// block's packet (one trip less, but the polls of 18,000 packet reads delay
+// the writes: 8.5 to 10.7 us at 36x36x64); x held in registers at 102x102x64
+// (7 slices a column, 384 threads: 14.6 us, too few warps); 3 slices a column
+// (832 threads, spills: 14.0); instances for tiles without a ragged edge
+// (13.9); one warp adding up all threads' values (14.7).
+#pragma once
+
+#include "kernels.h"
+#include "operator.cuh"
+
+namespace hmc {
+
+constexpr int kTileMaxGroup = 160;  // blocks of a cooperative launch at most (partials: 5 per lane)
+constexpr int kTileMaxCluster = 16;
+constexpr int kTileMaxWarps = 32;
+
+// One system on its tiles (J, T nominal: the last tile of a direction may be
+// smaller). Pointers to the solve's vectors in the precision of the kernel.
+struct TileSys {
+  Geo g;
+  int J, T, tiles_j, tiles_t;
+  int nseg;      // columns are cut into nseg pieces of S slices
+  int tab, rp;   // shared memory: the padding's table; (CL) the neighbours' r at the padding
+  FastDiv fq;    // division by the columns of a row, n / CW
+  const void* ph;  // FP32: phi as float, in [-pi, pi]; FP64: e^{i phi}
+  void *x, *r, *U;
+  CGScal* sc;
+};
+
+// Exchanges of a cooperative launch.
+struct GridSync {
+  double* part;    // [2][kTileMaxGroup] partials, 8 bytes each: the exchanges alternate
+  unsigned* word;  // arrivals: the top bit flips when every block has arrived
+  int* err;        // a block gave up
+  unsigned need;   // arrivals an exchange waits for
+  long long limit; // SM cycles
+};
+
+// ---------------------------------------------------------------------------
+// CW neighbouring complex values as (re, im) of a lane type L: two cells are
+// packed FP32 pairs, (re0, re1) and (im0, im1), so that every operation of the
+// stencil but the shift to the i-neighbour is one packed instruction; each lane
+// is rounded as the scalar instruction would round it.
+template <typename R, int CW>
+struct Lane;
+template <>
+struct Lane<float, 1> {
+  using L = float;
+  using V = float2;  // storage of (re, im)
+  static __device__ __forceinline__ L set(float a) { return a; }
+};
+template <>
+struct Lane<float, 2> {
+  using L = unsigned long long;
+  using V = ulonglong2;
+  static __device__ __forceinline__ L set(float a) { return pk2(Cx<float>{a, a}); }
+};
+template <>
+struct Lane<double, 1> {
+  using L = double;
+  using V = double2;
+  static __device__ __forceinline__ L set(double a) { return a; }
+};
+__device__ __forceinline__ float lfma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double lfma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ unsigned long long lfma(unsigned long long a, unsigned long long b, unsigned long long c) {
+  return fma_x2(a, b, c);
+}
+__device__ __forceinline__ float ladd(float a, float b) { return a + b; }
+__device__ __forceinline__ double ladd(double a, double b) { return a + b; }
+__device__ __forceinline__ unsigned long long ladd(unsigned long long a, unsigned long long b) { return add_x2(a, b); }
+__device__ __forceinline__ float lneg(float a) { return -a; }
+__device__ __forceinline__ double lneg(double a) { return -a; }
+__device__ __forceinline__ unsigned long long lneg(unsigned long long a) { return a ^ 0x8000000080000000ull; }
+// own cells + their neighbours at i - 1 (w: the column to the left) or i + 1
+__device__ __forceinline__ float add_left(float own, float w) { return own + w; }
+__device__ __forceinline__ double add_left(double own, double w) { return own + w; }
+__device__ __forceinline__ unsigned long long add_left(unsigned long long own, unsigned long long w) {
+  const Cx<float> o = upk2(own), l = upk2(w);
+  return pk2(Cx<float>{o.re + l.im, o.im + o.re});
+}
+__device__ __forceinline__ float add_right(float own, float w) { return own + w; }
+__device__ __forceinline__ double add_right(double own, double w) { return own + w; }
+__device__ __forceinline__ unsigned long long add_right(unsigned long long own, unsigned long long w) {
+  const Cx<float> o = upk2(own), r = upk2(w);
+  return pk2(Cx<float>{o.re + o.im, o.im + r.re});
+}
+
+template <typename L>
+struct CV {
+  L re, im;
+};
+__device__ __forceinline__ CV<float> unpack(float2 a) { return CV<float>{a.x, a.y}; }
+__device__ __forceinline__ CV<unsigned long long> unpack(ulonglong2 a) { return CV<unsigned long long>{a.x, a.y}; }
+__device__ __forceinline__ CV<double> unpack(double2 a) { return CV<double>{a.x, a.y}; }
+__device__ __forceinline__ float2 pack(CV<float> a) { return make_float2(a.re, a.im); }
+__device__ __forceinline__ ulonglong2 pack(CV<unsigned long long> a) { return make_ulonglong2(a.re, a.im); }
+__device__ __forceinline__ double2 pack(CV<double> a) { return make_double2(a.re, a.im); }
+// between the lanes and the vectors' own layout (re0, im0, re1, im1)
+__device__ __forceinline__ float2 swizzle(float2 a) { return a; }
+__device__ __forceinline__ double2 swizzle(double2 a) { return a; }
+__device__ __forceinline__ ulonglong2 swizzle(ulonglong2 a) {
+  const Cx<float> x = upk2(a.x), y = upk2(a.y);
+  return make_ulonglong2(pk2(Cx<float>{x.re, y.re}), pk2(Cx<float>{x.im, y.im}));
+}
+// a x + y
+template <typename L>
+__device__ __forceinline__ CV<L> vaxpy(L a, CV<L> x, CV<L> y) {
+  return CV<L>{lfma(a, x.re, y.re), lfma(a, x.im, y.im)};
+}
+template <typename L>
+__device__ __forceinline__ CV<L> vneg_if(CV<L> x, bool neg) {
+  return neg ? CV<L>{lneg(x.re), lneg(x.im)} : x;
+}
+// own + (f + i g) v, gm = -g
+template <typename L>
+__device__ __forceinline__ CV<L> hop_time(CV<L> own, L f, L g, L gm, CV<L> v) {
+  return CV<L>{lfma(f, v.re, lfma(gm, v.im, own.re)), lfma(f, v.im, lfma(g, v.re, own.im))};
+}
+// t + d (b + left of b + w)  /  t + d (a + right of a + w)
+template <typename L>
+__device__ __forceinline__ CV<L> hops_left(CV<L> t, L d, CV<L> b, CV<L> left, CV<L> w) {
+  return CV<L>{lfma(d, ladd(add_left(b.re, left.re), w.re), t.re), lfma(d, ladd(add_left(b.im, left.im), w.im), t.im)};
+}
+template <typename L>
+__device__ __forceinline__ CV<L> hops_right(CV<L> t, L d, CV<L> a, CV<L> right, CV<L> w) {
+  return CV<L>{lfma(d, ladd(add_right(a.re, right.re), w.re), t.re),
+               lfma(d, ladd(add_right(a.im, right.im), w.im), t.im)};
+}
+
+// Running sum of |v|^2 of one thread.
+template <typename L>
+struct SqAcc {
+  L s = L(0);
+  __device__ __forceinline__ void add(CV<L> a) { s = lfma(a.re, a.re, lfma(a.im, a.im, s)); }
+};
+__device__ __forceinline__ float total(SqAcc<float> a) { return a.s; }
+__device__ __forceinline__ double total(SqAcc<double> a) { return a.s; }
+__device__ __forceinline__ float total(SqAcc<unsigned long long> a) {
+  const Cx<float> t = upk2(a.s);
+  return t.re + t.im;
+}
+
+// Phases of a column's cells at one slice: the raw load (issued a slice ahead)
+// and dm - cos phi, sin phi, -sin phi made of it.
+template <typename R, int CW>
+struct PhLd;
+template <>
+struct PhLd<float, 1> {
+  using raw = float;
+  static __device__ __forceinline__ raw load(const void* ph, int k) { return __ldg((const float*)ph + k); }
+  static __device__ __forceinline__ void get(raw f, float dm, float& c, float& s, float& sm) {
+    float co;
+    __sincosf(f, &s, &co);
+    c = dm - co;
+    sm = -s;
+  }
+};
+template <>
+struct PhLd<float, 2> {
+  using raw = float2;
+  static __device__ __forceinline__ raw load(const void* ph, int k) { return __ldg((const float2*)ph + k); }
+  static __device__ __forceinline__ void get(raw f, unsigned long long dm, unsigned long long& c, unsigned long long& s,
+                                             unsigned long long& sm) {
+    float s0, c0, s1, c1;
+    __sincosf(f.x, &s0, &c0);
+    __sincosf(f.y, &s1, &c1);
+    const unsigned long long m1 = pk2(Cx<float>{-1.f, -1.f});
+    c = fma_x2(pk2(Cx<float>{c0, c1}), m1, dm);
+    s = pk2(Cx<float>{s0, s1});
+    sm = pk2(Cx<float>{-s0, -s1});
+  }
+};
+template <>
+struct PhLd<double, 1> {
+  using raw = double2;
+  static __device__ __forceinline__ raw load(const void* ph, int k) { return __ldg((const double2*)ph + k); }
+  static __device__ __forceinline__ void get(raw f, double dm, double& c, double& s, double& sm) {
+    c = dm - f.x;
+    s = f.y;
+    sm = -f.y;
+  }
+};
+
+// Sums over the group.
+template <typename R>
+struct Red;
+template <>
+struct Red<float> {
+  using T = float2;
+  static __device__ __forceinline__ T zero() { return make_float2(0.f, 0.f); }
+  static __device__ __forceinline__ T make(float a) { return make_float2(a, 0.f); }
+  // TwoSum of the high parts, the errors gathered in the low one without
+  // renormalising: the chain from one step to the next is a single addition.
+  static __device__ __forceinline__ T add(T a, T b) {
+    const float s = a.x + b.x;
+    const float v = s - a.x;
+    return make_float2(s, ((a.x - (s - v)) + (b.x - v)) + (a.y + b.y));
+  }
+  static __device__ __forceinline__ T shfl(T a, int o) {
+    return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
+  }
+  static __device__ __forceinline__ float value(T a) { return a.x + a.y; }
+};
+template <>
+struct Red<double> {
+  using T = double;
+  static __device__ __forceinline__ T zero() { return 0.0; }
+  static __device__ __forceinline__ T make(double a) { return a; }
+  static __device__ __forceinline__ T add(T a, T b) { return a + b; }
+  static __device__ __forceinline__ T shfl(T a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+  static __device__ __forceinline__ double value(T a) { return a; }
+};
+template <typename R>
+__device__ __forceinline__ typename Red<R>::T warp_sum(typename Red<R>::T v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = Red<R>::add(v, Red<R>::shfl(v, o));
+  return v;
+}
+
+// ---------------------------------------------------------------------------
+// Arrival word (CL = false).
+__device__ __forceinline__ void red_add_release(unsigned* p, unsigned x) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(x) : "memory");
+}
+
+// Warp 0: the sum of all blocks' partials, in every lane.
+template <typename R>
+__device__ __forceinline__ typename Red<R>::T gather(const double* part, int G) {
+  using T = typename Red<R>::T;
+  constexpr int L = kTileMaxGroup / 32;
+  const int lane = threadIdx.x & 31;
+  T w[L];
+#pragma unroll
+  for (int k = 0; k < L; ++k)
+    w[k] = lane + 32 * k < G ? __ldcg((const T*)part + lane + 32 * k) : Red<R>::zero();
+  T v = w[0];
+#pragma unroll
+  for (int k = 1; k < L; ++k) v = Red<R>::add(v, w[k]);
+  return warp_sum<R>(v);
+}
+
+// ---------------------------------------------------------------------------
+// Distributed shared memory (CL = true).
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ unsigned cluster_size() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ unsigned mapa(unsigned addr, unsigned rank) {
+  unsigned r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void st_remote(unsigned addr, float2 v) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void st_remote(unsigned addr, ulonglong2 v) {
+  asm volatile("st.shared::cluster.v2.u64 [%0], {%1, %2};" ::"r"(addr), "l"(v.x), "l"(v.y) : "memory");
+}
+__device__ __forceinline__ void st_remote(unsigned addr, double2 v) {
+  asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(addr), "d"(v.x), "d"(v.y) : "memory");
+}
+__device__ __forceinline__ void st_remote(unsigned addr, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
+}
+
+// Bytes from one of the four padded arrays to the next: constant, so that it is
+// an immediate of every access.
+template <bool CL>
+constexpr int tile_array_stride() {
+  return CL ? 44 * 1024 : 52 * 1024;
+}
+
+template <typename R>
+struct TileScal;
+template <>
+struct TileScal<float> {
+  static __device__ __forceinline__ void load(const CGScal* s, float& dm, float& sigma, float& rr, float& thresh) {
+    dm = s->dm32;
+    sigma = s->sigma32;
+    rr = s->rr32;
+    thresh = s->thresh32;
+  }
+};
+template <>
+struct TileScal<double> {
+  static __device__ __forceinline__ void load(const CGScal* s, double& dm, double& sigma, double& rr,
+                                              double& thresh) {
+    dm = s->dm;
+    sigma = s->sigma;
+    rr = s->rr;
+    thresh = s->thresh;
+  }
+};
+
+// ---------------------------------------------------------------------------
+// The value of i, recomputed from here on: keeps the compiler from holding the
+// addresses of every slice in registers from one phase to the next.
+__device__ __forceinline__ int fresh(int i) {
+  asm volatile("" : "+r"(i));
+  return i;
+}
+
+// Registers a thread holds for r of its column.
+template <typename R, int CW, int S>
+constexpr int tile_r_regs() {
+  return (int)sizeof(R) * CW * S;
+}
+template <typename R, int CW, int S>
+constexpr bool tile_x_in_registers() {
+  return tile_r_regs<R, CW, S>() <= 16;
+}
+// Largest block of an instance, from the registers it needs (r, x where it is
+// held, about 60 more for two cells or doubles, 45 for one) and those a thread
+// can have: the warps are dealt to four partitions of 16,384 registers, so 12,
+// 16, 20, 24 or 32 warps get 168, 128, 96, 80 or 64 registers a thread.
+template <typename R, int CW, int S>
+constexpr int tile_max_threads() {
+  const int r = tile_r_regs<R, CW, S>();
+  if (sizeof(R) == 8) return r <= 8 ? 640 : r <= 48 ? 512 : 384;
+  if (CW == 2) return r <= 8 ? 768 : 640;
+  return r <= 8 ? 1024 : 768;
+}
+
+// The solve of one system by the block `tile` of its group. sm: four padded
+// arrays AS bytes apart, the table of the padding (8 bytes a column) and, for CL,
+// the neighbours' r there.
+template <typename R, int CW, int S, bool CL, int AS>
+__device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync& gs, int tile, char* sm) {
+  using LN = Lane<R, CW>;
+  using L = typename LN::L;
+  using V = typename LN::V;
+  using C = CV<L>;
+  using RT = Red<R>;
+  using T = typename RT::T;
+  using PH = PhLd<R, CW>;
+  constexpr int VB = (int)sizeof(V);
+  constexpr int PA = 0, PB = AS, UA = 2 * AS, UB = 3 * AS;
+  const int TAB = ts.tab, RP = ts.rp;
+  __shared__ R s_a, s_ap;
+  __shared__ int s_stop, s_fail;
+  __shared__ T s_red[CL ? 2 * kTileMaxCluster * kTileMaxWarps : kTileMaxWarps];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = (blockDim.x + 31) >> 5;
+  const int m = ts.g.m, nt = ts.g.nt;
+  const int nq = ts.g.n / CW, Vq = ts.g.V / CW, Hq = ts.g.H / CW;  // all indices in columns of CW cells
+  const int J = ts.J, J1 = J + 1, TN = ts.T;
+  const bool used = tile < ts.tiles_j * ts.tiles_t;
+  const int bt = used ? tile / ts.tiles_j : 0, bj = used ? tile - bt * ts.tiles_j : 0;
+  const int j0 = bj * J, t0 = bt * TN;
+  const int Jt = used ? min(J, m - j0) : 0, Tt = used ? min(TN, nt - t0) : 0;
+  // the arrays, each of (T + 1) (J + 1) rows of nq columns:
+  //   p_A, u_B: rows 0..Jt (Jt: the row above) / -1..Jt-1, slices 0..Tt (Tt: the slice after)
+  //   p_B, u_A: rows -1..Jt-1 / 0..Jt, slices -1..Tt-1
+  const int NJ = J1 * nq;  // one slice
+  const bool wlo = t0 == 0, whi = t0 + Tt == nt;
+  const void* ph = ts.ph;
+  V* const rg = (V*)ts.r;
+  V* const xg = (V*)ts.x;
+  V* const Ug = (V*)ts.U;
+  auto lds = [&](int o) { return unpack(*(const V*)(sm + o)); };
+  auto sts = [&](int o, C v) { *(V*)(sm + o) = pack(v); };
+
+  // the thread's column: cells q of row jj, slices s0 .. s0 + S - 1 of the tile.
+  // With o = ((tt (J + 1) + jj) nq + q) VB the cell's values lie at
+  //   p_A(tt) = o, p_A(tt+1) = o + NJ, p_A(jj+1) = o + nq,
+  //   p_B(tt) = o + NJ + nq, p_B(jj-1) = o + NJ, p_B(tt-1) = o + nq,
+  //   u_A(tt) = o + NJ, u_A(tt-1) = o, u_A(jj+1) = o + NJ + nq,
+  //   u_B(tt) = o + nq, u_B(jj-1) = o, u_B(tt+1) = o + NJ + nq
+  // (NJ and nq times VB) of their arrays; the column to the left or right adds
+  // dl or dr.
+  const int row = (int)fdiv((uint32_t)tid, ts.fq), q = tid - row * nq;
+  const int seg = row / J, jj = row - seg * J, s0 = seg * S;
+  const int nrow = J * ts.nseg;
+  const bool act = row < nrow && jj < Jt;
+  const int ns = act ? min(S, Tt - s0) : 0;  // the thread's slices (<= 0: none)
+  const int dl = ((q == 0 ? nq - 1 : q - 1) - q) * VB, dr = ((q == nq - 1 ? 0 : q + 1) - q) * VB;
+  const int oNJ = NJ * VB, oq = nq * VB;
+  const int o_first = ((s0 * J1 + jj) * nq + q) * VB;
+  const int k_first = ((t0 + s0) * m + j0 + jj) * nq + q;  // lattice index of its first slice
+
+  // Padding: lines l = 0 .. 2 T + 2 J - 1 of nq columns each (nominal sizes):
+  // the row below, the row above, the slice before, the slice after. line():
+  // where column qq of line l of p and of u belongs (array and index in it),
+  // its lattice index, and whether the value there continues anti-periodically;
+  // false: no line. The A or B part of the lattice swaps between p and u for
+  // the last two kinds (p's is given).
+  const int lines = used ? 2 * TN + 2 * J : 0;
+  const int jdn = j0 == 0 ? m - 1 : j0 - 1, jup = j0 + Jt >= m ? 0 : j0 + Jt;
+  const int tdn = wlo ? nt - 1 : t0 - 1, tup = whi ? 0 : t0 + Tt;
+  auto line = [&](int l, int qq, int& kind, int& ip, int& iu, int& k) -> bool {
+    if (l < TN) {
+      kind = 0;  // p_B, u_B
+      ip = (l + 1) * NJ + qq;
+      iu = l * NJ + qq;
+      k = Hq + ((t0 + l) * m + jdn) * nq + qq;
+      return l < Tt;
+    }
+    l -= TN;
+    if (l < TN) {
+      kind = 1;  // p_A, u_A
+      ip = (l * J1 + Jt) * nq + qq;
+      iu = ip + NJ;
+      k = ((t0 + l) * m + jup) * nq + qq;
+      return l < Tt;
+    }
+    l -= TN;
+    if (l < J) {
+      kind = 2;  // p_B, u_A
+      ip = (l + 1) * nq + qq;
+      iu = l * nq + qq;
+      k = Hq + (tdn * m + j0 + l) * nq + qq;
+      return l < Jt;
+    }
+    l -= J;
+    kind = 3;  // p_A, u_B
+    ip = (Tt * J1 + l) * nq + qq;
+    iu = ip + nq;
+    k = (tup * m + j0 + l) * nq + qq;
+    return l < Jt;
+  };
+  // The padding's columns, decoded once into a table: shared-memory offsets
+  // over VB of p (low half of .x) and u (high half), lattice index of p with
+  // the sign in the top bit, the step to u's lattice index in the next two.
+  // CL = false: they belong to the warps after the first (which gathers the
+  // partials meanwhile), or to the only warp.
+  const int e_first = CL ? tid : nwarps > 1 ? tid - 32 : tid;
+  const int e_step = CL ? (int)blockDim.x : nwarps > 1 ? (int)blockDim.x - 32 : 32;
+  const int e_end = e_first < 0 ? e_first : lines * nq;
+  uint2* const tab = (uint2*)(sm + TAB);
+  for (int e = e_first; e < e_end; e += e_step) {
+    const int l = (int)fdiv((uint32_t)e, ts.fq);
+    int kind, ip, iu, k;
+    uint2 d = make_uint2(0xffffffffu, 0u);  // no column
+    if (line(l, e - l * nq, kind, ip, iu, k)) {
+      const bool neg = (kind == 2 && wlo) || (kind == 3 && whi);
+      const unsigned a = ((kind == 0 || kind == 2 ? PB : PA) / VB) + ip, b = ((kind == 0 || kind == 3 ? UB : UA) / VB) + iu;
+      d = make_uint2(a | b << 16, (unsigned)k | (neg ? 0x80000000u : 0u) | (kind == 2 ? 1u : kind == 3 ? 2u : 0u) << 29);
+    }
+    tab[e] = d;
+  }
+  auto for_padding = [&](auto&& f) {
+    for (int e = e_first; e < e_end; e += e_step) {
+      const uint2 d = tab[e];
+      if (d.x == 0xffffffffu) continue;
+      const unsigned st = (d.y >> 29) & 3u;
+      const int kp = (int)(d.y & 0x1fffffffu);
+      f(e, (int)(d.x & 0xffffu) * VB, (int)(d.x >> 16) * VB, kp, kp + (st == 1u ? -Hq : st == 2u ? Hq : 0),
+        (d.y >> 31) != 0u);
+    }
+  };
+  unsigned rem_dn = 0, rem_up = 0, rem_bf = 0, rem_af = 0;  // CL: the neighbours' shared memory
+  int JtD = 0, TtP = 0;  // CL: rows of the tile below, slices of the tile before
+  if constexpr (CL) {
+    const int bd = bj == 0 ? ts.tiles_j - 1 : bj - 1, bu = bj == ts.tiles_j - 1 ? 0 : bj + 1;
+    const int tb = bt == 0 ? ts.tiles_t - 1 : bt - 1, ta = bt == ts.tiles_t - 1 ? 0 : bt + 1;
+    const unsigned sb = (unsigned)__cvta_generic_to_shared(sm);
+    rem_dn = mapa(sb, bt * ts.tiles_j + bd);
+    rem_up = mapa(sb, bt * ts.tiles_j + bu);
+    rem_bf = mapa(sb, tb * ts.tiles_j + bj);
+    rem_af = mapa(sb, ta * ts.tiles_j + bj);
+    JtD = min(J, m - bd * J);
+    TtP = min(TN, nt - tb * TN);
+  }
+
+  R dm, sigma, rr, thresh;
+  TileScal<R>::load(ts.sc, dm, sigma, rr, thresh);
+  const L ldm = LN::set(dm), ldk = LN::set(geo_dk(ts.g, R(0))), lndk = LN::set(-geo_dk(ts.g, R(0)));
+  int iter = ts.sc->iter, done = ts.sc->done;
+  const int maxit = ts.sc->maxit;
+  R rr_prev = R(1), pAp = R(0), alpha = R(0), beta = R(0);
+  bool first = true;
+  // exchanges so far; CL = false: its parity is the arrival word's top bit
+  unsigned ep = CL ? 0u : *(const volatile unsigned*)gs.word >> 31;
+
+  // r and x of the thread's cells (A, B). With many slices per column x stays
+  // in memory (in the lanes' layout while the solve runs) and passes through
+  // registers in P, two slices in flight.
+  constexpr bool XREG = tile_x_in_registers<R, CW, S>();
+  C ra[S], rb[S];
+  C xa[XREG ? S : 2], xb[XREG ? S : 2];
+#pragma unroll
+  for (int s = 0; s < S; ++s)
+    if (s < ns) {
+      const int k = k_first + s * Vq;
+      ra[s] = unpack(swizzle(rg[k]));
+      rb[s] = unpack(swizzle(rg[Hq + k]));
+      if (XREG) {
+        xa[XREG ? s : 0] = unpack(swizzle(xg[k]));
+        xb[XREG ? s : 0] = unpack(swizzle(xg[Hq + k]));
+      } else {
+        xg[k] = swizzle(xg[k]);
+        xg[Hq + k] = swizzle(xg[Hq + k]);
+      }
+    }
+  // x += f p (p of the last iteration) and, if asked, p = r + fb p, slice by slice
+  auto x_and_p = [&](R f, R fb, bool newp) {
+    const L lf = LN::set(f), lb = LN::set(fb);
+    int o = fresh(o_first), k = fresh(k_first);
+    if (!XREG) {
+#pragma unroll
+      for (int s = 0; s < 2; ++s)
+        if (s < ns) {
+          xa[s] = unpack(xg[k + s * Vq]);
+          xb[s] = unpack(xg[Hq + k + s * Vq]);
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < S; ++s, o += oNJ, k += Vq)
+      if (s < ns) {
+        const int e = XREG ? s : (s & 1);
+        const C pa = lds(PA + o), pb = lds(PB + o + oNJ + oq);
+        const C na = vaxpy(lf, pa, xa[e]), nb = vaxpy(lf, pb, xb[e]);
+        if (XREG) {
+          xa[e] = na;
+          xb[e] = nb;
+        } else {
+          xg[k] = pack(na);
+          xg[Hq + k] = pack(nb);
+          if (s + 2 < S && s + 2 < ns) {
+            xa[e] = unpack(xg[k + 2 * Vq]);
+            xb[e] = unpack(xg[Hq + k + 2 * Vq]);
+          }
+        }
+        if (newp) {
+          sts(PA + o, vaxpy(lb, pa, ra[s]));
+          sts(PB + o + oNJ + oq, vaxpy(lb, pb, rb[s]));
+        }
+      }
+  };
+  // p = 0 before the first iteration (beta = 0 there), on the tile and its padding
+  for (int e = tid; e < (TN + 1) * NJ; e += blockDim.x) {
+    sts(PA + e * VB, C{L(0), L(0)});
+    sts(PB + e * VB, C{L(0), L(0)});
+  }
+  if (!CL && tid == 0) s_fail = 0;
+  if constexpr (CL) {
+    for_padding([&](int e, int, int, int kp, int, bool neg) {
+      sts(RP + e * VB, vneg_if(unpack(swizzle(rg[kp])), neg));
+    });
+    cluster_barrier();
+  }
+
+  // Sum over the group. CL: in every thread. Otherwise in warp 0; the other
+  // warps run `edges` meanwhile.
+  auto exchange = [&](R loc, auto&& edges, T* out) -> bool {
+    const T wsum = warp_sum<R>(RT::make(loc));
+    ++ep;
+    if constexpr (CL) {
+      const unsigned cs = cluster_size(), me = cluster_rank();
+      T* slots = s_red + (ep & 1u) * kTileMaxCluster * kTileMaxWarps;
+      if (lane < (int)cs) {
+        const unsigned a = (unsigned)__cvta_generic_to_shared(slots + me * nwarps + warp);
+        st_remote(mapa(a, lane), wsum);
+      }
+      cluster_barrier();
+      const int cnt = (int)cs * nwarps;
+      T v = RT::zero();
+      for (int k = lane; k < cnt; k += 32) v = RT::add(v, slots[k]);
+      *out = warp_sum<R>(v);
+      return true;
+    } else {
+      T* part = (T*)(gs.part + (ep & 1u) * kTileMaxGroup);
+      if (lane == 0) s_red[warp] = wsum;
+      __syncthreads();
+      if (warp == 0) {
+        const T v = warp_sum<R>(lane < nwarps ? s_red[lane] : RT::zero());
+        if (lane == 0) {
+          part[tile] = v;
+          __threadfence();  // the block's edges, ordered before this thread by the barrier above
+          red_add_release(gs.word, tile == 0 ? 0x80000000u - (gs.need - 1u) : 1u);
+          const unsigned want = (ep & 1u) << 31;
+          const long long tw = clock64();
+          unsigned spins = 0;
+          while ((ld_acquire_gpu(gs.word) & 0x80000000u) != want) {
+            if ((++spins & 31u) == 0u && (*(volatile int*)gs.err || clock64() - tw > gs.limit)) {
+              atomicExch(gs.err, 1);
+              s_fail = 1;
+              break;
+            }
+          }
+        }
+      }
+      __syncthreads();
+      if (s_fail) return false;
+      if (warp == 0) *out = gather<R>((const double*)part, gridDim.x);
+      if (warp != 0 || nwarps == 1) edges();
+      return true;
+    }
+  };
+
+  for (;;) {
+    if (CL || tid == 0) {
+      if (!done) {
+        if (!isfinite(rr))
+          done = CG_BREAKDOWN;
+        else if (rr <= thresh)
+          done = CG_CONVERGED;
+        else if (iter >= maxit)
+          done = CG_MAXIT;
+      }
+      beta = first ? R(0) : rr / rr_prev;
+    }
+    R fb = beta, fap = alpha;
+    int stop = done;
+    if constexpr (!CL) {
+      if (tid == 0) {
+        s_a = beta;
+        s_ap = alpha;
+        s_stop = done;
+      }
+      __syncthreads();
+      fb = s_a;
+      fap = s_ap;
+      stop = s_fail ? CG_TIMEOUT : s_stop;
+    }
+    if (stop) {
+      done = stop;
+      if (stop != CG_TIMEOUT && fap != R(0)) x_and_p(fap, R(0), false);  // the last iteration's x update
+      break;
+    }
+    // ---- P: the padding (r of the neighbours at hand: rp, or left in place of
+    // the padding of u by the edges below), then the tile
+    {
+      const L lb = LN::set(fb);
+      for_padding([&](int e, int op, int ou, int kp, int, bool neg) {
+        const C v = CL ? lds(RP + e * VB) : first ? vneg_if(unpack(swizzle(__ldcg(rg + kp))), neg) : lds(ou);
+        sts(op, vaxpy(lb, lds(op), v));
+      });
+    }
+    x_and_p(fap, fb, true);
+    // phases of the first slice: A at t + 1, B at t - 1
+    typename PH::raw fa{}, fbt{};
+    if (ns > 0) {
+      const int t = t0 + s0;
+      fa = PH::load(ph, t + 1 == nt ? k_first + Vq - Hq : k_first + Vq);
+      fbt = PH::load(ph, Hq + (t == 0 ? k_first - Vq + Hq : k_first - Vq));
+    }
+    __syncthreads();
+    // ---- U
+    SqAcc<L> acc, accp;
+    if (ns > 0) {
+      int o = fresh(o_first), k = fresh(k_first);
+      C pa = lds(PA + o), pbm = lds(PB + o + oq);
+#pragma unroll
+      for (int s = 0; s < S; ++s, o += oNJ, k += Vq)
+        if (s < ns) {
+          L f0, g0, h0, f1, g1, h1;
+          PH::get(fa, ldm, f0, g0, h0);
+          PH::get(fbt, ldm, f1, g1, h1);
+          if (s + 1 < S && s + 1 < ns) {
+            fa = PH::load(ph, t0 + s0 + s + 2 == nt ? k + 2 * Vq - Hq : k + 2 * Vq);
+            fbt = PH::load(ph, Hq + k);
+          }
+          const C pan = lds(PA + o + oNJ), pb = lds(PB + o + oNJ + oq);
+          const C va = hops_left(hop_time(pa, f0, g0, h0, pan), ldk, pb, lds(PB + o + oNJ + oq + dl), lds(PB + o + oNJ));
+          const C vb = hops_right(hop_time(pb, f1, h1, g1, pbm), lndk, pa, lds(PA + o + dr), lds(PA + o + oq));
+          sts(UA + o + oNJ, va);
+          sts(UB + o + oq, vb);
+          acc.add(va);
+          acc.add(vb);
+          if (sigma != R(0)) {
+            accp.add(pa);
+            accp.add(pb);
+          }
+          // edges the neighbours' M reads: u_A of the bottom row and the last
+          // slice, u_B of the top row and the first slice
+          const int tt = s0 + s;
+          if constexpr (CL) {
+            if (jj == 0) st_remote(rem_dn + UA + (((tt + 1) * J1 + JtD) * nq + q) * VB, pack(va));
+            if (tt == Tt - 1) st_remote(rem_af + UA + (jj * nq + q) * VB, pack(vneg_if(va, whi)));
+            if (jj == Jt - 1) st_remote(rem_up + UB + (tt * NJ + q) * VB, pack(vb));
+            if (tt == 0) st_remote(rem_bf + UB + ((TtP * J1 + jj + 1) * nq + q) * VB, pack(vneg_if(vb, wlo)));
+          } else {
+            if (jj == 0 || tt == Tt - 1) Ug[k] = pack(va);
+            if (jj == Jt - 1 || tt == 0) Ug[Hq + k] = pack(vb);
+          }
+          pa = pan;
+          pbm = pb;
+        }
+    }
+    T tot;
+    bool ok = exchange(total(acc) + (sigma != R(0) ? sigma * total(accp) : R(0)),
+                       [&] {
+                         for_padding([&](int, int, int ou, int, int ku, bool neg) {
+                           sts(ou, vneg_if(unpack(__ldcg(Ug + ku)), neg));
+                         });
+                       },
+                       &tot);
+    // phases of the first slice of M
+    if (ns > 0) {
+      fa = PH::load(ph, k_first);
+      fbt = PH::load(ph, Hq + k_first);
+    }
+    if (CL || tid == 0) {
+      pAp = ok ? RT::value(tot) : R(0);
+      const bool bad = !(pAp > R(0)) || !isfinite(pAp);
+      alpha = bad ? R(0) : rr / pAp;
+      if (bad) done = ok ? CG_BREAKDOWN : CG_TIMEOUT;
+    }
+    R fal = alpha;
+    if constexpr (!CL) {
+      if (tid == 0) {
+        s_a = alpha;
+        s_stop = done;
+      }
+      __syncthreads();
+      fal = s_a;
+      done = s_fail ? CG_TIMEOUT : s_stop;
+    }
+    if (done) break;
+    // ---- M
+    SqAcc<L> accr;
+    if (ns > 0) {
+      const L lal = LN::set(-fal), lsig = LN::set(sigma);
+      int o = fresh(o_first), k = fresh(k_first);
+      C uam = lds(UA + o), ub = lds(UB + o + oq);
+#pragma unroll
+      for (int s = 0; s < S; ++s, o += oNJ, k += Vq)
+        if (s < ns) {
+          L f0, g0, h0, f1, g1, h1;
+          PH::get(fa, ldm, f0, g0, h0);
+          PH::get(fbt, ldm, f1, g1, h1);
+          if (s + 1 < S && s + 1 < ns) {
+            fa = PH::load(ph, k + Vq);
+            fbt = PH::load(ph, Hq + k + Vq);
+          }
+          const C ua = lds(UA + o + oNJ), ubn = lds(UB + o + oNJ + oq);
+          C va = hops_left(hop_time(ua, f0, h0, g0, uam), lndk, ub, lds(UB + o + oq + dl), lds(UB + o));
+          C vb = hops_right(hop_time(ub, f1, g1, h1, ubn), ldk, ua, lds(UA + o + oNJ + dr), lds(UA + o + oNJ + oq));
+          if (sigma != R(0)) {
+            va = vaxpy(lsig, lds(PA + o), va);
+            vb = vaxpy(lsig, lds(PB + o + oNJ + oq), vb);
+          }
+          ra[s] = vaxpy(lal, va, ra[s]);
+          rb[s] = vaxpy(lal, vb, rb[s]);
+          accr.add(ra[s]);
+          accr.add(rb[s]);
+          // edges the neighbours' padding of p needs: r_B of the top row and the
+          // last slice, r_A of the bottom row and the first slice
+          const int tt = s0 + s;
+          if constexpr (CL) {
+            if (jj == Jt - 1) st_remote(rem_up + RP + (tt * nq + q) * VB, pack(rb[s]));
+            if (jj == 0) st_remote(rem_dn + RP + ((TN + tt) * nq + q) * VB, pack(ra[s]));
+            if (tt == Tt - 1) st_remote(rem_af + RP + ((2 * TN + jj) * nq + q) * VB, pack(vneg_if(rb[s], whi)));
+            if (tt == 0) st_remote(rem_bf + RP + ((2 * TN + J + jj) * nq + q) * VB, pack(vneg_if(ra[s], wlo)));
+          } else {
+            if (jj == 0 || tt == 0) rg[k] = pack(ra[s]);
+            if (jj == Jt - 1 || tt == Tt - 1) rg[Hq + k] = pack(rb[s]);
+          }
+          uam = ua;
+          ub = ubn;
+        }
+    }
+    // the neighbours' r waits in the padding of u, which nothing reads until the
+    // next exchange has refilled it (the block's barrier in `exchange` orders
+    // the reads of u above before these writes)
+    ok = exchange(total(accr),
+                  [&] {
+                    for_padding([&](int, int, int ou, int kp, int, bool neg) {
+                      sts(ou, vneg_if(unpack(__ldcg(rg + kp)), neg));
+                    });
+                  },
+                  &tot);
+    if (CL || tid == 0) {
+      rr_prev = rr;
+      if (ok)
+        rr = RT::value(tot);
+      else
+        done = CG_TIMEOUT;
+    }
+    ++iter;
+    first = false;
+  }
+#pragma unroll
+  for (int s = 0; s < S; ++s)
+    if (s < ns) {
+      const int k = k_first + s * Vq;
+      if (XREG) {
+        xg[k] = swizzle(pack(xa[XREG ? s : 0]));
+        xg[Hq + k] = swizzle(pack(xb[XREG ? s : 0]));
+      } else {
+        xg[k] = swizzle(xg[k]);
+        xg[Hq + k] = swizzle(xg[Hq + k]);
+      }
+    }
+  if (tile == 0 && tid == 0) {
+    CGScal* sc = ts.sc;
+    sc->rr = rr;
+    sc->rr_cur = rr;
+    sc->rr32 = sc->rr_cur32 = (float)rr;
+    sc->pAp = pAp;
+    sc->alpha = alpha;
+    sc->beta = beta;
+    sc->iter = iter;
+    sc->first = 0;
+    sc->done = done ? done : CG_MAXIT;
+  }
+}
+
+}  // namespace hmc

@@ -143,6 +143,31 @@ __device__ __forceinline__ R norm2(Cx<R> a) {
   return a.re * a.re + a.im * a.im;
 }
 
+// Packed FP32 pair arithmetic (add.rn.f32x2, fma.rn.f32x2; sm_100 and
+// later): each lane is rounded as the scalar instruction would round it, so
+// a sum formed this way equals the scalar one bit for bit.
+__device__ __forceinline__ unsigned long long pk2(Cx<float> v) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(v.re), "f"(v.im));
+  return r;
+}
+__device__ __forceinline__ Cx<float> upk2(unsigned long long v) {
+  Cx<float> r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.re), "=f"(r.im) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ unsigned long long add_x2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long fma_x2(unsigned long long a, unsigned long long b,
+                                                     unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
 // ---------------------------------------------------------------------------
 // Deterministic grid reductions.
 //

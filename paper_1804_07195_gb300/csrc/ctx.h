@@ -105,6 +105,17 @@ struct FusedShape {
   int pairs = 0;  // FP32: two cells per thread (n and Ti even; 16-byte aligned vectors)
 };
 
+// Tiles of the resident-tile CG (cg_tile.cuh) and the kernel instance that runs
+// them.
+struct TilePlan {
+  int cw = 0;       // cells per column (0: not searched yet, -1: does not fit)
+  int S = 1;        // slices per column
+  int J = 0, T = 0, tiles_j = 0, tiles_t = 0, nseg = 1;
+  int threads = 0;  // whole warps
+  int tab = 0, rp = 0;  // shared-memory offsets
+  size_t smem = 0;
+};
+
 struct ProfileState {
   bool timing = false;
   long long launches[K_COUNT] = {};
@@ -141,6 +152,11 @@ struct hmc_ctx {
   double* dscal = nullptr;         // device scalar results (64 doubles)
   double* dscal_host = nullptr;    // pinned mirror
   int max_grid = 0;
+  // resident-tile CG: the memory of its exchanges (stale: to be cleared before
+  // the next launch), and the plans of this lattice ([cells per column - 1])
+  void* tile_sync = nullptr;
+  bool tile_sync_stale = false;
+  hmc::TilePlan tile_plan32[2];
 
   hmc::ProfileState prof;
 

@@ -336,30 +336,6 @@ __device__ __forceinline__ Cx<float> lo_c(const float4& v) { return Cx<float>{v.
 __device__ __forceinline__ Cx<float> hi_c(const float4& v) { return Cx<float>{v.z, v.w}; }
 __device__ __forceinline__ float4 pack4(Cx<float> a, Cx<float> b) { return make_float4(a.re, a.im, b.re, b.im); }
 
-// Packed FP32 pair arithmetic (add.rn.f32x2, fma.rn.f32x2; sm_100 and
-// later): each lane is rounded as the scalar instruction would round it, so
-// a sum formed this way equals the scalar one bit for bit.
-__device__ __forceinline__ unsigned long long pk2(Cx<float> v) {
-  unsigned long long r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(v.re), "f"(v.im));
-  return r;
-}
-__device__ __forceinline__ Cx<float> upk2(unsigned long long v) {
-  Cx<float> r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.re), "=f"(r.im) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ unsigned long long add_x2(unsigned long long a, unsigned long long b) {
-  unsigned long long r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ unsigned long long fma_x2(unsigned long long a, unsigned long long b,
-                                                     unsigned long long c) {
-  unsigned long long r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
 // hopsum with both components in one packed pair: t - dk (a + b + c);
 // ndk = (-dk, -dk)
 __device__ __forceinline__ Cx<float> hopsum_x2(Cx<float> t, unsigned long long ndk, Cx<float> a, Cx<float> b,

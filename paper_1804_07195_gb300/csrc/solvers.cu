@@ -309,7 +309,7 @@ hmc_status cg_core(hmc_ctx* c, double ms, double sigma, const V2<R>* b, V2<R>* x
                               cg32_persist_ok(c, g));
     if (persistent) {
       if (resident)
-        HMC_TRY(cg32_resident_launch(c, g, (float2*)x, (float2*)r, (float2*)p, (float2*)q, (float2*)u, sc));
+        HMC_TRY(cg32_resident_launch(c, g, (float2*)x, (float2*)r, (float2*)u, sc));
       else
         HMC_TRY(cg32_persist_launch(c, g, (float2*)x, (float2*)r, (float2*)p, (float2*)q, (float2*)u, sc));
       HMC_CUDA(c, cudaMemcpyAsync(sch, sc, sizeof(CGScal), cudaMemcpyDeviceToHost, c->stream));
@@ -437,6 +437,7 @@ hmc_status cg_core(hmc_ctx* c, double ms, double sigma, const V2<R>* b, V2<R>* x
     st->true_rel = bb > 0 ? std::sqrt(rr / bb) : 0.0;
     if (sizeof(R) == 8) st->applies64++; else st->applies32++;
   }
+  if (sch->done == CG_TIMEOUT) c->tile_sync_stale = true;
   if (sch->done == CG_TIMEOUT) return fail(c, HMC_ERR_TIMEOUT, "persistent CG: a grid barrier wait gave up");
   if (sch->done == CG_BREAKDOWN) return fail(c, HMC_ERR_NAN, "CG breakdown: non-positive or non-finite curvature/residual");
   if (sch->done == CG_MAXIT) return fail(c, HMC_ERR_NOT_CONVERGED, "CG reached its iteration limit");
