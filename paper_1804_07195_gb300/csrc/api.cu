@@ -586,6 +586,7 @@ hmc_status hmc_set_cg_variant(hmc_ctx* c, int variant) {
   c->persist32 = false;
   c->cg1_32 = false;
   c->resident32 = false;
+  c->cluster32 = false;
   destroy_graphs(c);
   return HMC_OK;
 }

@@ -22,16 +22,12 @@ __global__ void __launch_bounds__(tile_max_threads<float, 2, S>(), 1) k_cg32_res
 }
 
 // Slices per column of the kernel instances (0 ends the list).
-template <typename R>
-static const int* tile_slices(int cw) {
+const int* tile_slices32(int cw) {
   static const int one[] = {1, 2, 4, 8, 0}, two[] = {1, 2, 4, 0};
   return cw == 2 ? two : one;
 }
 
-template <typename R>
-static int max_threads_of(int cw, int S);
-template <>
-int max_threads_of<float>(int cw, int S) {
+int max_threads32(int cw, int S) {
   if (cw == 1) switch (S) {
       case 1: return tile_max_threads<float, 1, 1>();
       case 2: return tile_max_threads<float, 1, 2>();
@@ -52,15 +48,14 @@ static size_t smem_cap(const hmc_ctx* c, size_t statics) {
   return optin > (int)statics ? (size_t)optin - statics : 0;
 }
 
-template <typename R>
-bool tile_plan_grid(const hmc_ctx* c, const Geo& g, int cw, TilePlan* out) {
+static bool plan_grid32(const hmc_ctx* c, const Geo& g, int cw, TilePlan* out) {
   if (g.n % cw) return false;
   const size_t cap = smem_cap(c, 2048);  // static arrays and the driver's 1 KB
   constexpr size_t AS = tile_array_stride<false>();
   const int nq = g.n / cw;
   bool found = false;
   double best = 0.0;
-  for (const int* S = tile_slices<R>(cw); *S; ++S)
+  for (const int* S = tile_slices32(cw); *S; ++S)
     for (int nseg = 1, fits = 1; fits && (nseg - 1) * *S < g.nt; ++nseg)
       for (int J = 1; J <= g.m; ++J) {
         TilePlan p;
@@ -71,10 +66,10 @@ bool tile_plan_grid(const hmc_ctx* c, const Geo& g, int cw, TilePlan* out) {
         p.T = nseg * *S;
         p.tiles_j = (g.m + J - 1) / J;
         p.tiles_t = (g.nt + p.T - 1) / p.T;
-        const size_t one = (size_t)(p.T + 1) * (J + 1) * g.n * 2 * sizeof(R);
+        const size_t one = (size_t)(p.T + 1) * (J + 1) * g.n * sizeof(float2);
         const long long th = ((long long)nq * J * nseg + 31) / 32 * 32;
         const size_t table = (size_t)2 * (p.T + J) * nq * sizeof(uint2);
-        if (one > AS || 3 * AS + one + table > cap || th > max_threads_of<R>(cw, *S)) {
+        if (one > AS || 3 * AS + one + table > cap || th > max_threads32(cw, *S)) {
           fits = J > 1;  // larger J, and for J = 1 larger nseg, only grow them
           break;
         }
@@ -95,7 +90,6 @@ bool tile_plan_grid(const hmc_ctx* c, const Geo& g, int cw, TilePlan* out) {
       }
   return found;
 }
-template bool tile_plan_grid<float>(const hmc_ctx*, const Geo&, int, TilePlan*);
 
 TileSys make_tile_sys(const Geo& g, const TilePlan& p, const void* ph, void* x, void* r, void* U, CGScal* sc) {
   TileSys ts;
@@ -153,11 +147,24 @@ static hmc_status grid_sync(hmc_ctx* c, int blocks, GridSync* gs) {
 // The context's plan for its lattice with cw cells per column, searched once.
 static const TilePlan* plan32(hmc_ctx* c, const Geo& g, int cw) {
   TilePlan& p = c->tile_plan32[cw - 1];
-  if (p.cw == 0 && !tile_plan_grid<float>(c, g, cw, &p)) p.cw = -1;
+  if (p.cw == 0 && !plan_grid32(c, g, cw, &p)) p.cw = -1;
   return p.cw > 0 ? &p : nullptr;
 }
 
 bool cg32_resident_ok(hmc_ctx* c, const Geo& g) { return plan32(c, g, 2) || plan32(c, g, 1); }
+
+bool cg32_prefer_cluster(hmc_ctx* c, const Geo& g) {
+  if (!cg32_cluster_ok(c, g)) return false;
+  const TilePlan* p = plan32(c, g, 2);
+  if (!p) p = plan32(c, g, 1);
+  if (!p) return true;
+  // us per iteration over all SMs: two exchanges through L2, phase latency, work
+  // (measured: 5.9 at 36x36x64, 8.2 at 72x72x64); cluster_us has the cluster's.
+  // The line between them runs near 100,000 sites (measured: 24x24x48 4.5 us on a
+  // cluster, 6.2 over all SMs)
+  const double cols = (double)p->J * std::min(p->T, g.nt) * (g.n / p->cw) * (p->cw == 2 ? 1.0 : 0.75);
+  return c->cluster_us < 5.2 + 2.6e-3 * cols;
+}
 
 hmc_status cg32_resident_launch(hmc_ctx* c, const Geo& g, float2* x, float2* r, float2* u, CGScal* sc) {
   // two cells per column where n is even and every vector is 16-byte aligned
@@ -167,8 +174,7 @@ hmc_status cg32_resident_launch(hmc_ctx* c, const Geo& g, float2* x, float2* r, 
   if (!pp) return fail(c, HMC_ERR_INVALID, "resident CG tiles do not fit on chip");
   const TilePlan& p = *pp;
   const void* kfn = grid_kernel32(p.cw, p.S);
-  if (cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem) != cudaSuccess)
-    return cuda_fail(c, cudaGetLastError(), "resident CG shared memory");
+  if (!tile_allow_smem(c, kfn)) return fail(c, HMC_ERR_CUDA, "resident CG shared memory");
   const int blocks = p.tiles_j * p.tiles_t;
   int occ = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kfn, p.threads, p.smem) != cudaSuccess ||

@@ -6,14 +6,23 @@
 
 namespace hmc {
 
-// Tiles for one cooperative launch: every tile resident, within the shared
-// memory a block may use. Among the plans that fit, the one with the fewest
-// cells per tile, then the fewest padding rows and slices per cell.
-template <typename R>
-bool tile_plan_grid(const hmc_ctx* c, const Geo& g, int cw, TilePlan* out);
-// Tiles for one cluster of cs blocks (cs = 1, 2, 4, 8 or 16).
-template <typename R>
-bool tile_plan_cluster(const hmc_ctx* c, const Geo& g, int cw, int cs, TilePlan* out);
+// Slices per column of the FP32 kernel instances (0 ends the list) and their
+// largest blocks.
+const int* tile_slices32(int cw);
+int max_threads32(int cw, int S);
+
+// Lets kernel k use all the shared memory a block may have (the same value for
+// every caller, so that plans of different lattices do not undo each other's).
+inline bool tile_allow_smem(const hmc_ctx* c, const void* k) {
+  int optin = 0;
+  cudaFuncAttributes a;
+  if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device) == cudaSuccess &&
+      cudaFuncGetAttributes(&a, k) == cudaSuccess &&
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)a.sharedSizeBytes) == cudaSuccess)
+    return true;
+  cudaGetLastError();
+  return false;
+}
 
 TileSys make_tile_sys(const Geo& g, const TilePlan& p, const void* ph, void* x, void* r, void* U, CGScal* sc);
 

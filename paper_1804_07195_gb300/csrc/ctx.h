@@ -113,6 +113,7 @@ struct TilePlan {
   int J = 0, T = 0, tiles_j = 0, tiles_t = 0, nseg = 1;
   int threads = 0;  // whole warps
   int tab = 0, rp = 0;  // shared-memory offsets
+  int stride = 0;       // bytes between the padded arrays (clusters)
   size_t smem = 0;
 };
 
@@ -157,6 +158,10 @@ struct hmc_ctx {
   void* tile_sync = nullptr;
   bool tile_sync_stale = false;
   hmc::TilePlan tile_plan32[2];
+  // the same on one thread block cluster (log2 of its blocks; -2: not looked for yet, -1: none)
+  int cluster_log2 = -2;
+  double cluster_us = 0.0;  // estimate per iteration
+  hmc::TilePlan cluster_plan;
 
   hmc::ProfileState prof;
 
@@ -169,6 +174,7 @@ struct hmc_ctx {
   bool persist32 = false;  // the tuner found the persistent FP32 CG kernel fastest
   bool cg1_32 = false;     // the tuner found the single-reduction FP32 CG fastest
   bool resident32 = false;  // the tuner found the resident-tile FP32 CG fastest
+  bool cluster32 = false;   // the tuner found it fastest on one cluster
   bool cg1_pinned = false;  // its tile was set by the caller
   hmc::FusedShape cg1_shape;  // tile of the single-reduction FP32 CG kernel
   // M M^dagger applications: 0 = choose per precision by timing on first use,

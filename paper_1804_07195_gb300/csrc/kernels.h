@@ -61,6 +61,11 @@ hmc_status set_cg1_shape(hmc_ctx* c, int Ti, int Tj, int Tt, int D);
 // chip; false / HMC_ERR_INVALID when the tiles do not fit there.
 bool cg32_resident_ok(hmc_ctx* c, const Geo& g);
 hmc_status cg32_resident_launch(hmc_ctx* c, const Geo& g, float2* x, float2* r, float2* u, CGScal* sc);
+// The same on one thread block cluster (small lattices).
+bool cg32_cluster_ok(hmc_ctx* c, const Geo& g);
+hmc_status cg32_cluster_launch(hmc_ctx* c, const Geo& g, float2* x, float2* r, CGScal* sc);
+// Whether the cluster is expected to be the faster of the two.
+bool cg32_prefer_cluster(hmc_ctx* c, const Geo& g);
 
 // CG building blocks on the state sc (see common.cuh).
 template <typename R>

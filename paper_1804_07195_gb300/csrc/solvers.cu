@@ -4,6 +4,7 @@
 // convergence flag every few iterations and only reads back small scalars.
 #include <cmath>
 #include <complex>
+#include <cstdint>
 #include <vector>
 
 #include "solvers.h"
@@ -170,6 +171,7 @@ static hmc_status tune_cg(hmc_ctx* c, double ms, double sigma, const V2<R>* b) {
     c->persist32 = false;
     c->cg1_32 = false;
     c->resident32 = false;
+    c->cluster32 = false;
     bool cg1_fit = false;
     if ((var == 0 || var == 6) && !c->capturing) {
       const CG1Bufs B = cg1_bufs(c, (float2*)r);
@@ -187,16 +189,17 @@ static hmc_status tune_cg(hmc_ctx* c, double ms, double sigma, const V2<R>* b) {
     if (var == 6) c->cg1_32 = cg1_fit;
     if (var == 0 && !c->capturing) {
       struct Design {
-        bool persist, cg1, resident;
+        bool persist, cg1, resident, cluster;
         int fam;  // pair family whose shapes the design runs (-1: the overall fastest)
       };
       std::vector<Design> designs;
       for (int f = 0; f < 5; ++f)
-        if (fam_t[f] < 1e30f) designs.push_back({false, false, false, f});
-      if (designs.empty()) designs.push_back({false, false, false, -1});
-      if (cg32_persist_ok(c, g)) designs.push_back({true, false, false, -1});
-      if (cg1_fit) designs.push_back({false, true, false, -1});
-      if (cg32_resident_ok(c, g)) designs.push_back({false, false, true, -1});
+        if (fam_t[f] < 1e30f) designs.push_back({false, false, false, false, f});
+      if (designs.empty()) designs.push_back({false, false, false, false, -1});
+      if (cg32_persist_ok(c, g)) designs.push_back({true, false, false, false, -1});
+      if (cg1_fit) designs.push_back({false, true, false, false, -1});
+      if (cg32_resident_ok(c, g)) designs.push_back({false, false, true, false, -1});
+      if (cg32_cluster_ok(c, g)) designs.push_back({false, false, false, true, -1});
       auto use_shapes = [&](int f) {
         for (int k = 0; k < nk; ++k) c->shape[ids[k]] = f >= 0 ? fam[f][k] : keep[k];
       };
@@ -206,6 +209,7 @@ static hmc_status tune_cg(hmc_ctx* c, double ms, double sigma, const V2<R>* b) {
         c->persist32 = designs[k].persist;
         c->cg1_32 = designs[k].cg1;
         c->resident32 = designs[k].resident;
+        c->cluster32 = designs[k].cluster;
         use_shapes(designs[k].fam);
         destroy_graphs(c);  // graphs hold the launch shapes they were captured with
         float tm = 1e30f;
@@ -219,6 +223,7 @@ static hmc_status tune_cg(hmc_ctx* c, double ms, double sigma, const V2<R>* b) {
             c->persist32 = false;
             c->cg1_32 = false;
             c->resident32 = false;
+            c->cluster32 = false;
             cudaEventDestroy(e0);
             cudaEventDestroy(e1);
             return st;
@@ -236,6 +241,7 @@ static hmc_status tune_cg(hmc_ctx* c, double ms, double sigma, const V2<R>* b) {
       c->persist32 = best_d.persist;
       c->cg1_32 = best_d.cg1;
       c->resident32 = best_d.resident;
+      c->cluster32 = best_d.cluster;
       use_shapes(best_d.fam);
       destroy_graphs(c);
     }
@@ -300,15 +306,21 @@ hmc_status cg_core(hmc_ctx* c, double ms, double sigma, const V2<R>* b, V2<R>* x
   // pinned variant) chose it
   bool persistent = false;
   if constexpr (sizeof(R) == 4) {
-    // the resident-tile kernel (one launch per solve, p and M^dagger p of
-    // each tile in shared memory) when the tuner or the pinned variant chose it
-    const bool resident = !c->capturing &&
-                          (c->cg32_variant == 7 || (c->cg32_variant == 0 && c->resident32)) &&
+    // the resident-tile kernel (one launch per solve) when the tuner or the
+    // pinned variant chose it: on one cluster, or over all SMs (there with the
+    // bounded waits of the wait test)
+    const bool pinned = c->cg32_variant == 7, tuned = c->cg32_variant == 0;
+    const bool cluster = !c->capturing && c->bar_extra == 0 &&
+                         ((pinned && cg32_prefer_cluster(c, g)) || (tuned && c->cluster32)) && cg32_cluster_ok(c, g) &&
+                         ((g.n & 1) || ((uintptr_t)x & 15u) == 0);  // pairs of cells are 16-byte accesses
+    const bool resident = !c->capturing && !cluster && (pinned || (tuned && (c->resident32 || c->cluster32))) &&
                           cg32_resident_ok(c, g);
-    persistent = resident || (!c->capturing && (c->cg32_variant == 4 || (c->cg32_variant == 0 && c->persist32)) &&
-                              cg32_persist_ok(c, g));
+    const bool whole = resident || cluster;
+    persistent = whole || (!c->capturing && (c->cg32_variant == 4 || (tuned && c->persist32)) && cg32_persist_ok(c, g));
     if (persistent) {
-      if (resident)
+      if (cluster)
+        HMC_TRY(cg32_cluster_launch(c, g, (float2*)x, (float2*)r, sc));
+      else if (resident)
         HMC_TRY(cg32_resident_launch(c, g, (float2*)x, (float2*)r, (float2*)u, sc));
       else
         HMC_TRY(cg32_persist_launch(c, g, (float2*)x, (float2*)r, (float2*)p, (float2*)q, (float2*)u, sc));
@@ -318,7 +330,7 @@ hmc_status cg_core(hmc_ctx* c, double ms, double sigma, const V2<R>* b, V2<R>* x
       // design keeps on chip: the operator with its dot (p and phi read, A p
       // written: 20 B, here rounded with the dot to 24 B), x and r updated
       // with the norm (48 B), p updated (24 B)
-      c->prof.bytes[resident ? K_CG_RES32 : K_CG_PERSIST32] += 96.0 * g.N * sch->iter;
+      c->prof.bytes[whole ? K_CG_RES32 : K_CG_PERSIST32] += 96.0 * g.N * sch->iter;
     }
   }
   // FP32: one single-reduction launch per iteration when the tuner (or the
