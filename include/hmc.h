@@ -334,13 +334,16 @@ hmc_status hmc_set_cg_variant(hmc_ctx* ctx, int variant);
 
 /* The FP32 CG of hmc_solve_batched (mixed = 1) runs in one of two designs:
  * 1 = a captured graph whose device-side loop repeats chunks of per-iteration
- * kernels (two launches per iteration over all systems); 2 = one persistent
- * cooperative launch per inner solve, whose blocks walk the systems' blocks
- * and separate the halves of an iteration by grid barriers (bounded waits: a
- * wait that gives up returns HMC_ERR_TIMEOUT). variant 0 (default) runs the
- * first inner solve of the context with 1 and the second with 2 and keeps the
- * one with the shorter time per iteration; 1 or 2 pins one. The variant in
- * use (0 = not chosen yet) is reported by hmc_batched_variant. */
+ * kernels (two launches per iteration over all systems); 2 = persistent
+ * launches that run the whole inner solve: every system on a thread block
+ * cluster of its own, none waiting for another, where all of them fit one (up
+ * to about 130,000 sites each), else one cooperative launch whose blocks walk
+ * the systems' blocks and separate the halves of an iteration by grid barriers
+ * (bounded waits: a wait that gives up returns HMC_ERR_TIMEOUT). variant 0
+ * (default) takes the clusters where they fit; otherwise it runs the first
+ * inner solve of the context with 1 and the second with 2 and keeps the one
+ * with the shorter time per iteration; 1 or 2 pins one. The variant in use
+ * (0 = not chosen yet) is reported by hmc_batched_variant. */
 hmc_status hmc_set_batched_variant(hmc_ctx* ctx, int variant);
 hmc_status hmc_batched_variant(hmc_ctx* ctx, int* variant);
 

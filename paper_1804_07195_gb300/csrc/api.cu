@@ -406,6 +406,11 @@ hmc_status hmc_destroy(hmc_ctx* c) {
   if (c->sc) cudaFree(c->sc);
   if (c->gbar) cudaFree(c->gbar);
   if (c->tile_sync) cudaFree(c->tile_sync);
+  for (int i = 0; i < hmc_ctx::kSideStreams; ++i) {
+    if (c->side[i]) cudaStreamDestroy(c->side[i]);
+    if (c->side_done[i]) cudaEventDestroy(c->side_done[i]);
+  }
+  if (c->side_start) cudaEventDestroy(c->side_start);
   if (c->loop_trips) cudaFree(c->loop_trips);
   if (c->loop_trips_host) cudaFreeHost(c->loop_trips_host);
   for (int i = 0; i < hmc_ctx::kBatchSlots; ++i)

@@ -14,12 +14,15 @@
 // mixed = 0: CG in FP64 to |r| <= tol |b|.
 // mixed = 1: FP64 defect correction: r = b - A x in FP64, an FP32 CG solve of
 //            A e = r, x += e, repeated until the FP64 true residual meets tol.
+//            The FP32 solves run on thread block clusters, one per system,
+//            where every system fits one (cg32_cluster.cu).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <map>
 #include <vector>
 
+#include "cg_tile.h"
 #include "operator.cuh"
 #include "solvers.h"
 #include "trace.h"
@@ -233,6 +236,11 @@ __global__ void kb_init(const BSys* __restrict__ sys, const int* __restrict__ bs
     bst[s_].alpha32 = bst[s_].beta32 = 0.f;
     c.done = (!bst[s_].active || tot[0] <= c.thresh) ? CG_CONVERGED : CG_RUNNING;
     if (!isfinite(tot[0])) c.done = CG_BREAKDOWN;
+    c.dm = S_.dm;
+    c.dm32 = S_.dm32;
+    c.sigma32 = S_.sigma32;
+    c.rr32 = (float)tot[0];
+    c.thresh32 = (float)c.thresh;
   }
 }
 
@@ -488,6 +496,10 @@ struct BatchWs {
   double2 *E = nullptr, *x = nullptr, *b = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *u = nullptr;
   float *phi32 = nullptr;
   float2 *r32 = nullptr, *e32 = nullptr, *p32v = nullptr, *q32v = nullptr, *u32 = nullptr, *rr32 = nullptr;
+  // FP32 CG on clusters: the launches, and their systems' descriptors
+  bool clusters = false;
+  std::vector<ClusterGroup> groups;
+  TileSys* tsys = nullptr;
   int nalloc = 0;  // pool slots taken by this call
   std::vector<void*> allocs;
 };
@@ -700,6 +712,21 @@ static hmc_status batched_cg(hmc_ctx* c, BatchWs& w, cudaStream_t s, const V2<R>
   kb_init<R><<<w.blocks, w.threads, 0, s>>>(w.sys, w.bsys, w.st, w.tol2, b, x, r, p, maxit, w.partials,
                                              w.tickets);
   HMC_CUDA(c, cudaGetLastError());
+  if constexpr (sizeof(R) == 4) {
+    if (w.clusters) {
+      c->batch_choice = 2;
+      cudaEvent_t a = nullptr;
+      prof_begin(c, K_BATCH_CG32, &a);
+      const hmc_status st = cg32_cluster_batch_launch(c, w.groups, w.tsys);
+      prof_end(c, K_BATCH_CG32, a);
+      c->prof.launches[K_BATCH_CG32]--;  // prof_begin counted one more
+      HMC_TRY(st);
+      HMC_CUDA(c, cudaMemcpyAsync(w.st_host, w.st, sizeof(BState) * w.nsys, cudaMemcpyDeviceToHost, s));
+      HMC_CUDA(c, cudaStreamSynchronize(s));
+      for (int i = 0; i < w.nsys; ++i) c->prof.bytes[K_BATCH_CG32] += (double)w.st_host[i].cg.iter * w.hsys[i].g.N * 88.0;
+      return HMC_OK;
+    }
+  }
   // systems already done at init (inactive, or converged at start) never pass
   // through kb_cg_m: count them from the states
   HMC_CUDA(c, cudaMemcpyAsync(w.st_host, w.st, sizeof(BState) * w.nsys, cudaMemcpyDeviceToHost, s));
@@ -930,6 +957,33 @@ extern "C" hmc_status hmc_solve_batched(hmc_ctx* c, int nsys, const hmc_system* 
       HMC_TRY(bmalloc(c, w, (void**)&w.u32, sizeof(float2) * Nt));
       HMC_TRY(bmalloc(c, w, (void**)&w.rr32, sizeof(float2) * Nt));
     }
+    // FP32 CG: every system on a cluster of its own where all of them fit one,
+    // unless the graph loop is pinned or the wait test needs the bounded waits
+    // of the cooperative launch
+    if (mixed && c->batch_variant != 1 && c->bar_extra == 0) {
+      std::vector<Geo> geos(nsys);
+      std::vector<double> its(nsys);
+      for (int i = 0; i < nsys; ++i) {
+        const BSys& S = w.hsys[i];
+        geos[i] = S.g;
+        // CG's bound, up to a factor: the lowest mode at phi = 0 with the mass and shift
+        const double sn = 2.0 * std::sin(1.5707963267948966 / S.g.nt);
+        its[i] = 1.0 / std::sqrt(sn * sn + S.dm * S.dm + S.sigma);
+      }
+      w.clusters = cg32_cluster_batch(c, geos, its, &w.groups);
+    }
+    if (w.clusters) {
+      HMC_TRY(bmalloc(c, w, (void**)&w.tsys, sizeof(TileSys) * nsys));
+      std::vector<TileSys> h;
+      for (const ClusterGroup& g : w.groups)
+        for (size_t k = 0; k < g.sys.size(); ++k) {
+          const BSys& S = w.hsys[g.sys[k]];
+          h.push_back(make_tile_sys(S.g, g.plans[k], w.phi32 + S.off, w.e32 + S.off, w.rr32 + S.off, nullptr,
+                                    &w.st[g.sys[k]].cg));
+        }
+      HMC_CUDA(c, cudaMemcpyAsync(w.tsys, h.data(), sizeof(TileSys) * nsys, cudaMemcpyHostToDevice, s));
+      HMC_CUDA(c, cudaStreamSynchronize(s));  // h is pageable and ends here
+    }
     HMC_TRY(bmalloc_host(c, 0, (void**)&w.st_host, sizeof(BState) * nsys));
     HMC_TRY(bmalloc_host(c, 1, (void**)&w.rrbb_host, sizeof(double) * 2 * nsys));
     HMC_TRY(bmalloc_host(c, 2, (void**)&w.ndone_host, sizeof(unsigned)));
@@ -1012,7 +1066,7 @@ extern "C" hmc_status hmc_solve_batched(hmc_ctx* c, int nsys, const hmc_system* 
         if (nact == 0) break;
         HMC_CUDA(c, cudaMemcpyAsync(w.tol2, tol2.data(), sizeof(double) * nsys, cudaMemcpyHostToDevice, s));
         HMC_CUDA(c, cudaMemcpyAsync(w.st, init.data(), sizeof(BState) * nsys, cudaMemcpyHostToDevice, s));
-        if (!tuned) {
+        if (!tuned && !w.clusters) {
           // r32 now holds the first right-hand sides: tune the FP32 block shape on them
           HMC_TRY(autotune<float>(c, w, s, w.e32, w.rr32, w.p32v, w.q32v, w.u32, w.r32, &threads, &ipt));
           plan_blocks(w, threads, ipt);

@@ -4,6 +4,8 @@
 #include "cg_tile.cuh"
 #include "ctx.h"
 
+#include <vector>
+
 namespace hmc {
 
 // Slices per column of the FP32 kernel instances (0 ends the list) and their
@@ -25,5 +27,22 @@ inline bool tile_allow_smem(const hmc_ctx* c, const void* k) {
 }
 
 TileSys make_tile_sys(const Geo& g, const TilePlan& p, const void* ph, void* x, void* r, void* U, CGScal* sc);
+
+// One launch of a batch: systems whose plans share a kernel instance, a cluster
+// size (2^log2 blocks) and a block size. plan: the instance, with the block
+// and the shared memory of the launch.
+struct ClusterGroup {
+  int log2 = 0, threads = 0;
+  TilePlan plan;
+  std::vector<int> sys;        // indices into the batch, longest first
+  std::vector<TilePlan> plans;  // theirs
+};
+// Groups for a batch of systems on the lattices geos; iters: expected
+// iterations, up to a common factor. false: a lattice does not fit a cluster.
+bool cg32_cluster_batch(hmc_ctx* c, const std::vector<Geo>& geos, const std::vector<double>& iters,
+                        std::vector<ClusterGroup>* groups);
+// Solve them all: list holds the systems in the order of the groups; ordered
+// on c->stream.
+hmc_status cg32_cluster_batch_launch(hmc_ctx* c, const std::vector<ClusterGroup>& groups, const TileSys* list);
 
 }  // namespace hmc

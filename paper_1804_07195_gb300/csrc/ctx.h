@@ -4,7 +4,9 @@
 
 #include <cuda_runtime.h>
 
+#include <array>
 #include <functional>
+#include <map>
 #include <string>
 #include <vector>
 
@@ -117,6 +119,13 @@ struct TilePlan {
   size_t smem = 0;
 };
 
+// Plans of one lattice on a cluster of 1, 2, 4, 8 or 16 blocks (cw <= 0: none),
+// with the estimated us per iteration.
+struct ClusterPlans {
+  TilePlan p[5];
+  double us[5];
+};
+
 struct ProfileState {
   bool timing = false;
   long long launches[K_COUNT] = {};
@@ -162,6 +171,12 @@ struct hmc_ctx {
   int cluster_log2 = -2;
   double cluster_us = 0.0;  // estimate per iteration
   hmc::TilePlan cluster_plan;
+  // plans of the lattices of batched solves by (n, m, nt), and the streams on
+  // which a batch's groups of clusters run side by side
+  std::map<std::array<int, 3>, hmc::ClusterPlans> batch_plans;
+  static constexpr int kSideStreams = 8;
+  cudaStream_t side[kSideStreams] = {};
+  cudaEvent_t side_done[kSideStreams] = {}, side_start = nullptr;
 
   hmc::ProfileState prof;
 

@@ -53,3 +53,30 @@ def test_one_cluster(shape, cols):
             assert rel_max(host(x).astype(np.complex128), ref.x) <= 2e-5 * k
         assert ctx.profile_read()["cg_resident_f32"]["design"] == (4 if cols == 2 else 0)
         assert ctx.check_guards() == 0
+
+
+@pytest.mark.parametrize("shapes", [[(24, 24, 33), (7, 5, 9), (36, 36, 48), (25, 3, 17), (6, 6, 16), (1, 2, 3)],
+                                    [(64, 64, 40), (6, 6, 16), (9, 4, 12)]])
+def test_batched_clusters(shapes):
+    """A mixed batch with every system on a cluster of its own (first list), and
+    one with a lattice that fits no cluster (the cooperative kernels take the
+    whole batch): each system's true residual by the oracle's operator."""
+    need_gpu()
+    import paper_1804_07195_gb300 as hmc
+    import torch
+    systems, refs = [], []
+    for k, sh in enumerate(shapes):
+        w = W.small(*sh, seed=1900 + k, U=3.0, beta=6.0)
+        p = w.lat
+        lat = hmc.Lattice(p.n, p.m, p.nt, p.kappa, p.U, p.beta)
+        for ms, sigma in ((0.2, 0.0), (1.0, 0.05)):
+            systems.append({"lattice": lat, "phi": dev(w.phi), "ms": ms, "sigma": sigma, "b": dev(w.b),
+                            "x": torch.empty(p.nsites, dtype=torch.complex128, device="cuda"), "tol": 1e-10})
+            refs.append((w, ms, sigma))
+    with ctx_for(refs[0][0].lat) as ctx:
+        infos = ctx.solve_batched(systems, mixed=True)
+        assert ctx.check_guards() == 0
+    for s, (w, ms, sigma), info in zip(systems, refs, infos):
+        ol = OLat.from_params(w.lat)
+        rel = osv.true_rel_residual(lambda v: of.apply_MMdag(ol, w.phi, ms, v, sigma), host(s["x"]), w.b)
+        assert rel <= 1.0001e-10 and abs(info["true_rel_res"] - rel) <= 1e-13, (w.name, ms, rel, info)
