@@ -48,14 +48,15 @@ static size_t smem_cap(const hmc_ctx* c, size_t statics) {
   return optin > (int)statics ? (size_t)optin - statics : 0;
 }
 
-static bool plan_grid32(const hmc_ctx* c, const Geo& g, int cw, TilePlan* out) {
+bool tile_plan_grid(const hmc_ctx* c, const Geo& g, int cw, int real, const int* slices, int (*max_threads)(int, int),
+                    TilePlan* out) {
   if (g.n % cw) return false;
-  const size_t cap = smem_cap(c, 2048);  // static arrays and the driver's 1 KB
+  const size_t cap = smem_cap(c, real == 8 ? 7168 : 2048);  // static arrays and the driver's 1 KB
   constexpr size_t AS = tile_array_stride<false>();
   const int nq = g.n / cw;
   bool found = false;
   double best = 0.0;
-  for (const int* S = tile_slices32(cw); *S; ++S)
+  for (const int* S = slices; *S; ++S)
     for (int nseg = 1, fits = 1; fits && (nseg - 1) * *S < g.nt; ++nseg)
       for (int J = 1; J <= g.m; ++J) {
         TilePlan p;
@@ -66,10 +67,10 @@ static bool plan_grid32(const hmc_ctx* c, const Geo& g, int cw, TilePlan* out) {
         p.T = nseg * *S;
         p.tiles_j = (g.m + J - 1) / J;
         p.tiles_t = (g.nt + p.T - 1) / p.T;
-        const size_t one = (size_t)(p.T + 1) * (J + 1) * g.n * sizeof(float2);
+        const size_t one = (size_t)(p.T + 1) * (J + 1) * g.n * 2 * real;
         const long long th = ((long long)nq * J * nseg + 31) / 32 * 32;
         const size_t table = (size_t)2 * (p.T + J) * nq * sizeof(uint2);
-        if (one > AS || 3 * AS + one + table > cap || th > max_threads32(cw, *S)) {
+        if (one > AS || 3 * AS + one + table > cap || th > max_threads(cw, *S)) {
           fits = J > 1;  // larger J, and for J = 1 larger nseg, only grow them
           break;
         }
@@ -144,10 +145,30 @@ static hmc_status grid_sync(hmc_ctx* c, int blocks, GridSync* gs) {
   return HMC_OK;
 }
 
+hmc_status tile_grid_launch(hmc_ctx* c, int id, const void* kfn, const TilePlan& p, const TileSys& system) {
+  if (!tile_allow_smem(c, kfn)) return fail(c, HMC_ERR_CUDA, "resident CG shared memory");
+  const int blocks = p.tiles_j * p.tiles_t;
+  int occ = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kfn, p.threads, p.smem) != cudaSuccess ||
+      (long long)occ * c->nsm < blocks) {
+    cudaGetLastError();
+    return fail(c, HMC_ERR_INVALID, "resident CG tiles cannot all be resident");
+  }
+  TileSys ts = system;
+  GridSync gs;
+  HMC_TRY(grid_sync(c, blocks, &gs));
+  void* args[] = {&ts, &gs};
+  cudaError_t le = cudaSuccess;
+  HMC_TRY(launch_b(c, id, 0.0, [&] {
+    le = cudaLaunchCooperativeKernel(kfn, dim3(blocks), dim3(p.threads), args, p.smem, c->stream);
+  }));
+  return le == cudaSuccess ? HMC_OK : cuda_fail(c, le, "resident CG launch");
+}
+
 // The context's plan for its lattice with cw cells per column, searched once.
 static const TilePlan* plan32(hmc_ctx* c, const Geo& g, int cw) {
   TilePlan& p = c->tile_plan32[cw - 1];
-  if (p.cw == 0 && !plan_grid32(c, g, cw, &p)) p.cw = -1;
+  if (p.cw == 0 && !tile_plan_grid(c, g, cw, sizeof(float), tile_slices32(cw), max_threads32, &p)) p.cw = -1;
   return p.cw > 0 ? &p : nullptr;
 }
 
@@ -174,23 +195,8 @@ hmc_status cg32_resident_launch(hmc_ctx* c, const Geo& g, float2* x, float2* r, 
   if (!pp) return fail(c, HMC_ERR_INVALID, "resident CG tiles do not fit on chip");
   const TilePlan& p = *pp;
   const void* kfn = grid_kernel32(p.cw, p.S);
-  if (!tile_allow_smem(c, kfn)) return fail(c, HMC_ERR_CUDA, "resident CG shared memory");
-  const int blocks = p.tiles_j * p.tiles_t;
-  int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kfn, p.threads, p.smem) != cudaSuccess ||
-      (long long)occ * c->nsm < blocks) {
-    cudaGetLastError();
-    return fail(c, HMC_ERR_INVALID, "resident CG tiles cannot all be resident");
-  }
-  TileSys ts = make_tile_sys(g, p, phase_of<float>(c).phi, x, r, u, sc);
-  GridSync gs;
-  HMC_TRY(grid_sync(c, blocks, &gs));
-  void* args[] = {&ts, &gs};
-  cudaError_t le = cudaSuccess;
-  HMC_TRY(launch_b(c, K_CG_RES32, 0.0, [&] {
-    le = cudaLaunchCooperativeKernel(kfn, dim3(blocks), dim3(p.threads), args, p.smem, c->stream);
-  }));
-  if (le != cudaSuccess) return cuda_fail(c, le, "resident CG launch");
+  const TileSys ts = make_tile_sys(g, p, phase_of<float>(c).phi, x, r, u, sc);
+  HMC_TRY(tile_grid_launch(c, K_CG_RES32, kfn, p, ts));
   c->shape[K_CG_RES32].tiled = p.cw == 2 ? 4 : 0;  // reported as the design
   return HMC_OK;
 }

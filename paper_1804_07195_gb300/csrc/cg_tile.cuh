@@ -401,7 +401,11 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
   const int TAB = ts.tab, RP = ts.rp;
   __shared__ R s_a, s_ap;
   __shared__ int s_stop, s_fail;
-  __shared__ T s_red[CL ? 2 * kTileMaxCluster * kTileMaxWarps : kTileMaxWarps];
+  // FP32: the warps' sums. FP64 (CL = false): every thread's value, added up by
+  // one warp: the FP64 pipe takes 16 cycles for a warp's addition, so that five
+  // shuffle steps in every warp cost more than 1400 cycles of a block of 18
+  constexpr bool BYTHREAD = !CL && sizeof(R) == 8;
+  __shared__ T s_red[CL ? 2 * kTileMaxCluster * kTileMaxWarps : BYTHREAD ? tile_max_threads<R, CW, S>() : kTileMaxWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = (blockDim.x + 31) >> 5;
   const int m = ts.g.m, nt = ts.g.nt;
   const int nq = ts.g.n / CW, Vq = ts.g.V / CW, Hq = ts.g.H / CW;  // all indices in columns of CW cells
@@ -605,9 +609,9 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
   // Sum over the group. CL: in every thread. Otherwise in warp 0; the other
   // warps run `edges` meanwhile.
   auto exchange = [&](R loc, auto&& edges, T* out) -> bool {
-    const T wsum = warp_sum<R>(RT::make(loc));
     ++ep;
     if constexpr (CL) {
+      const T wsum = warp_sum<R>(RT::make(loc));
       const unsigned cs = cluster_size(), me = cluster_rank();
       T* slots = s_red + (ep & 1u) * kTileMaxCluster * kTileMaxWarps;
       if (lane < (int)cs) {
@@ -622,10 +626,25 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
       return true;
     } else {
       T* part = (T*)(gs.part + (ep & 1u) * kTileMaxGroup);
-      if (lane == 0) s_red[warp] = wsum;
+      if constexpr (BYTHREAD) {
+        s_red[tid] = RT::make(loc);
+      } else {
+        const T wsum = warp_sum<R>(RT::make(loc));
+        if (lane == 0) s_red[warp] = wsum;
+      }
       __syncthreads();
       if (warp == 0) {
-        const T v = warp_sum<R>(lane < nwarps ? s_red[lane] : RT::zero());
+        T v;
+        if constexpr (BYTHREAD) {
+          T w[4] = {RT::zero(), RT::zero(), RT::zero(), RT::zero()};
+          for (int k = 0; k < nwarps; k += 4)
+#pragma unroll
+            for (int h = 0; h < 4; ++h)
+              if (k + h < nwarps) w[h] = RT::add(w[h], s_red[(k + h) * 32 + lane]);
+          v = warp_sum<R>(RT::add(RT::add(w[0], w[1]), RT::add(w[2], w[3])));
+        } else {
+          v = warp_sum<R>(lane < nwarps ? s_red[lane] : RT::zero());
+        }
         if (lane == 0) {
           part[tile] = v;
           __threadfence();  // the block's edges, ordered before this thread by the barrier above

@@ -50,6 +50,7 @@ enum KernelId {
   K_MMDAG_FUSED64,
   K_CG1_32,
   K_CG_RES32,
+  K_CG_RES64,
   K_COUNT
 };
 
@@ -167,6 +168,8 @@ struct hmc_ctx {
   void* tile_sync = nullptr;
   bool tile_sync_stale = false;
   hmc::TilePlan tile_plan32[2];
+  hmc::TilePlan tile_plan64;
+  bool resident64 = false;  // the tuner found the resident-tile FP64 CG fastest
   // the same on one thread block cluster (log2 of its blocks; -2: not looked for yet, -1: none)
   int cluster_log2 = -2;
   double cluster_us = 0.0;  // estimate per iteration

@@ -64,6 +64,9 @@ hmc_status cg32_resident_launch(hmc_ctx* c, const Geo& g, float2* x, float2* r, 
 // The same on one thread block cluster (small lattices).
 bool cg32_cluster_ok(hmc_ctx* c, const Geo& g);
 hmc_status cg32_cluster_launch(hmc_ctx* c, const Geo& g, float2* x, float2* r, CGScal* sc);
+// The same in FP64, over all SMs.
+bool cg64_resident_ok(hmc_ctx* c, const Geo& g);
+hmc_status cg64_resident_launch(hmc_ctx* c, const Geo& g, double2* x, double2* r, double2* u, CGScal* sc);
 // Whether the cluster is expected to be the faster of the two.
 bool cg32_prefer_cluster(hmc_ctx* c, const Geo& g);
 

@@ -161,6 +161,30 @@ static hmc_status tune_cg(hmc_ctx* c, double ms, double sigma, const V2<R>* b) {
     }
   }
   for (int k = 0; k < nk; ++k) c->shape[ids[k]] = keep[k];
+  // FP64: the three kernels (graph replay) against the resident-tile kernel,
+  // 48 iterations each, twice, best kept
+  if constexpr (sizeof(R) == 8) {
+    c->resident64 = false;
+    if (!c->capturing && c->bar_extra == 0 && cg64_resident_ok(c, g)) {
+      float best_t[2] = {1e30f, 1e30f};
+      for (int d = 0; d < 2; ++d) {
+        c->resident64 = d == 1;
+        for (int rep = 0; rep < 2; ++rep) {
+          SolveStats tmp;
+          HMC_CUDA(c, cudaEventRecord(e0, c->stream));
+          const hmc_status st = cg_core<R>(c, ms, sigma, b, x, true, 1e-30, 48, 2, false, &tmp);
+          HMC_CUDA(c, cudaEventRecord(e1, c->stream));
+          HMC_CUDA(c, cudaEventSynchronize(e1));
+          c->err.clear();
+          float t = 1e30f;
+          if (st == HMC_OK || st == HMC_ERR_NOT_CONVERGED) cudaEventElapsedTime(&t, e0, e1);
+          best_t[d] = std::min(best_t[d], t);
+        }
+      }
+      c->resident64 = best_t[1] < best_t[0];
+      destroy_graphs(c);
+    }
+  }
   // FP32: the single-reduction kernel's tile (variants 0 and 6), then the
   // designs against each other through the solver path they would run in
   // (graph replay with programmatic dependent launch; 48 iterations, twice
@@ -331,6 +355,16 @@ hmc_status cg_core(hmc_ctx* c, double ms, double sigma, const V2<R>* b, V2<R>* x
       // written: 20 B, here rounded with the dot to 24 B), x and r updated
       // with the norm (48 B), p updated (24 B)
       c->prof.bytes[whole ? K_CG_RES32 : K_CG_PERSIST32] += 96.0 * g.N * sch->iter;
+    }
+  }
+  // FP64: the resident-tile kernel when the tuner chose it
+  if constexpr (sizeof(R) == 8) {
+    if (!c->capturing && c->resident64 && c->bar_extra == 0 && cg64_resident_ok(c, g)) {
+      persistent = true;
+      HMC_TRY(cg64_resident_launch(c, g, (double2*)x, (double2*)r, (double2*)u, sc));
+      HMC_CUDA(c, cudaMemcpyAsync(sch, sc, sizeof(CGScal), cudaMemcpyDeviceToHost, c->stream));
+      HMC_CUDA(c, cudaStreamSynchronize(c->stream));
+      c->prof.bytes[K_CG_RES64] += 208.0 * g.N * sch->iter;
     }
   }
   // FP32: one single-reduction launch per iteration when the tuner (or the

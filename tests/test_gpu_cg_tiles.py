@@ -80,3 +80,27 @@ def test_batched_clusters(shapes):
         ol = OLat.from_params(w.lat)
         rel = osv.true_rel_residual(lambda v: of.apply_MMdag(ol, w.phi, ms, v, sigma), host(s["x"]), w.b)
         assert rel <= 1.0001e-10 and abs(info["true_rel_res"] - rel) <= 1e-13, (w.name, ms, rel, info)
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 4), (2, 5, 3), (7, 5, 9), (36, 35, 40), (36, 36, 64), (51, 33, 61),
+                                   (72, 40, 64), (33, 120, 64)])
+def test_fp64_tiles(shape):
+    """The FP64 CG on resident tiles (the context's tuner runs it beside the
+    three-kernel iteration and keeps the faster): x after two iterations and
+    from a starting guess against the oracle's CG."""
+    need_gpu()
+    w = W.small(*shape, seed=2000 + sum(shape))
+    ol = OLat.from_params(w.lat)
+    A = lambda v: of.apply_MMdag(ol, w.phi, 0.2, v, 0.05)
+    k = 1 if w.lat.nsites < 32 else 2
+    ref = osv.cg(A, w.b, tol=1e-30, maxit=k)
+    x0 = 0.1 * w.b
+    ref0 = osv.cg(A, w.b - A(x0), tol=1e-30, maxit=k)
+    with ctx_for(w.lat) as ctx:
+        x, info = ctx.solve_cg(dev(w.phi), 0.2, dev(w.b), sigma=0.05, tol=1e-30, maxit=k, allow_fail=True)
+        assert info["iters"] == k
+        assert rel_max(host(x), ref.x) <= 1e-13
+        x, _ = ctx.solve_cg(dev(w.phi), 0.2, dev(w.b), x=dev(x0), sigma=0.05, tol=1e-30, maxit=k, allow_fail=True)
+        assert rel_max(host(x), x0 + ref0.x) <= 1e-13
+        assert ctx.profile_read()["cg_resident_f64"]["launches"] >= 1
+        assert ctx.check_guards() == 0
