@@ -120,23 +120,38 @@ __device__ __forceinline__ unsigned long long lfma(unsigned long long a, unsigne
   return fma_x2(a, b, c);
 }
 __device__ __forceinline__ float ladd(float a, float b) { return a + b; }
-__device__ __forceinline__ double ladd(double a, double b) { return a + b; }
 __device__ __forceinline__ unsigned long long ladd(unsigned long long a, unsigned long long b) { return add_x2(a, b); }
 __device__ __forceinline__ float lneg(float a) { return -a; }
-__device__ __forceinline__ double lneg(double a) { return -a; }
+__device__ __forceinline__ double lneg(double a) { return dneg_if(a, true); }
 __device__ __forceinline__ unsigned long long lneg(unsigned long long a) { return a ^ 0x8000000080000000ull; }
 // own cells + their neighbours at i - 1 (w: the column to the left) or i + 1
 __device__ __forceinline__ float add_left(float own, float w) { return own + w; }
-__device__ __forceinline__ double add_left(double own, double w) { return own + w; }
 __device__ __forceinline__ unsigned long long add_left(unsigned long long own, unsigned long long w) {
   const Cx<float> o = upk2(own), l = upk2(w);
   return pk2(Cx<float>{o.re + l.im, o.im + o.re});
 }
 __device__ __forceinline__ float add_right(float own, float w) { return own + w; }
-__device__ __forceinline__ double add_right(double own, double w) { return own + w; }
 __device__ __forceinline__ unsigned long long add_right(unsigned long long own, unsigned long long w) {
   const Cx<float> o = upk2(own), r = upk2(w);
   return pk2(Cx<float>{o.re + o.im, o.im + r.re});
+}
+
+// the same + v
+template <typename L>
+__device__ __forceinline__ L sum_left(L own, L w, L v) {
+  return ladd(add_left(own, w), v);
+}
+template <typename L>
+__device__ __forceinline__ L sum_right(L own, L w, L v) {
+  return ladd(add_right(own, w), v);
+}
+template <>
+__device__ __forceinline__ double sum_left(double own, double w, double v) {
+  return sum3(own, w, v);
+}
+template <>
+__device__ __forceinline__ double sum_right(double own, double w, double v) {
+  return sum3(own, w, v);
 }
 
 template <typename L>
@@ -173,12 +188,11 @@ __device__ __forceinline__ CV<L> hop_time(CV<L> own, L f, L g, L gm, CV<L> v) {
 // t + d (b + left of b + w)  /  t + d (a + right of a + w)
 template <typename L>
 __device__ __forceinline__ CV<L> hops_left(CV<L> t, L d, CV<L> b, CV<L> left, CV<L> w) {
-  return CV<L>{lfma(d, ladd(add_left(b.re, left.re), w.re), t.re), lfma(d, ladd(add_left(b.im, left.im), w.im), t.im)};
+  return CV<L>{lfma(d, sum_left(b.re, left.re, w.re), t.re), lfma(d, sum_left(b.im, left.im, w.im), t.im)};
 }
 template <typename L>
 __device__ __forceinline__ CV<L> hops_right(CV<L> t, L d, CV<L> a, CV<L> right, CV<L> w) {
-  return CV<L>{lfma(d, ladd(add_right(a.re, right.re), w.re), t.re),
-               lfma(d, ladd(add_right(a.im, right.im), w.im), t.im)};
+  return CV<L>{lfma(d, sum_right(a.re, right.re, w.re), t.re), lfma(d, sum_right(a.im, right.im, w.im), t.im)};
 }
 
 // Running sum of |v|^2 of one thread.

@@ -137,6 +137,15 @@ template <typename R>
 __device__ __forceinline__ Cx<R> cneg_if(Cx<R> a, bool neg) {
   return neg ? Cx<R>{-a.re, -a.im} : a;
 }
+// FP64: on the sign bits (a negation that is not folded into another
+// instruction is an addition on the slow FP64 pipe).
+__device__ __forceinline__ double dneg_if(double a, bool neg) {
+  return __hiloint2double(__double2hiint(a) ^ (neg ? (int)0x80000000 : 0), __double2loint(a));
+}
+template <>
+__device__ __forceinline__ Cx<double> cneg_if(Cx<double> a, bool neg) {
+  return Cx<double>{dneg_if(a.re, neg), dneg_if(a.im, neg)};
+}
 
 template <typename R>
 __device__ __forceinline__ R norm2(Cx<R> a) {

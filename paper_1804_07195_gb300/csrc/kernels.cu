@@ -4,6 +4,8 @@
 // Passages: the operator of Eq. ferm_op (Section 2), CG (Section 3), the vector
 // steps of Algorithm A.1 (Appendix A), the force of Eqs. p_dot, f_chi_i and
 // def_xi_i, the energies of Eq. hamiltonian.
+#include <type_traits>
+
 #include "kernels.h"
 #include "launch.cuh"
 #include "operator.cuh"
@@ -69,27 +71,28 @@ __global__ void __launch_bounds__(kThreads) k_phase(int N, const double* __restr
 
 
 // out = M^dagger p (Eq. ferm_op, conjugate transpose), one cell-time per thread.
-template <typename R>
+template <typename R, bool MASS>
 __global__ void __launch_bounds__(kThreads) k_mdag(Geo g, Phase<R> ph, R dm,
                                                    const V2<R>* __restrict__ p,
                                                    V2<R>* __restrict__ out) {
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < g.H; q += gridDim.x * blockDim.x) {
     Nbr nb = neighbours(g, q);
-    PairOut<R> o = mdag_pair<R>(g, ph, dm, p, nb);
+    PairOut<R> o = mdag_pair<R, Phase<R>, MASS>(g, ph, dm, p, nb);
     st(out, q, o.a);
     st(out, g.H + q, o.b);
   }
 }
 
-// out = M u (Eq. ferm_op), one cell-time per thread.
-template <typename R>
+// out = M u + sigma y (Eq. ferm_op; SHIFT = false: sigma = 0), one cell-time per
+// thread.
+template <typename R, bool MASS, bool SHIFT>
 __global__ void __launch_bounds__(kThreads) k_m(Geo g, Phase<R> ph, R dm, const V2<R>* __restrict__ u,
                                                 const V2<R>* __restrict__ y, R sigma,
                                                 V2<R>* __restrict__ out) {
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < g.H; q += gridDim.x * blockDim.x) {
     Nbr nb = neighbours(g, q);
-    PairOut<R> o = m_pair<R>(g, ph, dm, u, nb);
-    if (y != nullptr) {
+    PairOut<R> o = m_pair<R, Phase<R>, MASS>(g, ph, dm, u, nb);
+    if (SHIFT) {
       Cx<R> ya = ld<R>(y, q), yb = ld<R>(y, g.H + q);
       o.a.re = fma(sigma, ya.re, o.a.re);
       o.a.im = fma(sigma, ya.im, o.a.im);
@@ -98,6 +101,29 @@ __global__ void __launch_bounds__(kThreads) k_m(Geo g, Phase<R> ph, R dm, const 
     }
     st(out, q, o.a);
     st(out, g.H + q, o.b);
+  }
+}
+
+// acc += |a|^2
+__device__ __forceinline__ void add_norm2(Cx<double> a, double& acc) {
+  acc = fma(a.re, a.re, fma(a.im, a.im, acc));
+}
+__device__ __forceinline__ void add_norm2(Cx<float> a, double& acc) { acc += (double)norm2(a); }
+
+// body(mass, shift) as std::true_type or std::false_type: dm and sigma are zero or not.
+template <typename R, typename F>
+__device__ __forceinline__ void cg_cases(R dm, R sigma, F&& body) {
+  using Y = std::true_type;
+  using N = std::false_type;
+  if (sigma != R(0)) {
+    if (dm != R(0))
+      body(Y{}, Y{});
+    else
+      body(N{}, Y{});
+  } else if (dm != R(0)) {
+    body(Y{}, N{});
+  } else {
+    body(N{}, N{});
   }
 }
 
@@ -113,15 +139,19 @@ __global__ void __launch_bounds__(kMaxThreads) k_cg_mdag(Geo g, Phase<R> ph,
   const R dm = (R)sc->dm;
   const R sigma = (R)sc->sigma;
   double acc[1] = {0.0};
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < g.H; q += gridDim.x * blockDim.x) {
-    Nbr nb = neighbours(g, q);
-    PairOut<R> o = mdag_pair<R>(g, ph, dm, p, nb);
-    st(u, q, o.a);
-    st(u, g.H + q, o.b);
-    R loc = norm2(o.a) + norm2(o.b);
-    if (sigma != (R)0) loc += sigma * (norm2(ld<R>(p, q)) + norm2(ld<R>(p, g.H + q)));
-    acc[0] += (double)loc;
-  }
+  // a loop per case: a predicated-off instruction takes the FP64 pipe too
+  auto body = [&](auto mass, auto shift) {
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < g.H; q += gridDim.x * blockDim.x) {
+      Nbr nb = neighbours(g, q);
+      PairOut<R> o = mdag_pair<R, Phase<R>, decltype(mass)::value>(g, ph, dm, p, nb);
+      st(u, q, o.a);
+      st(u, g.H + q, o.b);
+      R loc = norm2(o.a) + norm2(o.b);
+      if constexpr (decltype(shift)::value) loc += sigma * (norm2(ld<R>(p, q)) + norm2(ld<R>(p, g.H + q)));
+      acc[0] += (double)loc;
+    }
+  };
+  cg_cases(dm, sigma, body);
   pdl_trigger();
   double tot[1];
   if (grid_sum<1>(acc, partials, ticket, tot) && threadIdx.x == 0) {
@@ -150,27 +180,30 @@ __global__ void __launch_bounds__(kMaxThreads) k_cg_m(Geo g, Phase<R> ph,
   const R sigma = (R)sc->sigma;
   const R alpha = (R)sc->alpha;
   double acc[1] = {0.0};
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < g.H; q += gridDim.x * blockDim.x) {
-    Nbr nb = neighbours(g, q);
-    PairOut<R> o = m_pair<R>(g, ph, dm, u, nb);
-    R loc = 0;
+  auto body = [&](auto mass, auto shift) {
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < g.H; q += gridDim.x * blockDim.x) {
+      Nbr nb = neighbours(g, q);
+      PairOut<R> o = m_pair<R, Phase<R>, decltype(mass)::value>(g, ph, dm, u, nb);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int k = h ? g.H + q : q;
-      Cx<R> Ap = h ? o.b : o.a;
-      Cx<R> pk = ld<R>(p, k), xk = ld<R>(x, k), rk = ld<R>(r, k);
-      Ap.re = fma(sigma, pk.re, Ap.re);
-      Ap.im = fma(sigma, pk.im, Ap.im);
-      xk.re = fma(alpha, pk.re, xk.re);
-      xk.im = fma(alpha, pk.im, xk.im);
-      rk.re = fma(-alpha, Ap.re, rk.re);
-      rk.im = fma(-alpha, Ap.im, rk.im);
-      st(x, k, xk);
-      st(r, k, rk);
-      loc += norm2(rk);
+      for (int h = 0; h < 2; ++h) {
+        const int k = h ? g.H + q : q;
+        Cx<R> Ap = h ? o.b : o.a;
+        Cx<R> pk = ld<R>(p, k), xk = ld<R>(x, k), rk = ld<R>(r, k);
+        if constexpr (decltype(shift)::value) {
+          Ap.re = fma(sigma, pk.re, Ap.re);
+          Ap.im = fma(sigma, pk.im, Ap.im);
+        }
+        xk.re = fma(alpha, pk.re, xk.re);
+        xk.im = fma(alpha, pk.im, xk.im);
+        rk.re = fma(-alpha, Ap.re, rk.re);
+        rk.im = fma(-alpha, Ap.im, rk.im);
+        st(x, k, xk);
+        st(r, k, rk);
+        add_norm2(rk, acc[0]);
+      }
     }
-    acc[0] += (double)loc;
-  }
+  };
+  cg_cases(dm, sigma, body);
   pdl_trigger();
   double tot[1];
   if (grid_sum<1>(acc, partials, ticket, tot) && threadIdx.x == 0) {
@@ -624,23 +657,30 @@ __global__ void __launch_bounds__(kThreads) k_resid(Geo g, Phase<R> ph, R dm,
                                                     double dsigma, double ddm, double* out2,
                                                     double* partials, unsigned* ticket) {
   double acc[2] = {0.0, 0.0};
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < g.H; q += gridDim.x * blockDim.x) {
-    Nbr nb = neighbours(g, q);
-    PairOut<R> o = m_pair<R>(g, ph, dm, u, nb);
+  auto body = [&](auto mass, auto shift) {
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < g.H; q += gridDim.x * blockDim.x) {
+      Nbr nb = neighbours(g, q);
+      PairOut<R> o = m_pair<R, Phase<R>, decltype(mass)::value>(g, ph, dm, u, nb);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int k = h ? g.H + q : q;
-      Cx<R> Ax = h ? o.b : o.a;
-      Cx<R> xk = ld<R>(x, k), bk = ld<R>(b, k);
-      Cx<R> rk;
-      rk.re = bk.re - fma(sigma, xk.re, Ax.re);
-      rk.im = bk.im - fma(sigma, xk.im, Ax.im);
-      st(r, k, rk);
-      if (p != nullptr) st(p, k, rk);
-      acc[0] += (double)norm2(rk);
-      acc[1] += (double)norm2(bk);
+      for (int h = 0; h < 2; ++h) {
+        const int k = h ? g.H + q : q;
+        Cx<R> Ax = h ? o.b : o.a;
+        Cx<R> xk = ld<R>(x, k), bk = ld<R>(b, k);
+        Cx<R> rk;
+        if constexpr (decltype(shift)::value) {
+          Ax.re = fma(sigma, xk.re, Ax.re);
+          Ax.im = fma(sigma, xk.im, Ax.im);
+        }
+        rk.re = bk.re - Ax.re;
+        rk.im = bk.im - Ax.im;
+        st(r, k, rk);
+        if (p != nullptr) st(p, k, rk);
+        add_norm2(rk, acc[0]);
+        add_norm2(bk, acc[1]);
+      }
     }
-  }
+  };
+  cg_cases(dm, sigma, body);
   double tot[2];
   if (grid_sum<2>(acc, partials, ticket, tot) && threadIdx.x == 0) {
     if (out2 != nullptr) {
@@ -918,13 +958,31 @@ hmc_status k_phase_launch(hmc_ctx* c, const double* phi) {
 template <typename R>
 hmc_status mdag_launch(hmc_ctx* c, const Geo& g, R dm, const V2<R>* p, V2<R>* out) {
   return launch(c, sizeof(R) == 8 ? K_MDAG64 : K_MDAG32,
-                [&] { k_mdag<R><<<GRID(g.H)>>>(g, phase_of<R>(c), dm, p, out); });
+                [&] {
+                  if (dm != R(0))
+                    k_mdag<R, true><<<GRID(g.H)>>>(g, phase_of<R>(c), dm, p, out);
+                  else
+                    k_mdag<R, false><<<GRID(g.H)>>>(g, phase_of<R>(c), dm, p, out);
+                });
 }
 template <typename R>
 hmc_status m_launch(hmc_ctx* c, const Geo& g, R dm, const V2<R>* u, const V2<R>* y, R sigma,
                     V2<R>* out) {
   return launch(c, sizeof(R) == 8 ? K_M64 : K_M32,
-                [&] { k_m<R><<<GRID(g.H)>>>(g, phase_of<R>(c), dm, u, y, sigma, out); });
+                [&] {
+                  // an instance per case: a predicated-off instruction takes the FP64 pipe too
+                  const Phase<R> ph = phase_of<R>(c);
+                  if (dm != R(0)) {
+                    if (y != nullptr)
+                      k_m<R, true, true><<<GRID(g.H)>>>(g, ph, dm, u, y, sigma, out);
+                    else
+                      k_m<R, true, false><<<GRID(g.H)>>>(g, ph, dm, u, y, sigma, out);
+                  } else if (y != nullptr) {
+                    k_m<R, false, true><<<GRID(g.H)>>>(g, ph, dm, u, y, sigma, out);
+                  } else {
+                    k_m<R, false, false><<<GRID(g.H)>>>(g, ph, dm, u, y, sigma, out);
+                  }
+                });
 }
 template <typename R>
 hmc_status cg_mdag_launch(hmc_ctx* c, const Geo& g, const V2<R>* p, V2<R>* u, CGScal* sc,

@@ -49,12 +49,46 @@ __device__ __forceinline__ Cx<R> cfma(Cx<R> z, Cx<R> v, Cx<R> c) {
   return o;
 }
 
+// One addend of sum3 as a signed fixed-point number whose scale is that of the
+// exponent field em: the leading bit of a number of that exponent is bit 60.
+__device__ __forceinline__ long long sum3_aligned(double a, int em) {
+  const int h = __double2hiint(a);
+  const int d = (int)((unsigned)(em - (h & 0x7ff00000)) >> 20);
+  const unsigned long long m =
+      ((unsigned long long)(unsigned)((h & 0x000fffff) | 0x00100000) << 32) | (unsigned)__double2loint(a);
+  return (long long)((m << 8) >> min(d, 63)) ^ (long long)(h >> 31);
+}
+
+// Out of line, or its additions would be issued (with a false predicate) beside
+// every integer sum and take the FP64 pipe all the same.
+static __device__ __noinline__ double sum3_rare(double a, double b, double c) { return (a + b) + c; }
+
+// a + b + c in integer arithmetic, rounded once: 61-bit addends relative to the
+// largest, so the error is below 0.5 ulp of the sum plus 3/256 ulp of the
+// largest addend, where two FP64 additions may err by 1 ulp. The FP64 pipe of
+// this GPU takes 16 cycles for a warp's addition, and the integer one is idle.
+__device__ __forceinline__ double sum3(double a, double b, double c) {
+  const int em = max(max(__double2hiint(a) & 0x7ff00000, __double2hiint(b) & 0x7ff00000), __double2hiint(c) & 0x7ff00000);
+  // infinities, NaN, sums that may overflow, the smallest normal numbers and zeros
+  if ((unsigned)(em - 0x04000000) >= 0x7bc00000u) return sum3_rare(a, b, c);
+  const long long v = sum3_aligned(a, em) + sum3_aligned(b, em) + sum3_aligned(c, em);
+  const long long s = v >> 63;
+  const unsigned long long w = (unsigned long long)(v ^ s);
+  const int lz = __clzll((long long)w);  // at least 1
+  const unsigned long long r = (((w << (lz & 63)) >> 1) + 0x200ull) >> 10;  // 53 bits
+  const int e = em + ((2 - lz) << 20);
+  const unsigned long long bits =
+      (r + ((unsigned long long)(unsigned)e << 32)) | ((unsigned long long)s & 0x8000000000000000ull);
+  return w ? __longlong_as_double((long long)bits) : 0.0;
+}
+__device__ __forceinline__ float sum3(float a, float b, float c) { return a + b + c; }
+
 // t - dk (a + b + c)
 template <typename R>
 __device__ __forceinline__ Cx<R> hopsum(Cx<R> t, R dk, Cx<R> a, Cx<R> b, Cx<R> c) {
   Cx<R> o;
-  o.re = fma(-dk, a.re + b.re + c.re, t.re);
-  o.im = fma(-dk, a.im + b.im + c.im, t.im);
+  o.re = fma(-dk, sum3(a.re, b.re, c.re), t.re);
+  o.im = fma(-dk, sum3(a.im, b.im, c.im), t.im);
   return o;
 }
 
@@ -63,9 +97,24 @@ struct PairOut {
   Cx<R> a, b;
 };
 
+// The time-hop factors +-(cos phi - dm, +-sin phi): MASS = false for dm = 0, which
+// then costs no subtraction (1 of the 8 FP64 instructions left in a row).
+template <bool MASS, typename R>
+__device__ __forceinline__ R less_dm(R x, R dm) {
+  return MASS ? x - dm : x;
+}
+__device__ __forceinline__ float neg_of(float a) { return -a; }
+__device__ __forceinline__ double neg_of(double a) { return dneg_if(a, true); }
+// the factor (e.re - dm, sign e.im), negated where neg
+template <bool MASS, typename R>
+__device__ __forceinline__ Cx<R> time_factor(Cx<R> e, R dm, bool conj, bool neg) {
+  const Cx<R> z = cneg_if(Cx<R>{less_dm<MASS>(e.re, dm), e.im}, neg);
+  return Cx<R>{z.re, conj ? neg_of(z.im) : z.im};
+}
+
 // M^dagger applied at the cell-time of nb, reading p (precision R); PH is any
 // functor returning e^{i phi_k}.
-template <typename R, typename PH = Phase<R>>
+template <typename R, typename PH = Phase<R>, bool MASS = true>
 __device__ __forceinline__ PairOut<R> mdag_pair(const Geo& g, const PH& ph, R dm,
                                                 const typename Vec2<R>::type* __restrict__ p,
                                                 const Nbr& nb) {
@@ -73,13 +122,11 @@ __device__ __forceinline__ PairOut<R> mdag_pair(const Geo& g, const PH& ph, R dm
   const R dk = geo_dk(g, R(0));
   Cx<R> pa = ld<R>(p, nb.q), pb = ld<R>(p, H + nb.q);
   // A row: time partner (x, t+1), phase of A at t+1, conjugated
-  Cx<R> ea = ph(nb.tp);
-  Cx<R> za = cneg_if(Cx<R>{ea.re - dm, -ea.im}, nb.wrap_tp);
+  Cx<R> za = time_factor<MASS>(ph(nb.tp), dm, true, nb.wrap_tp);
   Cx<R> ta = cfma(za, ld<R>(p, nb.tp), Cx<R>{-pa.re, -pa.im});
   Cx<R> oa = hopsum(ta, dk, pb, ld<R>(p, H + nb.im1), ld<R>(p, H + nb.jm1));
   // B row: time partner (x, t-1), phase of B at t-1; the hop carries a minus sign
-  Cx<R> eb = ph(H + nb.tm);
-  Cx<R> zb = cneg_if(Cx<R>{dm - eb.re, -eb.im}, nb.wrap_tm);
+  Cx<R> zb = time_factor<MASS>(ph(H + nb.tm), dm, false, !nb.wrap_tm);
   Cx<R> tb = cfma(zb, ld<R>(p, H + nb.tm), pb);
   Cx<R> ob = hopsum(tb, dk, pa, ld<R>(p, nb.ip1), ld<R>(p, nb.jp1));
   return PairOut<R>{oa, ob};
@@ -119,7 +166,7 @@ __device__ __forceinline__ PairOut<R> m_pair_ld(const Geo& g, const PH& ph, R dm
 }
 
 // M applied at the cell-time of nb, reading u (precision R).
-template <typename R, typename PH = Phase<R>>
+template <typename R, typename PH = Phase<R>, bool MASS = true>
 __device__ __forceinline__ PairOut<R> m_pair(const Geo& g, const PH& ph, R dm,
                                              const typename Vec2<R>::type* __restrict__ u,
                                              const Nbr& nb) {
@@ -127,13 +174,11 @@ __device__ __forceinline__ PairOut<R> m_pair(const Geo& g, const PH& ph, R dm,
   const R dk = geo_dk(g, R(0));
   Cx<R> ua = ld<R>(u, nb.q), ub = ld<R>(u, H + nb.q);
   // A row: (e^{i phi_A(t)} - dm) u_A(t-1)
-  Cx<R> ea = ph(nb.q);
-  Cx<R> za = cneg_if(Cx<R>{ea.re - dm, ea.im}, nb.wrap_tm);
+  Cx<R> za = time_factor<MASS>(ph(nb.q), dm, false, nb.wrap_tm);
   Cx<R> ta = cfma(za, ld<R>(u, nb.tm), Cx<R>{-ua.re, -ua.im});
   Cx<R> oa = hopsum(ta, dk, ub, ld<R>(u, H + nb.im1), ld<R>(u, H + nb.jm1));
   // B row: -(e^{-i phi_B(t)} - dm) u_B(t+1)
-  Cx<R> eb = ph(H + nb.q);
-  Cx<R> zb = cneg_if(Cx<R>{dm - eb.re, eb.im}, nb.wrap_tp);
+  Cx<R> zb = time_factor<MASS>(ph(H + nb.q), dm, true, !nb.wrap_tp);
   Cx<R> tb = cfma(zb, ld<R>(u, H + nb.tp), ub);
   Cx<R> ob = hopsum(tb, dk, ua, ld<R>(u, nb.ip1), ld<R>(u, nb.jp1));
   return PairOut<R>{oa, ob};
