@@ -187,27 +187,54 @@ __device__ __forceinline__ unsigned long long fma_x2(unsigned long long a, unsig
 // result therefore does not depend on block scheduling.
 constexpr int kMaxBlockThreads = 256;
 
+// Sums of K <= 32 values over a warp: lane l ends with the total of value
+// l >> (5 - log2 P), P the power of two >= K. Every step halves the values a
+// lane carries as well as the lanes a value is spread over, so that K values
+// cost about K additions a warp and not 5 K: the FP64 pipe of this GPU takes
+// 16 cycles for each.
+constexpr int pow2_at_least(int k) { return k <= 1 ? 1 : 2 * pow2_at_least((k + 1) / 2); }
+template <int K>
+__device__ __forceinline__ double warp_multi_sum(const double (&v)[K]) {
+  constexpr int P = pow2_at_least(K);
+  static_assert(P <= 32, "at most one value per lane");
+  const int lane = threadIdx.x & 31;
+  double w[P];
+#pragma unroll
+  for (int i = 0; i < P; ++i) w[i] = i < K ? v[i] : 0.0;
+  int o = 16;
+#pragma unroll
+  for (int half = P / 2; half > 0; half /= 2, o /= 2) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < half; ++i) {
+      const double send = up ? w[i] : w[i + half], keep = up ? w[i + half] : w[i];
+      w[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  double x = w[0];
+#pragma unroll
+  for (; o > 0; o /= 2) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+
+// The block's sums of K values, in a fixed order; in v in every thread of warp 0.
 template <int K>
 __device__ __forceinline__ void block_sum(double (&v)[K], double* smem /* K * 32 */) {
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-  }
+  constexpr int P = pow2_at_least(K), STEP = 32 / P;
+  const double x = warp_multi_sum(v);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  if (lane == 0) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) smem[k * 32 + warp] = v[k];
-  }
+  const int mine = lane / STEP;  // the lane's value
+  if (lane % STEP == 0 && mine < K) smem[mine * 32 + warp] = x;
   __syncthreads();
   if (warp == 0) {
+    // STEP lanes per value, each adding up every STEP-th warp's partial
+    double t = 0.0;
+    if (mine < K)
+      for (int k = lane % STEP; k < nw; k += STEP) t += smem[mine * 32 + k];
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-      double x = lane < nw ? smem[k * 32 + lane] : 0.0;
+    for (int o = STEP / 2; o > 0; o /= 2) t += __shfl_xor_sync(0xffffffffu, t, o);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-      v[k] = x;
-    }
+    for (int k = 0; k < K; ++k) v[k] = __shfl_sync(0xffffffffu, t, k * STEP);
   }
   __syncthreads();
 }
