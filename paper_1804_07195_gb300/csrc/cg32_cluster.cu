@@ -36,20 +36,21 @@ static const void* cluster_kernel32(const TilePlan& p) {
   if (p.cw == cw_ && p.S == s_)                                                    \
     return p.stride == kStrideSmall ? (const void*)k_cg32_cluster<cw_, s_, kStrideSmall> \
                                     : (const void*)k_cg32_cluster<cw_, s_, kStrideLarge>;
-  HMC_CASE(1, 1) HMC_CASE(1, 2) HMC_CASE(1, 4) HMC_CASE(1, 8)
-  HMC_CASE(2, 1) HMC_CASE(2, 2) HMC_CASE(2, 4)
+  HMC_CASE(1, 1) HMC_CASE(1, 2) HMC_CASE(1, 4) HMC_CASE(1, 8) HMC_CASE(1, 8 + kXInMemory)
+  HMC_CASE(2, 1) HMC_CASE(2, 2) HMC_CASE(2, 4) HMC_CASE(2, 4 + kXInMemory)
 #undef HMC_CASE
   return nullptr;
 }
 
-// us per iteration of a system on a cluster of cs blocks, from the size of its
-// largest tile (pairs of cells; one cell per column counts 0.75): fixed phase
-// latency, two exchanges, work. Fitted to measured iterations (6x6x16 2.7,
-// 12x12x32 2.9, 18x18x48 3.9, 24x24x48 4.5 us); it only ranks the choices.
+// us per iteration of a system on a cluster of cs blocks, from the columns of its
+// largest tile. Fitted to measured iterations; it only ranks the choices:
+//   12x12x32 on 1, 2, 4, 8, 16 blocks: 8.8, 4.4, 3.4, 2.9, 3.0
+//   24x24x48 on 8, 16: 6.4, 4.5;  18x18x48 on 4, 8, 16: 6.8, 4.3, 3.9
+//   36x36x48 on 16: 7.2 (over all SMs 5.8);  25x24x48 on 8, 16: 8.2, 6.8
 static double cluster_us(const TilePlan& p, const Geo& g, int cs) {
-  const double exch = cs == 1 ? 0.35 : cs == 2 ? 0.6 : cs == 4 ? 0.7 : cs == 8 ? 0.85 : 1.15;
-  const double cols = (double)p.J * std::min(p.T, g.nt) * (g.n / p.cw) * (p.cw == 2 ? 1.0 : 0.75);
-  return 0.8 + 2.0 * exch + 1.9e-3 * cols;
+  const double cols = (double)p.J * std::min(p.T, g.nt) * (g.n / p.cw);
+  const double slope = p.cw == 1 ? 1.5e-3 : tile_slices(p.S) <= 2 ? 1.6e-3 : 2.25e-3;
+  return (cs == 16 ? 2.85 : 2.45) + slope * cols + (p.S >= kXInMemory ? 1.2 : 0.0);
 }
 
 // Tiles of one system for a cluster of cs blocks (cs a power of two): the split
@@ -65,15 +66,16 @@ static bool plan_cluster(const hmc_ctx* c, const Geo& g, int cs, TilePlan* out) 
   double best = 0.0;
   for (int tj = 1; tj <= cs; tj *= 2) {
     const int J = (g.m + tj - 1) / tj, T0 = (g.nt + cs / tj - 1) / (cs / tj);
-    for (const int* S = tile_slices32(cw); *S; ++S) {
+    for (const int* inst = tile_slices32(cw); *inst; ++inst) {
+      const int S = tile_slices(*inst);
       TilePlan p;
       p.cw = cw;
-      p.S = *S;
+      p.S = *inst;
       p.J = J;
-      p.nseg = (T0 + *S - 1) / *S;
-      p.T = p.nseg * *S;
+      p.nseg = (T0 + S - 1) / S;
+      p.T = p.nseg * S;
       const long long th = ((long long)nq * J * p.nseg + 31) / 32 * 32;
-      if (th > max_threads32(cw, *S)) continue;
+      if (th > max_threads32(cw, *inst)) continue;
       const long long one = (long long)(p.T + 1) * (J + 1) * nq * (long long)VB;
       const long long cols = 2LL * (p.T + J) * nq;
       if (one > kStrideLarge) continue;

@@ -21,9 +21,8 @@ __global__ void __launch_bounds__(tile_max_threads<float, 2, S>(), 1) k_cg32_res
   cg_tile_solve<float, 2, S, false, tile_array_stride<false>()>(ts, gs, blockIdx.x, (char*)s_tile);
 }
 
-// Slices per column of the kernel instances (0 ends the list).
 const int* tile_slices32(int cw) {
-  static const int one[] = {1, 2, 4, 8, 0}, two[] = {1, 2, 4, 0};
+  static const int one[] = {1, 2, 4, 8, 8 + kXInMemory, 0}, two[] = {1, 2, 4, 4 + kXInMemory, 0};
   return cw == 2 ? two : one;
 }
 
@@ -33,11 +32,13 @@ int max_threads32(int cw, int S) {
       case 2: return tile_max_threads<float, 1, 2>();
       case 4: return tile_max_threads<float, 1, 4>();
       case 8: return tile_max_threads<float, 1, 8>();
+      case 8 + kXInMemory: return tile_max_threads<float, 1, 8 + kXInMemory>();
     }
   switch (S) {
     case 1: return tile_max_threads<float, 2, 1>();
     case 2: return tile_max_threads<float, 2, 2>();
     case 4: return tile_max_threads<float, 2, 4>();
+    case 4 + kXInMemory: return tile_max_threads<float, 2, 4 + kXInMemory>();
   }
   return 0;
 }
@@ -57,14 +58,14 @@ bool tile_plan_grid(const hmc_ctx* c, const Geo& g, int cw, int real, const int*
   bool found = false;
   double best = 0.0;
   for (const int* S = slices; *S; ++S)
-    for (int nseg = 1, fits = 1; fits && (nseg - 1) * *S < g.nt; ++nseg)
+    for (int nseg = 1, fits = 1; fits && (nseg - 1) * tile_slices(*S) < g.nt; ++nseg)
       for (int J = 1; J <= g.m; ++J) {
         TilePlan p;
         p.cw = cw;
         p.S = *S;
         p.nseg = nseg;
         p.J = J;
-        p.T = nseg * *S;
+        p.T = nseg * tile_slices(*S);
         p.tiles_j = (g.m + J - 1) / J;
         p.tiles_t = (g.nt + p.T - 1) / p.T;
         const size_t one = (size_t)(p.T + 1) * (J + 1) * g.n * 2 * real;
@@ -80,9 +81,9 @@ bool tile_plan_grid(const hmc_ctx* c, const Geo& g, int cw, int real, const int*
         p.smem = p.tab + table;
         // the work of the largest tile: its cells, the padding it exchanges (about
         // a third of a cell's work each), a little for every slice of a column
-        // (fewer, longer columns overlap less)
+        // (fewer, longer columns overlap less), and x streamed from L2
         const int Tmax = std::min(p.T, g.nt);
-        const double cost = (double)J * Tmax * nq + 0.7 * (J + Tmax) * nq + 8.0 * *S;
+        const double cost = (double)J * Tmax * nq + 0.7 * (J + Tmax) * nq + 8.0 * tile_slices(*S) + (*S >= kXInMemory ? 300.0 : 0.0);
         if (!found || cost < best) {
           found = true;
           best = cost;
@@ -117,11 +118,13 @@ static const void* grid_kernel32(int cw, int S) {
       case 2: return (const void*)k_cg32_resident<2>;
       case 4: return (const void*)k_cg32_resident<4>;
       case 8: return (const void*)k_cg32_resident<8>;
+      case 8 + kXInMemory: return (const void*)k_cg32_resident<8 + kXInMemory>;
     }
   switch (S) {
     case 1: return (const void*)k_cg32_resident2<1>;
     case 2: return (const void*)k_cg32_resident2<2>;
     case 4: return (const void*)k_cg32_resident2<4>;
+    case 4 + kXInMemory: return (const void*)k_cg32_resident2<4 + kXInMemory>;
   }
   return nullptr;
 }

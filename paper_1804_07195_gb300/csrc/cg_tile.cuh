@@ -45,7 +45,7 @@
 // brackets the design before it, which read r, x and phi from L2 row by row in
 // both halves and published p as well):
 //   6x6x16 6.4 (9.0)   12x12x32 6.8 (8.6)   36x36x64 5.9 (7.5)
-//   51x51x64 7.9 (11.6)   72x72x64 8.2 (11.8)   102x102x64 14.1 (16.2)
+//   51x51x64 7.9 (11.6)   72x72x64 8.2 (11.8)   90x90x64 11.1   102x102x64 14.1 (16.2)
 // The two exchanges take about 2 us each (arrival and poll of one L2 word 1.4,
 // the gather or the edges 0.5), whatever the lattice. The rest is, at
 // 102x102x64, shared memory (4.3 us of wavefronts), instruction issue (4.1) and
@@ -53,7 +53,9 @@
 // phases overlap only in part. Tried and not kept: every block polling every
 // block's packet (one trip less, but the polls of 18,000 packet reads delay
 // the writes: 8.5 to 10.7 us at 36x36x64); x held in registers at 102x102x64
-// (7 slices a column, 384 threads: 14.6 us, too few warps); 3 slices a column
+// (7 slices a column, 384 threads: 14.6 us, too few warps; but 90x90x64, where 480
+// threads with 4 slices hold x, takes 11.1 us against 12.8 with x in memory, and a
+// cluster of 8 blocks 6.4 against 8.3 at 24x24x48); 3 slices a column
 // (832 threads, spills: 14.0); instances for tiles without a ragged edge
 // (13.9); one warp adding up all threads' values (14.7).
 #pragma once
@@ -377,31 +379,28 @@ __device__ __forceinline__ int fresh(int i) {
   return i;
 }
 
-// Registers a thread holds for r of its column.
-template <typename R, int CW, int S>
-constexpr int tile_r_regs() {
-  return (int)sizeof(R) * CW * S;
-}
-template <typename R, int CW, int S>
-constexpr bool tile_x_in_registers() {
-  return tile_r_regs<R, CW, S>() <= 16;
-}
-// Largest block of an instance, from the registers it needs (r, x where it is
-// held, about 60 more for two cells or doubles, 45 for one) and those a thread
-// can have: the warps are dealt to four partitions of 16,384 registers, so 12,
-// 16, 20, 24 or 32 warps get 168, 128, 96, 80 or 64 registers a thread.
-template <typename R, int CW, int S>
+// A kernel instance is named by its slices per column S, plus kXInMemory where x
+// stays in memory and only passes through registers (the others hold r and x).
+constexpr int kXInMemory = 100;
+constexpr int tile_slices(int inst) { return inst % kXInMemory; }
+// Largest block of an instance, from the registers it needs (r and x: 8 per slice
+// for complex64 cells, 16 for pairs and for complex128; about 60 more, 45 for one
+// complex64 cell) and those a thread can have: the warps are dealt to four
+// partitions of 16,384 registers, so 12, 16, 20, 24 or 32 warps get 168, 128, 96,
+// 80 or 64 registers a thread.
+template <typename R, int CW, int INST>
 constexpr int tile_max_threads() {
-  const int r = tile_r_regs<R, CW, S>();
-  if (sizeof(R) == 8) return r <= 8 ? 640 : r <= 48 ? 512 : 384;
-  if (CW == 2) return r <= 8 ? 768 : 640;
-  return r <= 8 ? 1024 : 768;
+  constexpr bool mem = INST >= kXInMemory;
+  constexpr int held = (int)sizeof(R) * CW * tile_slices(INST) * (mem ? 1 : 2);
+  if (sizeof(R) == 8) return held <= 16 ? 640 : mem && held > 48 ? 384 : 512;
+  if (CW == 2) return held <= 16 ? 768 : held <= 32 ? 640 : 512;
+  return held <= 16 ? 1024 : held <= 32 ? 768 : 512;
 }
 
 // The solve of one system by the block `tile` of its group. sm: four padded
 // arrays AS bytes apart, the table of the padding (8 bytes a column) and, for CL,
 // the neighbours' r there.
-template <typename R, int CW, int S, bool CL, int AS>
+template <typename R, int CW, int INST, bool CL, int AS>
 __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync& gs, int tile, char* sm) {
   using LN = Lane<R, CW>;
   using L = typename LN::L;
@@ -410,7 +409,7 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
   using RT = Red<R>;
   using T = typename RT::T;
   using PH = PhLd<R, CW>;
-  constexpr int VB = (int)sizeof(V);
+  constexpr int VB = (int)sizeof(V), S = tile_slices(INST);
   constexpr int PA = 0, PB = AS, UA = 2 * AS, UB = 3 * AS;
   const int TAB = ts.tab, RP = ts.rp;
   __shared__ R s_a, s_ap;
@@ -419,7 +418,7 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
   // one warp: the FP64 pipe takes 16 cycles for a warp's addition, so that five
   // shuffle steps in every warp cost more than 1400 cycles of a block of 18
   constexpr bool BYTHREAD = !CL && sizeof(R) == 8;
-  __shared__ T s_red[CL ? 2 * kTileMaxCluster * kTileMaxWarps : BYTHREAD ? tile_max_threads<R, CW, S>() : kTileMaxWarps];
+  __shared__ T s_red[CL ? 2 * kTileMaxCluster * kTileMaxWarps : BYTHREAD ? tile_max_threads<R, CW, INST>() : kTileMaxWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = (blockDim.x + 31) >> 5;
   const int m = ts.g.m, nt = ts.g.nt;
   const int nq = ts.g.n / CW, Vq = ts.g.V / CW, Hq = ts.g.H / CW;  // all indices in columns of CW cells
@@ -555,7 +554,7 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
   // r and x of the thread's cells (A, B). With many slices per column x stays
   // in memory (in the lanes' layout while the solve runs) and passes through
   // registers in P, two slices in flight.
-  constexpr bool XREG = tile_x_in_registers<R, CW, S>();
+  constexpr bool XREG = INST < kXInMemory;
   C ra[S], rb[S];
   C xa[XREG ? S : 2], xb[XREG ? S : 2];
 #pragma unroll

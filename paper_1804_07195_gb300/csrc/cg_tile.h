@@ -10,14 +10,13 @@ namespace hmc {
 
 // Tiles for one cooperative launch over all SMs: every tile resident, within the
 // shared memory a block may use; false when there are none. real: bytes of a
-// real number; slices: slices per column of the kernel instances (0 ends the
-// list) with their largest blocks.
+// real number; slices: the kernel instances (0 ends the list) with their largest
+// blocks.
 bool tile_plan_grid(const hmc_ctx* c, const Geo& g, int cw, int real, const int* slices, int (*max_threads)(int, int),
                     TilePlan* out);
 hmc_status tile_grid_launch(hmc_ctx* c, int id, const void* kfn, const TilePlan& p, const TileSys& system);
 
-// Slices per column of the FP32 kernel instances (0 ends the list) and their
-// largest blocks.
+// The FP32 kernel instances (0 ends the list) and their largest blocks.
 const int* tile_slices32(int cw);
 int max_threads32(int cw, int S);
 

@@ -112,7 +112,7 @@ struct FusedShape {
 // them.
 struct TilePlan {
   int cw = 0;       // cells per column (0: not searched yet, -1: does not fit)
-  int S = 1;        // slices per column
+  int S = 1;        // kernel instance: slices per column, plus kXInMemory
   int J = 0, T = 0, tiles_j = 0, tiles_t = 0, nseg = 1;
   int threads = 0;  // whole warps
   int tab = 0, rp = 0;  // shared-memory offsets
