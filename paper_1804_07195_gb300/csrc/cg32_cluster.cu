@@ -9,6 +9,9 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <functional>
+#include <queue>
+#include <utility>
 
 #include "cg_tile.h"
 #include "launch.cuh"
@@ -179,8 +182,8 @@ hmc_status cg32_cluster_launch(hmc_ctx* c, const Geo& g, float2* x, float2* r, C
 // ---------------------------------------------------------------------------
 // Batches: every system on a cluster of its own. Before, all systems of a batch
 // went through an iteration together, two launches (or grid barriers) each, until
-// the last had converged; 48 systems of 16 lattices took 22.8 ms, now 13.4, and
-// a trajectory of 8 chains 345 ms, now 158.
+// the last had converged; 48 systems of 16 lattices took 22.8 ms, now 10.5, and
+// a trajectory of 8 chains 345 ms, now 123.
 
 bool cg32_cluster_batch(hmc_ctx* c, const std::vector<Geo>& geos, const std::vector<double>& iters,
                         std::vector<ClusterGroup>* groups) {
@@ -192,78 +195,111 @@ bool cg32_cluster_batch(hmc_ctx* c, const std::vector<Geo>& geos, const std::vec
   // must lie in one of its groups of SMs and leave some unused (152, 76, 36, 15
   // and 7 at a time on 152 SMs)
   const double sms[5] = {1.0, 2.0, 4.2, 10.1, 21.7};
-  double total = 0.0;  // SM us
   for (int i = 0; i < ns; ++i) {
     const std::array<int, 3> key{geos[i].n, geos[i].m, geos[i].nt};
     auto it = c->batch_plans.find(key);
     if (it == c->batch_plans.end()) it = c->batch_plans.emplace(key, cluster_plans(c, geos[i])).first;
     cp[i] = &it->second;
-    // the smallest cluster that holds it: the least SM time
-    for (pick[i] = 0; pick[i] < 5 && cp[i]->p[pick[i]].cw <= 0; ++pick[i]) {
+  }
+  // For a time T every system takes the smallest cluster (the least SM time)
+  // that is expected to finish within T, or its fastest; the batch's end is that
+  // of running them longest first on the SMs that are free. Of up to 32 values
+  // of T, spread over the systems' possible times, the best end wins.
+  std::vector<double> cand;
+  auto time_at = [&](int i, int k) { return iters[i] * cp[i]->us[k]; };
+  for (int i = 0; i < ns; ++i) {
+    int any = 0;
+    for (int k = 0; k < 5; ++k)
+      if (cp[i]->p[k].cw > 0) {
+        cand.push_back(time_at(i, k));
+        any = 1;
+      }
+    if (!any) return false;
+  }
+  std::sort(cand.begin(), cand.end());
+  std::vector<int> trial(ns), order(ns);
+  double best = 0.0;
+  const int ncand = (int)cand.size(), tries = std::min(ncand, 32);
+  for (int v = 0; v < tries; ++v) {
+    const double T = cand[tries == ncand ? v : (size_t)v * (ncand - 1) / (tries - 1)];
+    for (int i = 0; i < ns; ++i) {
+      int k = -1;
+      for (int l = 0; l < 5; ++l)
+        if (cp[i]->p[l].cw > 0 && (k < 0 || time_at(i, k) > T) && (k < 0 || time_at(i, l) < time_at(i, k))) k = l;
+      trial[i] = k;
+      order[i] = i;
     }
-    if (pick[i] == 5) return false;
-    total += sms[pick[i]] * iters[i] * cp[i]->us[pick[i]];
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return time_at(a, trial[a]) > time_at(b, trial[b]); });
+    std::priority_queue<std::pair<double, double>, std::vector<std::pair<double, double>>, std::greater<>> running;
+    double free = c->nsm, now = 0.0, end = 0.0;
+    for (int i : order) {
+      const double need = sms[trial[i]];
+      while (free < need && !running.empty()) {
+        now = running.top().first;
+        free += running.top().second;
+        running.pop();
+      }
+      const double done = now + time_at(i, trial[i]);
+      running.push({done, need});
+      free -= need;
+      end = std::max(end, done);
+    }
+    // of values that end together the largest T: the least SM time
+    if (v == 0 || end <= 1.01 * best) {
+      best = v == 0 ? end : std::min(best, end);
+      pick = trial;
+    }
   }
-  // then larger clusters for the system that finishes last, while that shortens
-  // the batch: until the SM time, spread over all SMs, becomes the longer
-  auto time_of = [&](int i) { return iters[i] * cp[i]->us[pick[i]]; };
-  for (int step = 0; step < 4 * ns; ++step) {
-    int w = 0;
-    for (int i = 1; i < ns; ++i)
-      if (time_of(i) > time_of(w)) w = i;
-    int k = pick[w] + 1;
-    while (k < 5 && cp[w]->p[k].cw <= 0) ++k;
-    if (k >= 5 || cp[w]->us[k] >= cp[w]->us[pick[w]]) break;
-    const double more = iters[w] * (sms[k] * cp[w]->us[k] - sms[pick[w]] * cp[w]->us[pick[w]]);
-    if ((total + more) / c->nsm > time_of(w)) break;
-    total += more;
-    pick[w] = k;
-  }
-  // one launch per instance, cluster size and block size (in steps of 128
-  // threads); the systems that run longest first
-  std::vector<int> order(ns);
+  auto time_of = [&](int i) { return time_at(i, pick[i]); };
+  // one launch per instance and cluster size, with the largest block and shared
+  // memory of its systems; the systems that run longest first
   for (int i = 0; i < ns; ++i) order[i] = i;
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return time_of(a) > time_of(b); });
   groups->clear();
+  double load[hmc_ctx::kSideStreams] = {};
   for (int i : order) {
     const TilePlan& p = cp[i]->p[pick[i]];
-    const int th = std::min((p.threads + 127) / 128 * 128, max_threads32(p.cw, p.S));
     ClusterGroup* g = nullptr;
     for (ClusterGroup& h : *groups)
-      if (h.log2 == pick[i] && h.threads == th && h.plan.cw == p.cw && h.plan.S == p.S && h.plan.stride == p.stride) g = &h;
+      if (h.log2 == pick[i] && h.plan.cw == p.cw && h.plan.S == p.S && h.plan.stride == p.stride) g = &h;
     if (!g) {
       groups->push_back(ClusterGroup{});
       g = &groups->back();
       g->log2 = pick[i];
-      g->threads = th;
       g->plan = p;
+      // the launches of one stream run one after another: the one that has the
+      // least to do so far
+      int s = 0;
+      for (int k = 1; k < hmc_ctx::kSideStreams; ++k)
+        if (load[k] < load[s]) s = k;
+      g->stream = s;
+      load[s] += time_of(i);
     }
     g->plan.smem = std::max(g->plan.smem, p.smem);
+    g->plan.threads = std::max(g->plan.threads, p.threads);
     g->sys.push_back(i);
     g->plans.push_back(p);
   }
-  // a group's launch has the largest block and shared memory of its systems
-  for (ClusterGroup& g : *groups) {
-    g.plan.threads = g.threads;
+  for (const ClusterGroup& g : *groups)
     if (!cluster_runs(c, g.plan, 1 << g.log2)) return false;
-  }
   return true;
 }
 
 hmc_status cg32_cluster_batch_launch(hmc_ctx* c, const std::vector<ClusterGroup>& groups, const TileSys* list) {
   if (!c->side_start) HMC_CUDA(c, cudaEventCreateWithFlags(&c->side_start, cudaEventDisableTiming));
-  const int nstr = std::min((int)groups.size(), hmc_ctx::kSideStreams);
+  bool on[hmc_ctx::kSideStreams] = {};
   HMC_CUDA(c, cudaEventRecord(c->side_start, c->stream));
   int first = 0;
   hmc_status st = HMC_OK;
   for (size_t k = 0; k < groups.size() && st == HMC_OK; ++k) {
     const ClusterGroup& g = groups[k];
-    const int i = (int)(k % hmc_ctx::kSideStreams);
+    const int i = g.stream;
     if (!c->side[i]) {
       HMC_CUDA(c, cudaStreamCreateWithFlags(&c->side[i], cudaStreamNonBlocking));
       HMC_CUDA(c, cudaEventCreateWithFlags(&c->side_done[i], cudaEventDisableTiming));
     }
-    if (k < (size_t)nstr) HMC_CUDA(c, cudaStreamWaitEvent(c->side[i], c->side_start, 0));
+    if (!on[i]) HMC_CUDA(c, cudaStreamWaitEvent(c->side[i], c->side_start, 0));
+    on[i] = true;
     const TileSys* mine = list + first;
     const TileSys one{};
     void* args[] = {(void*)&mine, (void*)&one};
@@ -275,7 +311,8 @@ hmc_status cg32_cluster_batch_launch(hmc_ctx* c, const std::vector<ClusterGroup>
     c->prof.launches[K_BATCH_CG32]++;
     first += (int)g.sys.size();
   }
-  for (int i = 0; i < nstr; ++i) {  // also after a failure: nothing outlives the call
+  for (int i = 0; i < hmc_ctx::kSideStreams; ++i) {  // also after a failure: nothing outlives the call
+    if (!on[i]) continue;
     HMC_CUDA(c, cudaEventRecord(c->side_done[i], c->side[i]));
     HMC_CUDA(c, cudaStreamWaitEvent(c->stream, c->side_done[i], 0));
   }

@@ -35,11 +35,11 @@ inline bool tile_allow_smem(const hmc_ctx* c, const void* k) {
 
 TileSys make_tile_sys(const Geo& g, const TilePlan& p, const void* ph, void* x, void* r, void* U, CGScal* sc);
 
-// One launch of a batch: systems whose plans share a kernel instance, a cluster
-// size (2^log2 blocks) and a block size. plan: the instance, with the block
-// and the shared memory of the launch.
+// One launch of a batch: systems whose plans share a kernel instance and a
+// cluster size (2^log2 blocks). plan: the instance, with the block and the
+// shared memory of the launch; stream: the context's side stream it runs on.
 struct ClusterGroup {
-  int log2 = 0, threads = 0;
+  int log2 = 0, stream = 0;
   TilePlan plan;
   std::vector<int> sys;        // indices into the batch, longest first
   std::vector<TilePlan> plans;  // theirs
