@@ -8,6 +8,7 @@
 #include <cstring>
 #include <string>
 
+#include "phase.cuh"
 #include "solvers.h"
 #include "trace.h"
 #include "validate.h"
@@ -366,6 +367,13 @@ hmc_status hmc_create(hmc_ctx** out, const hmc_lattice* lat, void* stream) {
   c->ws_bytes[WS_E] = N * sizeof(double2);
   if (guarded_alloc(c, N * sizeof(float), &c->ws[WS_PHI32]) != HMC_OK) return bail(cudaErrorMemoryAllocation);
   c->ws_bytes[WS_PHI32] = N * sizeof(float);
+  {
+    std::vector<double2> tab(2 * kPhaseTable);
+    phase_table_host(tab.data());
+    if ((e = cudaMalloc(&c->phase_tab, sizeof(double2) * tab.size())) != cudaSuccess) return bail(e);
+    if ((e = cudaMemcpy(c->phase_tab, tab.data(), sizeof(double2) * tab.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
+      return bail(e);
+  }
   const size_t npart = (size_t)kMaxRed * std::max(c->max_grid, c->nsm * kOneItemBlocksPerSM);
   if ((e = cudaMalloc(&c->partials, sizeof(double) * npart)) != cudaSuccess) return bail(e);
   if ((e = cudaMalloc(&c->partA, sizeof(double) * c->nsm * 2 * kOneItemBlocksPerSM)) != cudaSuccess) return bail(e);
@@ -399,6 +407,7 @@ hmc_status hmc_destroy(hmc_ctx* c) {
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   for (int i = 0; i < WS_COUNT; ++i)
     if (c->ws[i]) guarded_free(c->ws[i]);
+  if (c->phase_tab) cudaFree(c->phase_tab);
   if (c->partials) cudaFree(c->partials);
   if (c->partA) cudaFree(c->partA);
   if (c->partB) cudaFree(c->partB);

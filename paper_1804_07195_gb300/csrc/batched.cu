@@ -24,6 +24,7 @@
 
 #include "cg_tile.h"
 #include "operator.cuh"
+#include "phase.cuh"
 #include "solvers.h"
 #include "trace.h"
 #include "validate.h"
@@ -181,14 +182,13 @@ struct BScal {
   const int lb = (vb) - S_.block0;                   \
   const int stride = S_.nblocks * blockDim.x
 
-__global__ void kb_phase(const BSys* __restrict__ sys, const int* __restrict__ bsys,
+__global__ void kb_phase(const BSys* __restrict__ sys, const int* __restrict__ bsys, PhaseTable tab,
                          double2* __restrict__ E, float* __restrict__ phi32) {
   BLOCK_SYS();
   for (int k = lb * blockDim.x + threadIdx.x; k < g.N; k += stride) {
-    double x = S_.phi[k], s, c;
-    sincos(x, &s, &c);
-    E[S_.off + k] = make_double2(c, s);
-    phi32[S_.off + k] = phi_to_f32(x);
+    const double x = S_.phi[k];
+    E[S_.off + k] = phase_of_field(tab, x);
+    phi32[S_.off + k] = field_to_f32(x);
   }
 }
 
@@ -994,7 +994,7 @@ extern "C" hmc_status hmc_solve_batched(hmc_ctx* c, int nsys, const hmc_system* 
                                   cudaMemcpyDeviceToDevice, s));
     plan_blocks(w, 256, 2);
     HMC_TRY(upload_plan<double>(c, w, s));
-    kb_phase<<<w.blocks, w.threads, 0, s>>>(w.sys, w.bsys, w.E, w.phi32);
+    kb_phase<<<w.blocks, w.threads, 0, s>>>(w.sys, w.bsys, PhaseTable{c->phase_tab}, w.E, w.phi32);
     HMC_CUDA(c, cudaGetLastError());
     c->prof.launches[K_BATCH_MISC]++;
 

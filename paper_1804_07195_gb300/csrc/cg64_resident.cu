@@ -1,6 +1,6 @@
 // Resident-tile CG over all SMs in FP64, one cooperative launch per solve
 // (cg_tile.cuh): the plain FP64 CG of Section 3 on lattices whose tiles fit the
-// chip (up to about 400,000 sites).
+// chip (up to about 500,000 sites).
 #include "cg_tile.h"
 #include "launch.cuh"
 
@@ -12,13 +12,12 @@ __global__ void __launch_bounds__(tile_max_threads<double, 1, S>(), 1) k_cg64_re
   cg_tile_solve<double, 1, S, false, tile_array_stride<false>()>(ts, gs, blockIdx.x, (char*)s_tile);
 }
 
-static const int kSlices64[] = {1, 2, 4 + kXInMemory, 8 + kXInMemory, 0};
+static const int kSlices64[] = {1, 2, 4 + kXInMemory, 0};
 static int max_threads64(int, int S) {
   switch (S) {
     case 1: return tile_max_threads<double, 1, 1>();
     case 2: return tile_max_threads<double, 1, 2>();
     case 4 + kXInMemory: return tile_max_threads<double, 1, 4 + kXInMemory>();
-    case 8 + kXInMemory: return tile_max_threads<double, 1, 8 + kXInMemory>();
   }
   return 0;
 }
@@ -27,7 +26,6 @@ static const void* kernel64(int S) {
     case 1: return (const void*)k_cg64_resident<1>;
     case 2: return (const void*)k_cg64_resident<2>;
     case 4 + kXInMemory: return (const void*)k_cg64_resident<4 + kXInMemory>;
-    case 8 + kXInMemory: return (const void*)k_cg64_resident<8 + kXInMemory>;
   }
   return nullptr;
 }

@@ -153,6 +153,7 @@ struct hmc_ctx {
   void* ws[hmc::WS_COUNT] = {};
   size_t ws_bytes[hmc::WS_COUNT] = {};
 
+  double2* phase_tab = nullptr;    // table of phase.cuh
   double* partials = nullptr;      // reduction partials, kPartials doubles
   double* partA = nullptr;         // per-block partials of the FP32 CG M^dagger kernel
   double* partB = nullptr;         // per-block partials of the FP32 CG M kernel
@@ -169,7 +170,6 @@ struct hmc_ctx {
   bool tile_sync_stale = false;
   hmc::TilePlan tile_plan32[2];
   hmc::TilePlan tile_plan64;
-  bool resident64 = false;  // the tuner found the resident-tile FP64 CG fastest
   // the same on one thread block cluster (log2 of its blocks; -2: not looked for yet, -1: none)
   int cluster_log2 = -2;
   double cluster_us = 0.0;  // estimate per iteration

@@ -4,11 +4,15 @@
 // Passages: the operator of Eq. ferm_op (Section 2), CG (Section 3), the vector
 // steps of Algorithm A.1 (Appendix A), the force of Eqs. p_dot, f_chi_i and
 // def_xi_i, the energies of Eq. hamiltonian.
+#include <cmath>
+#include <cstring>
+#include <mutex>
 #include <type_traits>
 
 #include "kernels.h"
 #include "launch.cuh"
 #include "operator.cuh"
+#include "phase.cuh"
 
 namespace hmc {
 
@@ -56,17 +60,36 @@ const double kKernelBytesPerSite[K_COUNT] = {
     0};                  // resident CG f64: 208 B (the pair of kernels and the p update)
 
 // ---------------------------------------------------------------------------
-// e^{i phi} for the FP64 stencils of Eq. ferm_op, and phi rounded to float.
-__global__ void __launch_bounds__(kThreads) k_phase(int N, const double* __restrict__ phi,
+// e^{i phi} for the FP64 stencils of Eq. ferm_op, and phi rounded to float. Bound
+// by the FP64 pipe: 102x102x64 45 us (74 with sincos), 51x51x64 14.4 (22.5).
+__global__ void __launch_bounds__(kThreads) k_phase(int N, const double* __restrict__ phi, PhaseTable tab,
                                                     double2* __restrict__ E,
                                                     float* __restrict__ phi32) {
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
-    double s, co;
-    double x = phi[k];
-    sincos(x, &s, &co);
-    E[k] = make_double2(co, s);
-    phi32[k] = phi_to_f32(x);
+    const double x = phi[k];
+    E[k] = phase_of_field(tab, x);
+    phi32[k] = field_to_f32(x);
   }
+}
+
+void phase_table_host(double2* out) {
+  // filled once a process; e^{i 2 pi k / K} to more than 60 bits
+  static double2 table[2 * kPhaseTable];
+  static std::once_flag once;
+  std::call_once(once, [] {
+    const long double two_pi = 6.283185307179586476925286766559005768L;
+    for (int k = 0; k < kPhaseTable; ++k) {
+      // by the angle of the first octant: quarter turns are exact
+      const int quarter = k / (kPhaseTable / 4), j = k % (kPhaseTable / 4);
+      const long double a = two_pi * j / kPhaseTable;
+      const long double c = std::cos(a), s = std::sin(a);
+      const long double v[2] = {quarter == 0 ? c : quarter == 1 ? -s : quarter == 2 ? -c : s,
+                                quarter == 0 ? s : quarter == 1 ? c : quarter == 2 ? -s : -c};
+      table[k] = make_double2((double)v[0], (double)v[1]);
+      table[kPhaseTable + k] = make_double2((double)(v[0] - (double)v[0]), (double)(v[1] - (double)v[1]));
+    }
+  });
+  std::memcpy(out, table, sizeof(table));
 }
 
 
@@ -951,7 +974,7 @@ __global__ void __launch_bounds__(kThreads) k_half_sq(int N, const double* __res
 hmc_status k_phase_launch(hmc_ctx* c, const double* phi) {
   const int N = c->geo.N;
   return launch(c, K_PHASE, [&] {
-    k_phase<<<GRID(N)>>>(N, phi, (double2*)c->ws[WS_E], (float*)c->ws[WS_PHI32]);
+    k_phase<<<GRID(N)>>>(N, phi, PhaseTable{c->phase_tab}, (double2*)c->ws[WS_E], (float*)c->ws[WS_PHI32]);
   });
 }
 

@@ -161,30 +161,6 @@ static hmc_status tune_cg(hmc_ctx* c, double ms, double sigma, const V2<R>* b) {
     }
   }
   for (int k = 0; k < nk; ++k) c->shape[ids[k]] = keep[k];
-  // FP64: the three kernels (graph replay) against the resident-tile kernel,
-  // 48 iterations each, twice, best kept
-  if constexpr (sizeof(R) == 8) {
-    c->resident64 = false;
-    if (!c->capturing && c->bar_extra == 0 && cg64_resident_ok(c, g)) {
-      float best_t[2] = {1e30f, 1e30f};
-      for (int d = 0; d < 2; ++d) {
-        c->resident64 = d == 1;
-        for (int rep = 0; rep < 2; ++rep) {
-          SolveStats tmp;
-          HMC_CUDA(c, cudaEventRecord(e0, c->stream));
-          const hmc_status st = cg_core<R>(c, ms, sigma, b, x, true, 1e-30, 48, 2, false, &tmp);
-          HMC_CUDA(c, cudaEventRecord(e1, c->stream));
-          HMC_CUDA(c, cudaEventSynchronize(e1));
-          c->err.clear();
-          float t = 1e30f;
-          if (st == HMC_OK || st == HMC_ERR_NOT_CONVERGED) cudaEventElapsedTime(&t, e0, e1);
-          best_t[d] = std::min(best_t[d], t);
-        }
-      }
-      c->resident64 = best_t[1] < best_t[0];
-      destroy_graphs(c);
-    }
-  }
   // FP32: the single-reduction kernel's tile (variants 0 and 6), then the
   // designs against each other through the solver path they would run in
   // (graph replay with programmatic dependent launch; 48 iterations, twice
@@ -279,7 +255,13 @@ template <typename R>
 hmc_status cg_core(hmc_ctx* c, double ms, double sigma, const V2<R>* b, V2<R>* x, bool x_zero,
                    double tol, int maxit, int sc_slot, bool want_true_res, SolveStats* st) {
   const Geo& g = c->geo;
-  if (!c->capturing) HMC_TRY(tune_cg<R>(c, ms, sigma, b));
+  // FP64 solves take the resident tiles wherever they fit (the wait test and a
+  // capture excepted), without timing: they were the faster at every size
+  // (us per iteration against the three kernels: 3x3x8 11.2 / 15.2, 24x24x48 11.4 /
+  // 19.2, 36x36x64 18.6 / 27.4, 51x51x64 32.6 / 34.3, 64x64x64 40.3 / 41.5; with
+  // eight slices a column, 66x66x64, they lost, 50.1 / 41.8, and have no instance)
+  const bool tiles64 = sizeof(R) == 8 && !c->capturing && c->bar_extra == 0 && cg64_resident_ok(c, c->geo);
+  if (!c->capturing && !tiles64) HMC_TRY(tune_cg<R>(c, ms, sigma, b));
   const R dm = (R)(c->delta * ms);
   V2<R> *r, *p, *u;
   HMC_TRY(vec_slots<R>(c, &r, &p, &u));
@@ -357,9 +339,8 @@ hmc_status cg_core(hmc_ctx* c, double ms, double sigma, const V2<R>* b, V2<R>* x
       c->prof.bytes[whole ? K_CG_RES32 : K_CG_PERSIST32] += 96.0 * g.N * sch->iter;
     }
   }
-  // FP64: the resident-tile kernel when the tuner chose it
   if constexpr (sizeof(R) == 8) {
-    if (!c->capturing && c->resident64 && c->bar_extra == 0 && cg64_resident_ok(c, g)) {
+    if (tiles64) {
       persistent = true;
       HMC_TRY(cg64_resident_launch(c, g, (double2*)x, (double2*)r, (double2*)u, sc));
       HMC_CUDA(c, cudaMemcpyAsync(sch, sc, sizeof(CGScal), cudaMemcpyDeviceToHost, c->stream));
