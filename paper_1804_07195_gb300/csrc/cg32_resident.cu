@@ -183,7 +183,7 @@ bool cg32_prefer_cluster(hmc_ctx* c, const Geo& g) {
   if (!p) p = plan32(c, g, 1);
   if (!p) return true;
   // us per iteration over all SMs: two exchanges through L2, phase latency, work
-  // (measured: 5.9 at 36x36x64, 8.2 at 72x72x64); cluster_us has the cluster's.
+  // (measured: 5.6 at 36x36x64, 7.95 at 72x72x64); cluster_us has the cluster's.
   // The line between them runs near 100,000 sites (measured: 24x24x48 4.5 us on a
   // cluster, 6.2 over all SMs)
   const double cols = (double)p->J * std::min(p->T, g.nt) * (g.n / p->cw) * (p->cw == 2 ? 1.0 : 0.75);

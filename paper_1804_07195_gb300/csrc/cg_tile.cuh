@@ -44,8 +44,8 @@
 // What bounds an FP32 iteration of a cooperative launch (us, 2070 MHz; in
 // brackets the design before it, which read r, x and phi from L2 row by row in
 // both halves and published p as well):
-//   6x6x16 6.4 (9.0)   12x12x32 6.8 (8.6)   36x36x64 5.9 (7.5)
-//   51x51x64 7.9 (11.6)   72x72x64 8.2 (11.8)   90x90x64 11.1   102x102x64 14.1 (16.2)
+//   6x6x16 6.4 (9.0)   12x12x32 6.8 (8.6)   36x36x64 5.6 (7.5)
+//   51x51x64 7.55 (11.6)   72x72x64 7.95 (11.8)   90x90x64 11.0   102x102x64 14.0 (16.2)
 // The two exchanges take about 2 us each (arrival and poll of one L2 word 1.4,
 // the gather or the edges 0.5), whatever the lattice. The rest is, at
 // 102x102x64, shared memory (4.3 us of wavefronts), instruction issue (4.1) and
@@ -289,8 +289,10 @@ __device__ __forceinline__ typename Red<R>::T warp_sum(typename Red<R>::T v) {
 
 // ---------------------------------------------------------------------------
 // Arrival word (CL = false).
-__device__ __forceinline__ void red_add_release(unsigned* p, unsigned x) {
-  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(x) : "memory");
+// Relaxed: the __threadfence before it orders the block's writes already, and the
+// release form fences once more (51x51x64: 7.8 us an iteration, relaxed 7.55).
+__device__ __forceinline__ void red_add_relaxed(unsigned* p, unsigned x) {
+  asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(x) : "memory");
 }
 
 // Warp 0: the sum of all blocks' partials, in every lane.
@@ -661,7 +663,7 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
         if (lane == 0) {
           part[tile] = v;
           __threadfence();  // the block's edges, ordered before this thread by the barrier above
-          red_add_release(gs.word, tile == 0 ? 0x80000000u - (gs.need - 1u) : 1u);
+          red_add_relaxed(gs.word, tile == 0 ? 0x80000000u - (gs.need - 1u) : 1u);
           const unsigned want = (ep & 1u) << 31;
           const long long tw = clock64();
           unsigned spins = 0;
