@@ -614,6 +614,7 @@ hmc_status fgmres_core(hmc_ctx* c, double ms, double sigma, const double2* b, do
   const int ldh = restart + 1;
   std::vector<cd> H((size_t)ldh * restart), gvec(restart + 1), rs(restart);
   std::vector<double> rc(restart);
+  std::vector<const double2*> zvec(restart);
   while (err > tol * bnorm && arnoldi < maxit) {
     const double rnorm = err;
     std::fill(H.begin(), H.end(), cd(0));
@@ -626,14 +627,16 @@ hmc_status fgmres_core(hmc_ctx* c, double ms, double sigma, const double2* b, do
       if (err < tol * bnorm) break;
       double2* Vj = Vb + (size_t)j * N;
       double2* Zj = Zb + (size_t)j * N;
-      // v_j = w / |w|
-      HMC_TRY(scale_launch(c, N, 1.0 / wnorm, wsrc, Vj, v32));
-      // z_j: spCG with tolerance TOL a |b| / ERR, or z_j = v_j
+      // z_j: spCG with tolerance TOL a |b| / ERR, or z_j = v_j itself (no copy, and
+      // no float copy of v_j, which only the spCG reads)
       const double t = tol * a * bnorm / err;
-      HMC_TRY(precondition_solve(c, ms, sigma, Vj, v32, Zj, t < 1.0 ? std::max(t, inner_floor) : 1.0,
-                           inner_prec, inner_maxit, st));
+      // v_j = w / |w|
+      HMC_TRY(scale_launch(c, N, 1.0 / wnorm, wsrc, Vj, t < 1.0 ? v32 : nullptr));
+      if (t < 1.0)
+        HMC_TRY(precondition_solve(c, ms, sigma, Vj, v32, Zj, std::max(t, inner_floor), inner_prec, inner_maxit, st));
+      zvec[j] = t < 1.0 ? Zj : Vj;
       // w = A z_j, h_ij = v_i^H w (i <= j), w -= sum h_ij v_i, h_{j+1,j} = |w|
-      HMC_TRY(apply_A64(c, ms, sigma, Zj, w));
+      HMC_TRY(apply_A64(c, ms, sigma, zvec[j], w));
       st->applies64++;
       VecList V;
       for (int i = 0; i <= j; ++i) V.v[i] = Vb + (size_t)i * N;
@@ -684,7 +687,7 @@ hmc_status fgmres_core(hmc_ctx* c, double ms, double sigma, const double2* b, do
     VecList Z;
     CoefList coef;
     for (int i = 0; i < k; ++i) {
-      Z.v[i] = Zb + (size_t)i * N;
+      Z.v[i] = zvec[i];
       coef.re[i] = y[i].real();
       coef.im[i] = y[i].imag();
     }
