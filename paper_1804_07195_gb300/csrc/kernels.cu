@@ -805,29 +805,56 @@ __global__ void __launch_bounds__(kThreads) k_redot(int N, const double2* __rest
 }
 
 // Arnoldi step of Algorithm A.1 (classical Gram-Schmidt in two passes):
-// h[i] = V_i^H w for the NV basis vectors (NV a compile-time constant, so the
-// basis pointers stay in the parameter bank and every loop unrolls).
-template <int NV>
-__global__ void __launch_bounds__(kThreads) k_mdot(int N, VecList V, const double2* __restrict__ w,
-                                                   double* hout, double* partials, unsigned* ticket) {
-  double acc[2 * NV];
+// h[i] = V_i^H w. Bound by the FP64 pipe, 4 operations per site and vector at 16
+// cycles a warp (8.5 us per vector at 102x102x64), and on small lattices by the sum
+// over the threads, which takes the same pipe. So a block takes one vector and one
+// of the lattice's chunks: it has 2 sums instead of 2 nv, w is read once per vector
+// (from L2), and the last block's warps each add up whole values. Times in us for
+// nv vectors, in brackets all vectors per thread with 8 blocks a SM:
+//   12x12x32 nv 5, 10: 8.3, 10.3 (11.4, 18.0)   36x36x64: 14.4, 21.5 (28.8, 51.3)
+//   102x102x64 nv 1, 5, 10: 17.5, 56, 102 (22.5, 76, 151)
+// Two or four vectors a block are no faster (102x102x64 nv 10: 102, 119).
+__global__ void __launch_bounds__(kThreads) k_mdot(int N, VecList V, int nv, int chunks,
+                                                   const double2* __restrict__ w, double* hout,
+                                                   double* partials, unsigned* ticket) {
+  const int i = (int)blockIdx.x / chunks, ch = (int)blockIdx.x - i * chunks;
+  const double2* __restrict__ v = V.v[i];
+  double acc[2] = {0.0, 0.0};
+#pragma unroll 2
+  for (int k = ch * kThreads + threadIdx.x; k < N; k += chunks * kThreads) {
+    const double2 wk = w[k], vk = v[k];
+    // conj(v) w
+    acc[0] = fma(vk.x, wk.x, fma(vk.y, wk.y, acc[0]));
+    acc[1] = fma(vk.x, wk.y, fma(-vk.y, wk.x, acc[1]));
+  }
+  __shared__ double smem[2 * 32];
+  __shared__ bool am_last;
+  block_sum<2>(acc, smem);
+  if (threadIdx.x == 0) {
+    partials[2 * i * chunks + ch] = acc[0];
+    partials[(2 * i + 1) * chunks + ch] = acc[1];
+    __threadfence();
+    am_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!am_last) return;
+  __threadfence();
+  // the last block: a warp per value, four loads in flight a lane
+  const int lane = threadIdx.x & 31;
+  for (int h = threadIdx.x >> 5; h < 2 * nv; h += kThreads / 32) {
+    double t = 0.0;
+    for (int q = lane; q < chunks; q += 128) {
+      double p[4];
 #pragma unroll
-  for (int i = 0; i < 2 * NV; ++i) acc[i] = 0.0;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
-    double2 wk = w[k];
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      double2 vk = V.v[i][k];
-      // conj(v) w
-      acc[2 * i] = fma(vk.x, wk.x, fma(vk.y, wk.y, acc[2 * i]));
-      acc[2 * i + 1] = fma(vk.x, wk.y, fma(-vk.y, wk.x, acc[2 * i + 1]));
+      for (int e = 0; e < 4; ++e)
+        p[e] = q + 32 * e < chunks ? __ldcg(&partials[h * chunks + q + 32 * e]) : 0.0;
+      t += (p[0] + p[1]) + (p[2] + p[3]);
     }
-  }
-  double tot[2 * NV];
-  if (grid_sum<2 * NV>(acc, partials, ticket, tot) && threadIdx.x == 0) {
 #pragma unroll
-    for (int i = 0; i < 2 * NV; ++i) hout[i] = tot[i];
+    for (int o = 16; o > 0; o /= 2) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) hout[h] = t;
   }
+  if (threadIdx.x == 0) *ticket = 0u;
 }
 
 // w -= sum_i h[i] V_i over the NV basis vectors, then |w|^2.
@@ -1159,22 +1186,27 @@ hmc_status redot_launch(hmc_ctx* c, int N, const double2* u, const double2* v, d
 hmc_status mdot_launch(hmc_ctx* c, int N, VecList V, int nv, const double2* w, double* hout,
                        unsigned* ticket) {
   if (nv < 1 || nv > kMaxRestart) return fail(c, HMC_ERR_INVALID, "basis size out of range");
+  // Blocks per SM: one as long as an SM has few sites to work through, as every
+  // block more is a sum more (us, one and two: 36x36x64 nv 1, 3 8.3, 10.4 and 10.3,
+  // 12.4; 51x51x64 nv 5 20.6 and 20.6, nv 10 33.1 and 32.9, nv 16 63 and 49)
+  const int per_sm = (double)N * nv <= 64.0 * kThreads * c->nsm ? 1 : 2;
+  const int chunks = std::max(1, std::min((N + kThreads - 1) / kThreads, per_sm * c->nsm / nv));
   return launch_b(c, K_MDOT, 16.0 * N * (nv + 1), [&] {
-    switch (nv) {
-#define X(n) \
-  case n: k_mdot<n><<<GRID(N)>>>(N, V, w, hout, c->partials, ticket); break;
-      NV_CASES(X)
-#undef X
-    }
+    k_mdot<<<nv * chunks, kThreads, 0, c->stream>>>(N, V, nv, chunks, w, hout, c->partials, ticket);
   });
 }
 hmc_status gsupd_launch(hmc_ctx* c, int N, VecList V, int nv, const double* h, double2* w,
                         double* ww, unsigned* ticket) {
   if (nv < 1 || nv > kMaxRestart) return fail(c, HMC_ERR_INVALID, "basis size out of range");
+  // Blocks per SM: 2 while their threads have at most 8 sites each, else 4 (us for
+  // nv 5, 10, with 8, 4 and 2 blocks: 36x36x64 16.5, 22.6; 16.1, 22.6; 14.4, 20.7;
+  // 102x102x64 61.5, 108.7; 59.8, 108.6; 58.8, 117)
+  const int cap = (N <= 8 * 2 * kThreads * c->nsm ? 2 : 4) * c->nsm;
+  const int grid = std::min(grid_for(c, N), cap);
   return launch_b(c, K_GSUPD, 16.0 * N * (nv + 2), [&] {
     switch (nv) {
 #define X(n) \
-  case n: k_gsupd<n><<<GRID(N)>>>(N, V, h, w, ww, c->partials, ticket); break;
+  case n: k_gsupd<n><<<grid, kThreads, 0, c->stream>>>(N, V, h, w, ww, c->partials, ticket); break;
       NV_CASES(X)
 #undef X
     }

@@ -226,3 +226,37 @@ def test_spcg_two_cell_kernels_with_an_unaligned_solution_vector():
     assert info.iters == ia["iters"]
     assert np.array_equal(host(buf[1:]), host(xa))
     assert true_rel(ol, w.phi, 0.1, 0.0, host(buf[1:]).astype(np.complex128), w.b.astype(np.complex64).astype(np.complex128)) < 1e-4
+
+
+@pytest.mark.parametrize("shape,steps", [((3, 5, 7), 1), ((3, 5, 7), 16), ((6, 6, 16), 7), ((34, 35, 66), 16),
+                                         ((51, 51, 64), 10), ((70, 71, 64), 3), ((70, 71, 64), 16)])
+def test_arnoldi_steps_against_numpy(shape, steps):
+    """x after one cycle of 1 .. 16 unpreconditioned steps (a tol >= 1) against
+    GMRES in numpy: the dots and updates of every basis size, on lattices with
+    fewer sites than threads and on both sides of the block counts' rules."""
+    need_gpu()
+    w = W.small(*shape, seed=2100 + sum(shape))
+    ol = OLat.from_params(w.lat)
+    A = lambda v: of.apply_MMdag(ol, w.phi, 0.3, v, 5.0)
+    V = [w.b / np.linalg.norm(w.b)]
+    H = np.zeros((steps + 1, steps), complex)
+    for j in range(steps):
+        q = A(V[j])
+        for _ in range(2):
+            for i in range(j + 1):
+                h = np.vdot(V[i], q)
+                H[i, j] += h
+                q = q - h * V[i]
+        H[j + 1, j] = np.linalg.norm(q)
+        V.append(q / H[j + 1, j])
+    e = np.zeros(steps + 1, complex)
+    e[0] = np.linalg.norm(w.b)
+    y = np.linalg.lstsq(H, e, rcond=None)[0]
+    ref = sum(y[i] * V[i] for i in range(steps))
+    with ctx_for(w.lat) as ctx:
+        x, info = ctx.solve_fgmres(dev(w.phi), 0.3, dev(w.b), sigma=5.0, tol=1e-30, restart=16, a=1e32, maxit=steps,
+                                   allow_fail=True)
+    assert info["iters"] == steps and info["iters_inner"] == 0
+    # cond(H) < 10: the normal equations and one pass of Gram-Schmidt lose its square,
+    # 100 x 2.2e-16 x 16 steps = 4e-13; five times that
+    assert np.linalg.norm(host(x) - ref) <= 2e-12 * np.linalg.norm(ref)
