@@ -65,6 +65,8 @@ const double kKernelBytesPerSite[K_COUNT] = {
 __global__ void __launch_bounds__(kThreads) k_phase(int N, const double* __restrict__ phi, PhaseTable tab,
                                                     double2* __restrict__ E,
                                                     float* __restrict__ phi32) {
+  pdl_wait();
+  pdl_trigger();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     const double x = phi[k];
     E[k] = phase_of_field(tab, x);
@@ -98,6 +100,8 @@ template <typename R, bool MASS>
 __global__ void __launch_bounds__(kThreads) k_mdag(Geo g, Phase<R> ph, R dm,
                                                    const V2<R>* __restrict__ p,
                                                    V2<R>* __restrict__ out) {
+  pdl_wait();
+  pdl_trigger();
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < g.H; q += gridDim.x * blockDim.x) {
     Nbr nb = neighbours(g, q);
     PairOut<R> o = mdag_pair<R, Phase<R>, MASS>(g, ph, dm, p, nb);
@@ -112,6 +116,8 @@ template <typename R, bool MASS, bool SHIFT>
 __global__ void __launch_bounds__(kThreads) k_m(Geo g, Phase<R> ph, R dm, const V2<R>* __restrict__ u,
                                                 const V2<R>* __restrict__ y, R sigma,
                                                 V2<R>* __restrict__ out) {
+  pdl_wait();
+  pdl_trigger();
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < g.H; q += gridDim.x * blockDim.x) {
     Nbr nb = neighbours(g, q);
     PairOut<R> o = m_pair<R, Phase<R>, MASS>(g, ph, dm, u, nb);
@@ -679,6 +685,8 @@ __global__ void __launch_bounds__(kThreads) k_resid(Geo g, Phase<R> ph, R dm,
                                                     CGScal* init, double tol2, int maxit,
                                                     double dsigma, double ddm, double* out2,
                                                     double* partials, unsigned* ticket) {
+  pdl_wait();
+  pdl_trigger();
   double acc[2] = {0.0, 0.0};
   auto body = [&](auto mass, auto shift) {
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < g.H; q += gridDim.x * blockDim.x) {
@@ -737,6 +745,8 @@ __global__ void __launch_bounds__(kThreads) k_init0(int N, const V2<R>* __restri
                                                     V2<R>* __restrict__ p, CGScal* sc, double tol2,
                                                     int maxit, double sigma, double ddm,
                                                     double* partials, unsigned* ticket) {
+  pdl_wait();
+  pdl_trigger();
   double acc[1] = {0.0};
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     Cx<R> bk = ld<R>(b, k);
@@ -768,6 +778,8 @@ __global__ void __launch_bounds__(kThreads) k_init0(int N, const V2<R>* __restri
 
 __global__ void __launch_bounds__(kThreads) k_to32(int N, const double2* __restrict__ in,
                                                    float2* __restrict__ out) {
+  pdl_wait();
+  pdl_trigger();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     double2 v = in[k];
     out[k] = make_float2((float)v.x, (float)v.y);
@@ -775,6 +787,8 @@ __global__ void __launch_bounds__(kThreads) k_to32(int N, const double2* __restr
 }
 __global__ void __launch_bounds__(kThreads) k_to64(int N, const float2* __restrict__ in,
                                                    double2* __restrict__ out) {
+  pdl_wait();
+  pdl_trigger();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     float2 v = in[k];
     out[k] = make_double2((double)v.x, (double)v.y);
@@ -783,6 +797,8 @@ __global__ void __launch_bounds__(kThreads) k_to64(int N, const float2* __restri
 
 __global__ void __launch_bounds__(kThreads) k_norm2(int N, const double2* __restrict__ v, double* out,
                                                     double* partials, unsigned* ticket) {
+  pdl_wait();
+  pdl_trigger();
   double acc[1] = {0.0};
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     double2 a = v[k];
@@ -795,6 +811,8 @@ __global__ void __launch_bounds__(kThreads) k_norm2(int N, const double2* __rest
 __global__ void __launch_bounds__(kThreads) k_redot(int N, const double2* __restrict__ u,
                                                     const double2* __restrict__ v, double* out,
                                                     double* partials, unsigned* ticket) {
+  pdl_wait();
+  pdl_trigger();
   double acc[1] = {0.0};
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     double2 a = u[k], b = v[k];
@@ -817,6 +835,8 @@ __global__ void __launch_bounds__(kThreads) k_redot(int N, const double2* __rest
 __global__ void __launch_bounds__(kThreads) k_mdot(int N, VecList V, int nv, int chunks,
                                                    const double2* __restrict__ w, double* hout,
                                                    double* partials, unsigned* ticket) {
+  pdl_wait();
+  pdl_trigger();
   const int i = (int)blockIdx.x / chunks, ch = (int)blockIdx.x - i * chunks;
   const double2* __restrict__ v = V.v[i];
   double acc[2] = {0.0, 0.0};
@@ -862,6 +882,8 @@ template <int NV>
 __global__ void __launch_bounds__(kThreads) k_gsupd(int N, VecList V, const double* h,
                                                     double2* __restrict__ w, double* ww,
                                                     double* partials, unsigned* ticket) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ double hs[2 * NV];
   if (threadIdx.x < 2 * NV) hs[threadIdx.x] = h[threadIdx.x];
   __syncthreads();
@@ -886,6 +908,8 @@ __global__ void __launch_bounds__(kThreads) k_gsupd(int N, VecList V, const doub
 // v_j = w / |w| (Algorithm A.1).
 __global__ void __launch_bounds__(kThreads) k_scale(int N, double s, const double2* __restrict__ w,
                                                     double2* __restrict__ v, float2* __restrict__ v32) {
+  pdl_wait();
+  pdl_trigger();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     double2 a = w[k];
     a.x *= s;
@@ -898,6 +922,8 @@ __global__ void __launch_bounds__(kThreads) k_scale(int N, double s, const doubl
 // x += sum_i y_i z_i, the update of Algorithm A.1 after the least-squares solve.
 __global__ void __launch_bounds__(kThreads) k_xupd(int N, VecList Z, CoefList y, int nz,
                                                    double2* __restrict__ x) {
+  pdl_wait();
+  pdl_trigger();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     double2 xk = x[k];
     for (int i = 0; i < nz; ++i) {
@@ -912,12 +938,16 @@ __global__ void __launch_bounds__(kThreads) k_xupd(int N, VecList Z, CoefList y,
 // The MD updates phi += c dt pi and pi -= d dt F (Sections 2, 4 and 5.2).
 __global__ void __launch_bounds__(kThreads) k_axpy_real(int N, double a, const double* __restrict__ x,
                                                         double* __restrict__ y) {
+  pdl_wait();
+  pdl_trigger();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x)
     y[k] = fma(a, x[k], y[k]);
 }
 
 __global__ void __launch_bounds__(kThreads) k_axpby_c(int N, double a, const double2* __restrict__ x,
                                                       double b, double2* __restrict__ y) {
+  pdl_wait();
+  pdl_trigger();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     double2 xv = x[k], yv = y[k];
     y[k] = make_double2(fma(a, xv.x, b * yv.x), fma(a, xv.y, b * yv.y));
@@ -934,6 +964,8 @@ __global__ void __launch_bounds__(kThreads) k_force(Geo g, Phase<double> ph,
                                                     const double2* __restrict__ xi,
                                                     const double2* __restrict__ chi,
                                                     double* __restrict__ grad) {
+  pdl_wait();
+  pdl_trigger();
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < g.H; q += gridDim.x * blockDim.x) {
     Nbr nb = neighbours(g, q);
 #pragma unroll
@@ -964,6 +996,8 @@ __global__ void __launch_bounds__(kThreads) k_force(Geo g, Phase<double> ph,
 __global__ void __launch_bounds__(kThreads) k_gauss_grad(int N, const double* __restrict__ phi,
                                                          double inv_dU, int accumulate,
                                                          double* __restrict__ grad) {
+  pdl_wait();
+  pdl_trigger();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     double v = phi[k] * inv_dU;
     grad[k] = accumulate ? grad[k] + v : v;
@@ -974,6 +1008,8 @@ __global__ void __launch_bounds__(kThreads) k_gauss_grad(int N, const double* __
 __global__ void __launch_bounds__(kThreads) k_half_sq(int N, const double* __restrict__ a, double sa,
                                                       const double* __restrict__ b, double* out,
                                                       double* partials, unsigned* ticket) {
+  pdl_wait();
+  pdl_trigger();
   double acc[2] = {0.0, 0.0};
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     double x = a[k];
@@ -992,16 +1028,13 @@ __global__ void __launch_bounds__(kThreads) k_half_sq(int N, const double* __res
 
 // ---------------------------------------------------------------------------
 // Launchers
-#define GRID(work) grid_for(c, (work)), kThreads, 0, c->stream
+#define GRID(work) dim3(grid_for(c, (work))), kThreads, c->stream
 #define PDL(id, work) dim3(shape_grid(c, (id), (work))), c->shape[(id)].threads, c->stream
-
-// tuned launch shape of a CG kernel
-#define SHAPE(id, work) shape_grid(c, (id), (work)), c->shape[(id)].threads, 0, c->stream
 
 hmc_status k_phase_launch(hmc_ctx* c, const double* phi) {
   const int N = c->geo.N;
   return launch(c, K_PHASE, [&] {
-    k_phase<<<GRID(N)>>>(N, phi, PhaseTable{c->phase_tab}, (double2*)c->ws[WS_E], (float*)c->ws[WS_PHI32]);
+    launch_pdl(c, k_phase, GRID(N), N, phi, PhaseTable{c->phase_tab}, (double2*)c->ws[WS_E], (float*)c->ws[WS_PHI32]);
   });
 }
 
@@ -1010,9 +1043,9 @@ hmc_status mdag_launch(hmc_ctx* c, const Geo& g, R dm, const V2<R>* p, V2<R>* ou
   return launch(c, sizeof(R) == 8 ? K_MDAG64 : K_MDAG32,
                 [&] {
                   if (dm != R(0))
-                    k_mdag<R, true><<<GRID(g.H)>>>(g, phase_of<R>(c), dm, p, out);
+                    launch_pdl(c, k_mdag<R, true>, GRID(g.H), g, phase_of<R>(c), dm, p, out);
                   else
-                    k_mdag<R, false><<<GRID(g.H)>>>(g, phase_of<R>(c), dm, p, out);
+                    launch_pdl(c, k_mdag<R, false>, GRID(g.H), g, phase_of<R>(c), dm, p, out);
                 });
 }
 template <typename R>
@@ -1024,13 +1057,13 @@ hmc_status m_launch(hmc_ctx* c, const Geo& g, R dm, const V2<R>* u, const V2<R>*
                   const Phase<R> ph = phase_of<R>(c);
                   if (dm != R(0)) {
                     if (y != nullptr)
-                      k_m<R, true, true><<<GRID(g.H)>>>(g, ph, dm, u, y, sigma, out);
+                      launch_pdl(c, k_m<R, true, true>, GRID(g.H), g, ph, dm, u, y, sigma, out);
                     else
-                      k_m<R, true, false><<<GRID(g.H)>>>(g, ph, dm, u, y, sigma, out);
+                      launch_pdl(c, k_m<R, true, false>, GRID(g.H), g, ph, dm, u, y, sigma, out);
                   } else if (y != nullptr) {
-                    k_m<R, false, true><<<GRID(g.H)>>>(g, ph, dm, u, y, sigma, out);
+                    launch_pdl(c, k_m<R, false, true>, GRID(g.H), g, ph, dm, u, y, sigma, out);
                   } else {
-                    k_m<R, false, false><<<GRID(g.H)>>>(g, ph, dm, u, y, sigma, out);
+                    launch_pdl(c, k_m<R, false, false>, GRID(g.H), g, ph, dm, u, y, sigma, out);
                   }
                 });
 }
@@ -1060,7 +1093,7 @@ hmc_status resid_launch(hmc_ctx* c, const Geo& g, R dm, const V2<R>* u, const V2
                         const V2<R>* b, double sigma, V2<R>* r, V2<R>* p, CGScal* init,
                         double tol2, int maxit, double* out2, unsigned* ticket, double ddm) {
   return launch(c, sizeof(R) == 8 ? K_RESID64 : K_RESID32, [&] {
-    k_resid<R><<<GRID(g.H)>>>(g, phase_of<R>(c), dm, u, x, b, (R)sigma, r, p, init, tol2, maxit,
+    launch_pdl(c, k_resid<R>, GRID(g.H), g, phase_of<R>(c), dm, u, x, b, (R)sigma, r, p, init, tol2, maxit,
                               sigma, ddm, out2, c->partials, ticket);
   });
 }
@@ -1068,7 +1101,7 @@ template <typename R>
 hmc_status init0_launch(hmc_ctx* c, int N, const V2<R>* b, V2<R>* x, V2<R>* r, V2<R>* p, CGScal* sc,
                         double tol2, int maxit, double sigma, unsigned* ticket, double ddm) {
   return launch(c, K_INIT0, [&] {
-    k_init0<R><<<GRID(N)>>>(N, b, x, r, p, sc, tol2, maxit, sigma, ddm, c->partials, ticket);
+    launch_pdl(c, k_init0<R>, GRID(N), N, b, x, r, p, sc, tol2, maxit, sigma, ddm, c->partials, ticket);
   });
 }
 
@@ -1169,17 +1202,17 @@ int cg_kernel_occupancy(int id, int threads, int pairs) {
 }
 
 hmc_status to32_launch(hmc_ctx* c, int N, const double2* in, float2* out) {
-  return launch(c, K_CONVERT, [&] { k_to32<<<GRID(N)>>>(N, in, out); });
+  return launch(c, K_CONVERT, [&] { launch_pdl(c, k_to32, GRID(N), N, in, out); });
 }
 hmc_status to64_launch(hmc_ctx* c, int N, const float2* in, double2* out) {
-  return launch(c, K_CONVERT, [&] { k_to64<<<GRID(N)>>>(N, in, out); });
+  return launch(c, K_CONVERT, [&] { launch_pdl(c, k_to64, GRID(N), N, in, out); });
 }
 hmc_status norm2_launch(hmc_ctx* c, int N, const double2* v, double* out, unsigned* ticket) {
-  return launch(c, K_NORM, [&] { k_norm2<<<GRID(N)>>>(N, v, out, c->partials, ticket); });
+  return launch(c, K_NORM, [&] { launch_pdl(c, k_norm2, GRID(N), N, v, out, c->partials, ticket); });
 }
 hmc_status redot_launch(hmc_ctx* c, int N, const double2* u, const double2* v, double* out,
                         unsigned* ticket) {
-  return launch(c, K_NORM, [&] { k_redot<<<GRID(N)>>>(N, u, v, out, c->partials, ticket); });
+  return launch(c, K_NORM, [&] { launch_pdl(c, k_redot, GRID(N), N, u, v, out, c->partials, ticket); });
 }
 #define NV_CASES(X) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12) X(13) X(14) X(15) X(16)
 
@@ -1191,8 +1224,15 @@ hmc_status mdot_launch(hmc_ctx* c, int N, VecList V, int nv, const double2* w, d
   // 12.4; 51x51x64 nv 5 20.6 and 20.6, nv 10 33.1 and 32.9, nv 16 63 and 49)
   const int per_sm = (double)N * nv <= 64.0 * kThreads * c->nsm ? 1 : 2;
   const int chunks = std::max(1, std::min((N + kThreads - 1) / kThreads, per_sm * c->nsm / nv));
+  // Ordinary launch behind an M with more blocks than SMs: its few blocks, placed
+  // as M's leave, would share the first SMs that empty (solve at 36x36x64, early
+  // 4.96 ms, ordinary 4.89; 102x102x64 13.2, 12.5; 24x24x48 and below the same)
+  const bool early = grid_for(c, N / 2) <= c->nsm;
   return launch_b(c, K_MDOT, 16.0 * N * (nv + 1), [&] {
-    k_mdot<<<nv * chunks, kThreads, 0, c->stream>>>(N, V, nv, chunks, w, hout, c->partials, ticket);
+    if (early)
+      launch_pdl(c, k_mdot, dim3(nv * chunks), kThreads, c->stream, N, V, nv, chunks, w, hout, c->partials, ticket);
+    else
+      k_mdot<<<nv * chunks, kThreads, 0, c->stream>>>(N, V, nv, chunks, w, hout, c->partials, ticket);
   });
 }
 hmc_status gsupd_launch(hmc_ctx* c, int N, VecList V, int nv, const double* h, double2* w,
@@ -1206,37 +1246,37 @@ hmc_status gsupd_launch(hmc_ctx* c, int N, VecList V, int nv, const double* h, d
   return launch_b(c, K_GSUPD, 16.0 * N * (nv + 2), [&] {
     switch (nv) {
 #define X(n) \
-  case n: k_gsupd<n><<<grid, kThreads, 0, c->stream>>>(N, V, h, w, ww, c->partials, ticket); break;
+  case n: launch_pdl(c, k_gsupd<n>, dim3(grid), kThreads, c->stream, N, V, h, w, ww, c->partials, ticket); break;
       NV_CASES(X)
 #undef X
     }
   });
 }
 hmc_status scale_launch(hmc_ctx* c, int N, double s, const double2* w, double2* v, float2* v32) {
-  return launch(c, K_SCALE, [&] { k_scale<<<GRID(N)>>>(N, s, w, v, v32); });
+  return launch(c, K_SCALE, [&] { launch_pdl(c, k_scale, GRID(N), N, s, w, v, v32); });
 }
 hmc_status xupd_launch(hmc_ctx* c, int N, VecList Z, CoefList y, int nz, double2* x) {
-  return launch_b(c, K_XUPD, 16.0 * N * (nz + 2), [&] { k_xupd<<<GRID(N)>>>(N, Z, y, nz, x); });
+  return launch_b(c, K_XUPD, 16.0 * N * (nz + 2), [&] { launch_pdl(c, k_xupd, GRID(N), N, Z, y, nz, x); });
 }
 hmc_status axpy_real_launch(hmc_ctx* c, int N, double a, const double* x, double* y) {
-  return launch(c, K_AXPY, [&] { k_axpy_real<<<GRID(N)>>>(N, a, x, y); });
+  return launch(c, K_AXPY, [&] { launch_pdl(c, k_axpy_real, GRID(N), N, a, x, y); });
 }
 hmc_status axpby_c_launch(hmc_ctx* c, int N, double a, const double2* x, double b, double2* y) {
-  return launch(c, K_AXPY, [&] { k_axpby_c<<<GRID(N)>>>(N, a, x, b, y); });
+  return launch(c, K_AXPY, [&] { launch_pdl(c, k_axpby_c, GRID(N), N, a, x, b, y); });
 }
 hmc_status force_launch(hmc_ctx* c, const Geo& g, const double2* eta, const double2* xi,
                         const double2* chi, double* grad) {
   return launch(c, K_FORCE,
-                [&] { k_force<<<GRID(g.H)>>>(g, phase_of<double>(c), eta, xi, chi, grad); });
+                [&] { launch_pdl(c, k_force, GRID(g.H), g, phase_of<double>(c), eta, xi, chi, grad); });
 }
 hmc_status gauss_grad_launch(hmc_ctx* c, int N, const double* phi, double inv_dU, int accumulate,
                              double* grad) {
-  return launch(c, K_MD, [&] { k_gauss_grad<<<GRID(N)>>>(N, phi, inv_dU, accumulate, grad); });
+  return launch(c, K_MD, [&] { launch_pdl(c, k_gauss_grad, GRID(N), N, phi, inv_dU, accumulate, grad); });
 }
 hmc_status half_sq_launch(hmc_ctx* c, int N, const double* a, double sa, const double* b, double* out,
                           unsigned* ticket) {
   return launch(c, K_NORM,
-                [&] { k_half_sq<<<GRID(N)>>>(N, a, sa, b, out, c->partials, ticket); });
+                [&] { launch_pdl(c, k_half_sq, GRID(N), N, a, sa, b, out, c->partials, ticket); });
 }
 
 }  // namespace hmc
