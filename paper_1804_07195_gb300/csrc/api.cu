@@ -239,14 +239,14 @@ void destroy_graphs(hmc_ctx* c) {
   c->graphs.clear();
 }
 
-hmc_status prepare_field(hmc_ctx* c, const double* phi) {
+hmc_status prepare_field(hmc_ctx* c, const double* phi, Tables t) {
   if (phi == nullptr) {
     if (!c->field_loaded) return fail(c, HMC_ERR_INVALID, "phi is NULL and no field was loaded");
     return HMC_OK;
   }
   if (((uintptr_t)phi) % 8) return fail(c, HMC_ERR_INVALID, "phi is not 8-byte aligned");
   c->field_loaded = false;
-  return k_phase_launch(c, phi);
+  return t == Tables::none ? HMC_OK : k_phase_launch(c, phi, t == Tables::all);
 }
 
 }  // namespace hmc
@@ -453,6 +453,16 @@ hmc_status hmc_load_field(hmc_ctx* c, const double* phi) {
   return HMC_OK;
 }
 
+// A single M or M^dagger: *own is the field to form the phases from in the kernel,
+// NULL where they come from the tables (the loaded field, or a phi that out
+// overlaps, which has to be read before out is written).
+static hmc_status prepare_own(hmc_ctx* c, const double* phi, const void* out, int prec, const double** own) {
+  const bool direct = phi != nullptr && !ranges_overlap(phi, out, vec_bytes(c, 64));
+  HMC_TRY(prepare_field(c, phi, direct ? Tables::none : prec == 64 ? Tables::all : Tables::f32));
+  *own = direct ? phi : nullptr;
+  return HMC_OK;
+}
+
 hmc_status hmc_apply_M(hmc_ctx* c, const double* phi, double ms, const void* in, void* out, int prec) {
   if (!c) return HMC_ERR_INVALID;
   HMC_TRACE("hmc_apply_M");
@@ -461,10 +471,10 @@ hmc_status hmc_apply_M(hmc_ctx* c, const double* phi, double ms, const void* in,
   HMC_TRY(check_vec(c, out, prec, "out"));
   HMC_TRY(check_mass(c, ms));
   if (ranges_overlap(in, out, vec_bytes(c, prec))) return fail(c, HMC_ERR_INVALID, "in and out must not overlap");
-  HMC_TRY(prepare_field(c, phi));
+  HMC_TRY(prepare_own(c, phi, out, prec, &phi));
   if (prec == 64)
-    return m_launch<double>(c, c->geo, c->delta * ms, (const double2*)in, nullptr, 0.0, (double2*)out);
-  return m_launch<float>(c, c->geo, (float)(c->delta * ms), (const float2*)in, nullptr, 0.f, (float2*)out);
+    return m_launch<double>(c, c->geo, c->delta * ms, (const double2*)in, nullptr, 0.0, (double2*)out, phi);
+  return m_launch<float>(c, c->geo, (float)(c->delta * ms), (const float2*)in, nullptr, 0.f, (float2*)out, phi);
 }
 
 hmc_status hmc_apply_Mdag(hmc_ctx* c, const double* phi, double ms, const void* in, void* out, int prec) {
@@ -475,9 +485,9 @@ hmc_status hmc_apply_Mdag(hmc_ctx* c, const double* phi, double ms, const void* 
   HMC_TRY(check_vec(c, out, prec, "out"));
   HMC_TRY(check_mass(c, ms));
   if (ranges_overlap(in, out, vec_bytes(c, prec))) return fail(c, HMC_ERR_INVALID, "in and out must not overlap");
-  HMC_TRY(prepare_field(c, phi));
-  if (prec == 64) return mdag_launch<double>(c, c->geo, c->delta * ms, (const double2*)in, (double2*)out);
-  return mdag_launch<float>(c, c->geo, (float)(c->delta * ms), (const float2*)in, (float2*)out);
+  HMC_TRY(prepare_own(c, phi, out, prec, &phi));
+  if (prec == 64) return mdag_launch<double>(c, c->geo, c->delta * ms, (const double2*)in, (double2*)out, phi);
+  return mdag_launch<float>(c, c->geo, (float)(c->delta * ms), (const float2*)in, (float2*)out, phi);
 }
 
 hmc_status hmc_apply_MMdag(hmc_ctx* c, const double* phi, double ms, double sigma, const void* in,
@@ -490,7 +500,11 @@ hmc_status hmc_apply_MMdag(hmc_ctx* c, const double* phi, double ms, double sigm
   HMC_TRY(check_mass(c, ms));
   if (!(sigma >= 0.0) || !std::isfinite(sigma)) return fail(c, HMC_ERR_INVALID, "sigma must be finite and >= 0");
   if (ranges_overlap(in, out, vec_bytes(c, prec))) return fail(c, HMC_ERR_INVALID, "in and out must not overlap");
-  HMC_TRY(prepare_field(c, phi));
+  // FP64 in two passes: M^dagger forms the phases and leaves them for M
+  const bool two_pass = (c->apply_variant ? c->apply_variant : c->apply_choice[1]) == 1;
+  const bool direct = prec == 64 && phi != nullptr && two_pass;
+  HMC_TRY(prepare_field(c, phi, direct ? Tables::none : prec == 64 ? Tables::all : Tables::f32));
+  if (direct) return apply_A64(c, ms, sigma, (const double2*)in, (double2*)out, phi);
   if (prec == 64) return apply_A<double>(c, ms, sigma, (const double2*)in, (double2*)out);
   return apply_A<float>(c, ms, sigma, (const float2*)in, (float2*)out);
 }
@@ -547,7 +561,7 @@ hmc_status hmc_solve_spcg(hmc_ctx* c, const double* phi, double ms, double sigma
   HMC_TRACE("hmc_solve_spcg");
   const double t0 = now_s();
   HMC_TRY(solve_checks(c, ms, sigma, b, x, 32, tol, maxit));
-  HMC_TRY(prepare_field(c, phi));
+  HMC_TRY(prepare_field(c, phi, Tables::f32));
   SolveStats s;
   // the kernels with two cells per thread access x in 16-byte units: an x
   // that is only 8-byte aligned is solved in a workspace vector and copied

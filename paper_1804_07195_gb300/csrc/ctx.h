@@ -353,7 +353,10 @@ GraphEntry* find_graph(hmc_ctx* c, int kind, const void* const key[6]);
 GraphEntry* add_graph(hmc_ctx* c, int kind, const void* const key[6], cudaGraphExec_t exec);
 void destroy_graphs(hmc_ctx* c);
 
-// Build the phase tables of phi (or reuse the loaded field when phi is NULL).
-hmc_status prepare_field(hmc_ctx* c, const double* phi);
+// Build the phase tables of phi (or reuse the loaded field when phi is NULL):
+// both, the float one only (a call in single precision; what is built for a call
+// serves that call alone), or none (the call forms its phases itself).
+enum class Tables { none, f32, all };
+hmc_status prepare_field(hmc_ctx* c, const double* phi, Tables t = Tables::all);
 
 }  // namespace hmc

@@ -4,6 +4,7 @@
 // Passages: the operator of Eq. ferm_op (Section 2), CG (Section 3), the vector
 // steps of Algorithm A.1 (Appendix A), the force of Eqs. p_dot, f_chi_i and
 // def_xi_i, the energies of Eq. hamiltonian.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -60,16 +61,17 @@ const double kKernelBytesPerSite[K_COUNT] = {
     0};                  // resident CG f64: 208 B (the pair of kernels and the p update)
 
 // ---------------------------------------------------------------------------
-// e^{i phi} for the FP64 stencils of Eq. ferm_op, and phi rounded to float. Bound
-// by the FP64 pipe: 102x102x64 45 us (74 with sincos), 51x51x64 14.4 (22.5).
+// e^{i phi} for the FP64 stencils of Eq. ferm_op (E, not formed where NULL: calls
+// that stay in single precision), and phi rounded to float. Bound by the FP64 pipe:
+// 102x102x64 42.8 us (74 with sincos), 51x51x64 11.9 (22.5). Without E by memory: FP32
+// M M^dagger with its field at 102x102x64 54.9 -> 12.7 us.
 __global__ void __launch_bounds__(kThreads) k_phase(int N, const double* __restrict__ phi, PhaseTable tab,
                                                     double2* __restrict__ E,
                                                     float* __restrict__ phi32) {
   pdl_wait();
-  pdl_trigger();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     const double x = phi[k];
-    E[k] = phase_of_field(tab, x);
+    if (E != nullptr) E[k] = phase_of_field(tab, x);
     phi32[k] = field_to_f32(x);
   }
 }
@@ -96,15 +98,18 @@ void phase_table_host(double2* out) {
 
 
 // out = M^dagger p (Eq. ferm_op, conjugate transpose), one cell-time per thread.
-template <typename R, bool MASS>
-__global__ void __launch_bounds__(kThreads) k_mdag(Geo g, Phase<R> ph, R dm,
+// PH: the phases from the tables, or from the field (FieldPhase) for a single
+// application, whose rows use each phase once: no pass to build the tables, no
+// table read back (us, M^dagger with its field: FP64 at 6x6x16 6.8 -> 4.9, 51x51x64
+// 18.7 -> 16.1, 102x102x64 65.5 -> 58.0; FP32 at 102x102x64 49.1 -> 4.9).
+template <typename R, bool MASS, typename PH>
+__global__ void __launch_bounds__(kThreads) k_mdag(Geo g, PH ph, R dm,
                                                    const V2<R>* __restrict__ p,
                                                    V2<R>* __restrict__ out) {
   pdl_wait();
-  pdl_trigger();
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < g.H; q += gridDim.x * blockDim.x) {
     Nbr nb = neighbours(g, q);
-    PairOut<R> o = mdag_pair<R, Phase<R>, MASS>(g, ph, dm, p, nb);
+    PairOut<R> o = mdag_pair<R, PH, MASS>(g, ph, dm, p, nb);
     st(out, q, o.a);
     st(out, g.H + q, o.b);
   }
@@ -112,15 +117,14 @@ __global__ void __launch_bounds__(kThreads) k_mdag(Geo g, Phase<R> ph, R dm,
 
 // out = M u + sigma y (Eq. ferm_op; SHIFT = false: sigma = 0), one cell-time per
 // thread.
-template <typename R, bool MASS, bool SHIFT>
-__global__ void __launch_bounds__(kThreads) k_m(Geo g, Phase<R> ph, R dm, const V2<R>* __restrict__ u,
+template <typename R, bool MASS, bool SHIFT, typename PH>
+__global__ void __launch_bounds__(kThreads) k_m(Geo g, PH ph, R dm, const V2<R>* __restrict__ u,
                                                 const V2<R>* __restrict__ y, R sigma,
                                                 V2<R>* __restrict__ out) {
   pdl_wait();
-  pdl_trigger();
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < g.H; q += gridDim.x * blockDim.x) {
     Nbr nb = neighbours(g, q);
-    PairOut<R> o = m_pair<R, Phase<R>, MASS>(g, ph, dm, u, nb);
+    PairOut<R> o = m_pair<R, PH, MASS>(g, ph, dm, u, nb);
     if (SHIFT) {
       Cx<R> ya = ld<R>(y, q), yb = ld<R>(y, g.H + q);
       o.a.re = fma(sigma, ya.re, o.a.re);
@@ -686,7 +690,6 @@ __global__ void __launch_bounds__(kThreads) k_resid(Geo g, Phase<R> ph, R dm,
                                                     double dsigma, double ddm, double* out2,
                                                     double* partials, unsigned* ticket) {
   pdl_wait();
-  pdl_trigger();
   double acc[2] = {0.0, 0.0};
   auto body = [&](auto mass, auto shift) {
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < g.H; q += gridDim.x * blockDim.x) {
@@ -746,7 +749,6 @@ __global__ void __launch_bounds__(kThreads) k_init0(int N, const V2<R>* __restri
                                                     int maxit, double sigma, double ddm,
                                                     double* partials, unsigned* ticket) {
   pdl_wait();
-  pdl_trigger();
   double acc[1] = {0.0};
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     Cx<R> bk = ld<R>(b, k);
@@ -779,7 +781,6 @@ __global__ void __launch_bounds__(kThreads) k_init0(int N, const V2<R>* __restri
 __global__ void __launch_bounds__(kThreads) k_to32(int N, const double2* __restrict__ in,
                                                    float2* __restrict__ out) {
   pdl_wait();
-  pdl_trigger();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     double2 v = in[k];
     out[k] = make_float2((float)v.x, (float)v.y);
@@ -788,7 +789,6 @@ __global__ void __launch_bounds__(kThreads) k_to32(int N, const double2* __restr
 __global__ void __launch_bounds__(kThreads) k_to64(int N, const float2* __restrict__ in,
                                                    double2* __restrict__ out) {
   pdl_wait();
-  pdl_trigger();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     float2 v = in[k];
     out[k] = make_double2((double)v.x, (double)v.y);
@@ -798,7 +798,6 @@ __global__ void __launch_bounds__(kThreads) k_to64(int N, const float2* __restri
 __global__ void __launch_bounds__(kThreads) k_norm2(int N, const double2* __restrict__ v, double* out,
                                                     double* partials, unsigned* ticket) {
   pdl_wait();
-  pdl_trigger();
   double acc[1] = {0.0};
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     double2 a = v[k];
@@ -812,7 +811,6 @@ __global__ void __launch_bounds__(kThreads) k_redot(int N, const double2* __rest
                                                     const double2* __restrict__ v, double* out,
                                                     double* partials, unsigned* ticket) {
   pdl_wait();
-  pdl_trigger();
   double acc[1] = {0.0};
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     double2 a = u[k], b = v[k];
@@ -836,7 +834,6 @@ __global__ void __launch_bounds__(kThreads) k_mdot(int N, VecList V, int nv, int
                                                    const double2* __restrict__ w, double* hout,
                                                    double* partials, unsigned* ticket) {
   pdl_wait();
-  pdl_trigger();
   const int i = (int)blockIdx.x / chunks, ch = (int)blockIdx.x - i * chunks;
   const double2* __restrict__ v = V.v[i];
   double acc[2] = {0.0, 0.0};
@@ -883,7 +880,6 @@ __global__ void __launch_bounds__(kThreads) k_gsupd(int N, VecList V, const doub
                                                     double2* __restrict__ w, double* ww,
                                                     double* partials, unsigned* ticket) {
   pdl_wait();
-  pdl_trigger();
   __shared__ double hs[2 * NV];
   if (threadIdx.x < 2 * NV) hs[threadIdx.x] = h[threadIdx.x];
   __syncthreads();
@@ -909,7 +905,6 @@ __global__ void __launch_bounds__(kThreads) k_gsupd(int N, VecList V, const doub
 __global__ void __launch_bounds__(kThreads) k_scale(int N, double s, const double2* __restrict__ w,
                                                     double2* __restrict__ v, float2* __restrict__ v32) {
   pdl_wait();
-  pdl_trigger();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     double2 a = w[k];
     a.x *= s;
@@ -923,7 +918,6 @@ __global__ void __launch_bounds__(kThreads) k_scale(int N, double s, const doubl
 __global__ void __launch_bounds__(kThreads) k_xupd(int N, VecList Z, CoefList y, int nz,
                                                    double2* __restrict__ x) {
   pdl_wait();
-  pdl_trigger();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     double2 xk = x[k];
     for (int i = 0; i < nz; ++i) {
@@ -939,7 +933,6 @@ __global__ void __launch_bounds__(kThreads) k_xupd(int N, VecList Z, CoefList y,
 __global__ void __launch_bounds__(kThreads) k_axpy_real(int N, double a, const double* __restrict__ x,
                                                         double* __restrict__ y) {
   pdl_wait();
-  pdl_trigger();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x)
     y[k] = fma(a, x[k], y[k]);
 }
@@ -947,7 +940,6 @@ __global__ void __launch_bounds__(kThreads) k_axpy_real(int N, double a, const d
 __global__ void __launch_bounds__(kThreads) k_axpby_c(int N, double a, const double2* __restrict__ x,
                                                       double b, double2* __restrict__ y) {
   pdl_wait();
-  pdl_trigger();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     double2 xv = x[k], yv = y[k];
     y[k] = make_double2(fma(a, xv.x, b * yv.x), fma(a, xv.y, b * yv.y));
@@ -965,7 +957,6 @@ __global__ void __launch_bounds__(kThreads) k_force(Geo g, Phase<double> ph,
                                                     const double2* __restrict__ chi,
                                                     double* __restrict__ grad) {
   pdl_wait();
-  pdl_trigger();
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < g.H; q += gridDim.x * blockDim.x) {
     Nbr nb = neighbours(g, q);
 #pragma unroll
@@ -997,7 +988,6 @@ __global__ void __launch_bounds__(kThreads) k_gauss_grad(int N, const double* __
                                                          double inv_dU, int accumulate,
                                                          double* __restrict__ grad) {
   pdl_wait();
-  pdl_trigger();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     double v = phi[k] * inv_dU;
     grad[k] = accumulate ? grad[k] + v : v;
@@ -1009,7 +999,6 @@ __global__ void __launch_bounds__(kThreads) k_half_sq(int N, const double* __res
                                                       const double* __restrict__ b, double* out,
                                                       double* partials, unsigned* ticket) {
   pdl_wait();
-  pdl_trigger();
   double acc[2] = {0.0, 0.0};
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < N; k += gridDim.x * blockDim.x) {
     double x = a[k];
@@ -1029,43 +1018,65 @@ __global__ void __launch_bounds__(kThreads) k_half_sq(int N, const double* __res
 // ---------------------------------------------------------------------------
 // Launchers
 #define GRID(work) dim3(grid_for(c, (work))), kThreads, c->stream
+// One item a thread in blocks of 128, for the kernels whose FP64 work per site makes
+// the SM with the most blocks the last (us, with 256 threads and 8 blocks a SM:
+// M^dagger at 51x51x64 6.1 (6.45), 102x102x64 18.5 (20.2); phases 11.9, 42.8 (11.9,
+// 43.3); both in one 18.3, 58.0 (18.6, 62.8), 36x36x64 9.6 (11.3))
+inline int grid_128(const hmc_ctx* c, long long work) {
+  return (int)std::max(1ll, std::min((work + 127) / 128, (long long)c->nsm * kOneItemBlocksPerSM * 2));
+}
+#define GRID128(work) dim3(grid_128(c, (work))), 128, c->stream
 #define PDL(id, work) dim3(shape_grid(c, (id), (work))), c->shape[(id)].threads, c->stream
 
-hmc_status k_phase_launch(hmc_ctx* c, const double* phi) {
+hmc_status k_phase_launch(hmc_ctx* c, const double* phi, bool table64) {
   const int N = c->geo.N;
+  const PhaseTable tab{c->phase_tab};
+  float* const phi32 = (float*)c->ws[WS_PHI32];
   return launch(c, K_PHASE, [&] {
-    launch_pdl(c, k_phase, GRID(N), N, phi, PhaseTable{c->phase_tab}, (double2*)c->ws[WS_E], (float*)c->ws[WS_PHI32]);
+    if (table64)
+      launch_pdl(c, k_phase, GRID128(N), N, phi, tab, (double2*)c->ws[WS_E], phi32);
+    else
+      launch_pdl(c, k_phase, GRID(N), N, phi, tab, (double2*)nullptr, phi32);
   });
 }
 
 template <typename R>
-hmc_status mdag_launch(hmc_ctx* c, const Geo& g, R dm, const V2<R>* p, V2<R>* out) {
-  return launch(c, sizeof(R) == 8 ? K_MDAG64 : K_MDAG32,
-                [&] {
-                  if (dm != R(0))
-                    launch_pdl(c, k_mdag<R, true>, GRID(g.H), g, phase_of<R>(c), dm, p, out);
-                  else
-                    launch_pdl(c, k_mdag<R, false>, GRID(g.H), g, phase_of<R>(c), dm, p, out);
-                });
+hmc_status mdag_launch(hmc_ctx* c, const Geo& g, R dm, const V2<R>* p, V2<R>* out, const double* phi, bool keep) {
+  return launch(c, sizeof(R) == 8 ? K_MDAG64 : K_MDAG32, [&] {
+    auto go = [&](auto ph) {
+      using PH = decltype(ph);
+      auto* const k = dm != R(0) ? k_mdag<R, true, PH> : k_mdag<R, false, PH>;
+      if (sizeof(R) == 8)
+        launch_pdl(c, k, GRID128(g.H), g, ph, dm, p, out);
+      else
+        launch_pdl(c, k, GRID(g.H), g, ph, dm, p, out);
+    };
+    if (phi != nullptr)
+      go(field_phase<R>(c, phi, keep));
+    else
+      go(phase_of<R>(c));
+  });
 }
 template <typename R>
-hmc_status m_launch(hmc_ctx* c, const Geo& g, R dm, const V2<R>* u, const V2<R>* y, R sigma,
-                    V2<R>* out) {
-  return launch(c, sizeof(R) == 8 ? K_M64 : K_M32,
-                [&] {
-                  // an instance per case: a predicated-off instruction takes the FP64 pipe too
-                  const Phase<R> ph = phase_of<R>(c);
-                  if (dm != R(0)) {
-                    if (y != nullptr)
-                      launch_pdl(c, k_m<R, true, true>, GRID(g.H), g, ph, dm, u, y, sigma, out);
-                    else
-                      launch_pdl(c, k_m<R, true, false>, GRID(g.H), g, ph, dm, u, y, sigma, out);
-                  } else if (y != nullptr) {
-                    launch_pdl(c, k_m<R, false, true>, GRID(g.H), g, ph, dm, u, y, sigma, out);
-                  } else {
-                    launch_pdl(c, k_m<R, false, false>, GRID(g.H), g, ph, dm, u, y, sigma, out);
-                  }
-                });
+hmc_status m_launch(hmc_ctx* c, const Geo& g, R dm, const V2<R>* u, const V2<R>* y, R sigma, V2<R>* out,
+                    const double* phi) {
+  return launch(c, sizeof(R) == 8 ? K_M64 : K_M32, [&] {
+    // an instance per case: a predicated-off instruction takes the FP64 pipe too
+    auto go = [&](auto k, auto ph) {
+      if (sizeof(R) == 8)
+        launch_pdl(c, k, GRID128(g.H), g, ph, dm, u, y, sigma, out);
+      else
+        launch_pdl(c, k, GRID(g.H), g, ph, dm, u, y, sigma, out);
+    };
+    using F = FieldPhase<R>;
+    using P = Phase<R>;
+    if (phi != nullptr)  // M alone: no shift
+      go(dm != R(0) ? k_m<R, true, false, F> : k_m<R, false, false, F>, field_phase<R>(c, phi, false));
+    else if (y != nullptr)
+      go(dm != R(0) ? k_m<R, true, true, P> : k_m<R, false, true, P>, phase_of<R>(c));
+    else
+      go(dm != R(0) ? k_m<R, true, false, P> : k_m<R, false, false, P>, phase_of<R>(c));
+  });
 }
 template <typename R>
 hmc_status cg_mdag_launch(hmc_ctx* c, const Geo& g, const V2<R>* p, V2<R>* u, CGScal* sc,
@@ -1106,9 +1117,10 @@ hmc_status init0_launch(hmc_ctx* c, int N, const V2<R>* b, V2<R>* x, V2<R>* r, V
 }
 
 #define INST(R)                                                                                   \
-  template hmc_status mdag_launch<R>(hmc_ctx*, const Geo&, R, const V2<R>*, V2<R>*);             \
+  template hmc_status mdag_launch<R>(hmc_ctx*, const Geo&, R, const V2<R>*, V2<R>*, const double*, \
+                                     bool);                                                       \
   template hmc_status m_launch<R>(hmc_ctx*, const Geo&, R, const V2<R>*, const V2<R>*, R,        \
-                                  V2<R>*);                                                        \
+                                  V2<R>*, const double*);                                         \
   template hmc_status cg_mdag_launch<R>(hmc_ctx*, const Geo&, const V2<R>*, V2<R>*, CGScal*,     \
                                         unsigned*);                                               \
   template hmc_status cg_m_launch<R>(hmc_ctx*, const Geo&, const V2<R>*, const V2<R>*,           \
@@ -1224,15 +1236,8 @@ hmc_status mdot_launch(hmc_ctx* c, int N, VecList V, int nv, const double2* w, d
   // 12.4; 51x51x64 nv 5 20.6 and 20.6, nv 10 33.1 and 32.9, nv 16 63 and 49)
   const int per_sm = (double)N * nv <= 64.0 * kThreads * c->nsm ? 1 : 2;
   const int chunks = std::max(1, std::min((N + kThreads - 1) / kThreads, per_sm * c->nsm / nv));
-  // Ordinary launch behind an M with more blocks than SMs: its few blocks, placed
-  // as M's leave, would share the first SMs that empty (solve at 36x36x64, early
-  // 4.96 ms, ordinary 4.89; 102x102x64 13.2, 12.5; 24x24x48 and below the same)
-  const bool early = grid_for(c, N / 2) <= c->nsm;
   return launch_b(c, K_MDOT, 16.0 * N * (nv + 1), [&] {
-    if (early)
-      launch_pdl(c, k_mdot, dim3(nv * chunks), kThreads, c->stream, N, V, nv, chunks, w, hout, c->partials, ticket);
-    else
-      k_mdot<<<nv * chunks, kThreads, 0, c->stream>>>(N, V, nv, chunks, w, hout, c->partials, ticket);
+    launch_pdl(c, k_mdot, dim3(nv * chunks), kThreads, c->stream, N, V, nv, chunks, w, hout, c->partials, ticket);
   });
 }
 hmc_status gsupd_launch(hmc_ctx* c, int N, VecList V, int nv, const double* h, double2* w,

@@ -11,15 +11,18 @@ namespace hmc {
 template <typename R>
 using V2 = typename Vec2<R>::type;
 
-// Phase tables: E = e^{i phi} (complex128) and phi rounded to float.
-hmc_status k_phase_launch(hmc_ctx* c, const double* phi);
+// Phase tables: E = e^{i phi} (complex128; with table64) and phi rounded to float.
+hmc_status k_phase_launch(hmc_ctx* c, const double* phi, bool table64);
 
-// out = M^dagger p, out = M u + sigma y (y may be NULL).
+// out = M^dagger p, out = M u + sigma y (y may be NULL). With phi the phases are
+// formed from that field and not read from the tables (M: y NULL; the FP64
+// M^dagger fills the complex128 table with them if `keep`).
 template <typename R>
-hmc_status mdag_launch(hmc_ctx* c, const Geo& g, R dm, const V2<R>* p, V2<R>* out);
+hmc_status mdag_launch(hmc_ctx* c, const Geo& g, R dm, const V2<R>* p, V2<R>* out, const double* phi = nullptr,
+                       bool keep = false);
 template <typename R>
 hmc_status m_launch(hmc_ctx* c, const Geo& g, R dm, const V2<R>* u, const V2<R>* y, R sigma,
-                    V2<R>* out);
+                    V2<R>* out, const double* phi = nullptr);
 
 // out = (M M^dagger + sigma) in in one pass, u = M^dagger in kept on chip
 // (fused.cu); the tile shape is tuned on the first call per precision.

@@ -6,6 +6,7 @@
 
 #include "kernels.h"
 #include "operator.cuh"
+#include "phase.cuh"
 
 namespace hmc {
 
@@ -21,10 +22,47 @@ inline Phase<float> phase_of<float>(hmc_ctx* c) {
   return Phase<float>{(const float*)c->ws[WS_PHI32]};
 }
 
+// e^{i phi_k} straight from the field, for one application: the numbers of the
+// tables without the pass that builds them. E (may be NULL) keeps what was formed.
+template <typename R>
+struct FieldPhase;
+template <>
+struct FieldPhase<double> {
+  const double* __restrict__ phi;
+  PhaseTable tab;
+  double2* E;
+  __device__ __forceinline__ Cx<double> operator()(int k) const {
+    const double2 e = phase_of_field(tab, phi[k]);
+    if (E != nullptr) E[k] = e;
+    return Cx<double>{e.x, e.y};
+  }
+};
+template <>
+struct FieldPhase<float> {
+  const double* __restrict__ phi;
+  __device__ __forceinline__ Cx<float> operator()(int k) const {
+    const float x = field_to_f32(phi[k]);
+    return Phase<float>{&x}(0);
+  }
+};
+template <typename R>
+inline FieldPhase<R> field_phase(hmc_ctx* c, const double* phi, bool keep);
+template <>
+inline FieldPhase<double> field_phase<double>(hmc_ctx* c, const double* phi, bool keep) {
+  return FieldPhase<double>{phi, PhaseTable{c->phase_tab}, keep ? (double2*)c->ws[WS_E] : nullptr};
+}
+template <>
+inline FieldPhase<float> field_phase<float>(hmc_ctx*, const double* phi, bool) {
+  return FieldPhase<float>{phi};
+}
+
 // Launch with the programmatic-serialization attribute (see pdl_wait): the blocks
-// of a kernel are placed while the last ones of the kernel before it still run, and
-// wait there, which hides the launch (51x51x64 phases and M^dagger 22.5 -> 18.7 us;
-// a trajectory at 12x12x32, some 2,300 short kernels, 57.4 -> 53.2 ms).
+// of a kernel are placed when those of the kernel before it have ended, without
+// waiting for its memory to be flushed, which hides most of the launch (phases and
+// M^dagger at 51x51x64 22.5 -> 18 us; a trajectory at 12x12x32, some 2,300 short
+// kernels, 57.4 -> 51.5 ms). The kernels of the FP64 path don't trigger earlier:
+// placed among running blocks, those of a grid below one wave crowd on some SMs
+// (M^dagger at 51x51x64 7.4 us, without 6.45; the dots of 102x102x64 102 -> 150).
 // Ordinary launches are those that have no kernel before them in a graph: the first
 // of a capture, and any while somebody else captures the stream.
 template <typename... KA, typename... A>

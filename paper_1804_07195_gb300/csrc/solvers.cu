@@ -476,11 +476,11 @@ template hmc_status cg_core<double>(hmc_ctx*, double, double, const double2*, do
 template hmc_status cg_core<float>(hmc_ctx*, double, double, const float2*, float2*, bool, double,
                                    int, int, bool, SolveStats*);
 
-hmc_status apply_A64(hmc_ctx* c, double ms, double sigma, const double2* in, double2* out) {
+hmc_status apply_A64(hmc_ctx* c, double ms, double sigma, const double2* in, double2* out, const double* phi) {
   double2* u;
   HMC_TRY(ws_get(c, WS_U64, sizeof(double2) * (size_t)c->geo.N, (void**)&u));
   const double dm = c->delta * ms;
-  HMC_TRY(mdag_launch<double>(c, c->geo, dm, in, u));
+  HMC_TRY(mdag_launch<double>(c, c->geo, dm, in, u, phi, true));
   return m_launch<double>(c, c->geo, dm, u, sigma != 0.0 ? in : nullptr, sigma, out);
 }
 

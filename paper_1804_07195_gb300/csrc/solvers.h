@@ -37,7 +37,8 @@ hmc_status solve_opts(hmc_ctx* c, double ms, double sigma, const double2* b, dou
                       const hmc_solver_opts* opts, SolveStats* st);
 
 // out = (M_ms M_ms^dagger + sigma) in, FP64, using the context's U64 slot.
-hmc_status apply_A64(hmc_ctx* c, double ms, double sigma, const double2* in, double2* out);
+hmc_status apply_A64(hmc_ctx* c, double ms, double sigma, const double2* in, double2* out,
+                     const double* phi = nullptr);
 
 void add_stats(hmc_solve_info* info, const SolveStats& s);
 hmc_solver_opts default_opts();
