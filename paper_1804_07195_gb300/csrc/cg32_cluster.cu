@@ -70,6 +70,8 @@ static bool plan_cluster(const hmc_ctx* c, const Geo& g, int cs, TilePlan* out) 
   for (int tj = 1; tj <= cs; tj *= 2) {
     const int J = (g.m + tj - 1) / tj, T0 = (g.nt + cs / tj - 1) / (cs / tj);
     for (const int* inst = tile_slices32(cw); *inst; ++inst) {
+      // x out of registers: only the longest columns, it streams through L2 here
+      if (*inst > kXInMemory && *inst != (cw == 1 ? 8 : 4) + kXInMemory) continue;
       const int S = tile_slices(*inst);
       TilePlan p;
       p.cw = cw;

@@ -22,7 +22,7 @@ __global__ void __launch_bounds__(tile_max_threads<float, 2, S>(), 1) k_cg32_res
 }
 
 const int* tile_slices32(int cw) {
-  static const int one[] = {1, 2, 4, 8, 8 + kXInMemory, 0}, two[] = {1, 2, 4, 4 + kXInMemory, 0};
+  static const int one[] = {1, 2, 4, 4 + kXInMemory, 8, 8 + kXInMemory, 0}, two[] = {1, 2, 2 + kXInMemory, 4, 4 + kXInMemory, 0};
   return cw == 2 ? two : one;
 }
 
@@ -31,12 +31,14 @@ int max_threads32(int cw, int S) {
       case 1: return tile_max_threads<float, 1, 1>();
       case 2: return tile_max_threads<float, 1, 2>();
       case 4: return tile_max_threads<float, 1, 4>();
+      case 4 + kXInMemory: return tile_max_threads<float, 1, 4 + kXInMemory>();
       case 8: return tile_max_threads<float, 1, 8>();
       case 8 + kXInMemory: return tile_max_threads<float, 1, 8 + kXInMemory>();
     }
   switch (S) {
     case 1: return tile_max_threads<float, 2, 1>();
     case 2: return tile_max_threads<float, 2, 2>();
+    case 2 + kXInMemory: return tile_max_threads<float, 2, 2 + kXInMemory>();
     case 4: return tile_max_threads<float, 2, 4>();
     case 4 + kXInMemory: return tile_max_threads<float, 2, 4 + kXInMemory>();
   }
@@ -81,9 +83,9 @@ bool tile_plan_grid(const hmc_ctx* c, const Geo& g, int cw, int real, const int*
         p.smem = p.tab + table;
         // the work of the largest tile: its cells, the padding it exchanges (about
         // a third of a cell's work each), a little for every slice of a column
-        // (fewer, longer columns overlap less), and x streamed from L2
+        // (fewer, longer columns overlap less)
         const int Tmax = std::min(p.T, g.nt);
-        const double cost = (double)J * Tmax * nq + 0.7 * (J + Tmax) * nq + 8.0 * tile_slices(*S) + (*S >= kXInMemory ? 300.0 : 0.0);
+        const double cost = (double)J * Tmax * nq + 0.7 * (J + Tmax) * nq + 8.0 * tile_slices(*S);
         if (!found || cost < best) {
           found = true;
           best = cost;
@@ -117,12 +119,14 @@ static const void* grid_kernel32(int cw, int S) {
       case 1: return (const void*)k_cg32_resident<1>;
       case 2: return (const void*)k_cg32_resident<2>;
       case 4: return (const void*)k_cg32_resident<4>;
+      case 4 + kXInMemory: return (const void*)k_cg32_resident<4 + kXInMemory>;
       case 8: return (const void*)k_cg32_resident<8>;
       case 8 + kXInMemory: return (const void*)k_cg32_resident<8 + kXInMemory>;
     }
   switch (S) {
     case 1: return (const void*)k_cg32_resident2<1>;
     case 2: return (const void*)k_cg32_resident2<2>;
+    case 2 + kXInMemory: return (const void*)k_cg32_resident2<2 + kXInMemory>;
     case 4: return (const void*)k_cg32_resident2<4>;
     case 4 + kXInMemory: return (const void*)k_cg32_resident2<4 + kXInMemory>;
   }

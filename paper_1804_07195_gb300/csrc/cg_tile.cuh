@@ -49,8 +49,12 @@
 // The two exchanges take about 2 us each (arrival and poll of one L2 word 1.4,
 // the gather or the edges 0.5), whatever the lattice. The rest is, at
 // 102x102x64, shared memory (4.3 us of wavefronts), instruction issue (4.1) and
-// L2 (x streamed, phi twice, edges: 2.4 us at 64 B a cycle and SM), which the
-// phases overlap only in part. Tried and not kept: every block polling every
+// L2 (phi twice, edges), which the phases overlap only in part. x of the columns
+// of four slices and more lives in tensor memory: read and written there by the
+// lane that owns it, 8 columns a slice, instead of streamed through L2 every
+// iteration (102x102x64 14.0 -> 12.0 us, 97x101x63 16.0 -> 14.9), and the registers
+// it leaves free allow blocks of more threads with fewer slices each (80x80x64 9.85
+// -> 8.7, 85x85x64 14.7 -> 11.2). Tried and not kept: every block polling every
 // block's packet (one trip less, but the polls of 18,000 packet reads delay
 // the writes: 8.5 to 10.7 us at 36x36x64); x held in registers at 102x102x64
 // (7 slices a column, 384 threads: 14.6 us, too few warps; but 90x90x64, where 480
@@ -295,6 +299,55 @@ __device__ __forceinline__ void red_add_relaxed(unsigned* p, unsigned x) {
   asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(x) : "memory");
 }
 
+// ---------------------------------------------------------------------------
+// Tensor memory as a store of x: a lane's 32-bit columns are its own (warp w of
+// the block reaches lanes 32 (w mod 4) ..; the warps w, w + 4, .. take different
+// columns). Every instruction is for the whole warp.
+__device__ __forceinline__ void tmem_alloc(unsigned* where, int columns) {
+  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n\t"
+               "tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::"r"(
+                   (unsigned)__cvta_generic_to_shared(where)), "r"(columns) : "memory");
+}
+__device__ __forceinline__ void tmem_free(unsigned at, int columns) {
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(at), "r"(columns) : "memory");
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// 8 and 4 columns: a slice's cells A and B
+__device__ __forceinline__ void tmem_ld(unsigned at, uint4& a, uint4& b) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+               : "r"(at) : "memory");
+}
+__device__ __forceinline__ void tmem_st(unsigned at, uint4 a, uint4 b) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(at), "r"(a.x),
+               "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w) : "memory");
+}
+__device__ __forceinline__ void tmem_ld(unsigned at, uint2& a, uint2& b) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(a.x), "=r"(a.y), "=r"(b.x), "=r"(b.y) : "r"(at) : "memory");
+}
+__device__ __forceinline__ void tmem_st(unsigned at, uint2 a, uint2 b) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(a.x), "r"(a.y),
+               "r"(b.x), "r"(b.y) : "memory");
+}
+// the bits of a column's value
+__device__ __forceinline__ uint2 bits(float2 v) { return make_uint2(__float_as_uint(v.x), __float_as_uint(v.y)); }
+__device__ __forceinline__ uint4 bits(ulonglong2 v) {
+  return make_uint4((unsigned)v.x, (unsigned)(v.x >> 32), (unsigned)v.y, (unsigned)(v.y >> 32));
+}
+__device__ __forceinline__ uint4 bits(double2 v) {
+  return make_uint4((unsigned)__double2loint(v.x), (unsigned)__double2hiint(v.x), (unsigned)__double2loint(v.y),
+                    (unsigned)__double2hiint(v.y));
+}
+__device__ __forceinline__ void from_bits(uint2 b, float2& v) { v = make_float2(__uint_as_float(b.x), __uint_as_float(b.y)); }
+__device__ __forceinline__ void from_bits(uint4 b, ulonglong2& v) {
+  v = make_ulonglong2(b.x | (unsigned long long)b.y << 32, b.z | (unsigned long long)b.w << 32);
+}
+__device__ __forceinline__ void from_bits(uint4 b, double2& v) {
+  v = make_double2(__hiloint2double((int)b.y, (int)b.x), __hiloint2double((int)b.w, (int)b.z));
+}
+
 // Warp 0: the sum of all blocks' partials, in every lane.
 template <typename R>
 __device__ __forceinline__ typename Red<R>::T gather(const double* part, int G) {
@@ -382,7 +435,9 @@ __device__ __forceinline__ int fresh(int i) {
 }
 
 // A kernel instance is named by its slices per column S, plus kXInMemory where x
-// stays in memory and only passes through registers (the others hold r and x).
+// only passes through registers (the others hold r and x): kept in tensor memory,
+// which nothing else here needs, or by a cluster's blocks, which may share an SM
+// and could then wait for its columns on each other, in its own memory.
 constexpr int kXInMemory = 100;
 constexpr int tile_slices(int inst) { return inst % kXInMemory; }
 // Largest block of an instance, from the registers it needs (r and x: 8 per slice
@@ -553,14 +608,29 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
   // exchanges so far; CL = false: its parity is the arrival word's top bit
   unsigned ep = CL ? 0u : *(const volatile unsigned*)gs.word >> 31;
 
-  // r and x of the thread's cells (A, B). With many slices per column x stays
-  // in memory (in the lanes' layout while the solve runs) and passes through
-  // registers in P, two slices in flight.
-  constexpr bool XREG = INST < kXInMemory;
+  // r and x of the thread's cells (A, B). With many slices per column x is kept
+  // elsewhere in the lanes' layout and passes through registers in P, two slices
+  // in flight: in tensor memory (CL = false: one block an SM), or in its own memory.
+  constexpr bool XREG = INST < kXInMemory, XTM = !XREG && !CL;
+  constexpr int XC = VB / 2;  // columns of a slice's cells A and B
+  using B = decltype(bits(V{}));
+  __shared__ unsigned s_tmem;
+  static_assert(!XTM || XC * S * ((tile_max_threads<R, CW, INST>() / 32 + 3) / 4) <= 512, "tensor memory of an SM");
+  const int xcols = XC * S * ((nwarps + 3) / 4);
+  const int xalloc = xcols <= 32 ? 32 : xcols <= 64 ? 64 : xcols <= 128 ? 128 : xcols <= 256 ? 256 : 512;
+  unsigned xt = 0;
+  if constexpr (XTM) {
+    if (warp == 0) tmem_alloc(&s_tmem, xalloc);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    xt = s_tmem + ((unsigned)(warp & 3) << 21) + (unsigned)(warp >> 2) * (XC * S);
+  }
   C ra[S], rb[S];
   C xa[XREG ? S : 2], xb[XREG ? S : 2];
 #pragma unroll
-  for (int s = 0; s < S; ++s)
+  for (int s = 0; s < S; ++s) {
+    B ba{}, bb{};
     if (s < ns) {
       const int k = k_first + s * Vq;
       ra[s] = unpack(swizzle(rg[k]));
@@ -568,15 +638,59 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
       if (XREG) {
         xa[XREG ? s : 0] = unpack(swizzle(xg[k]));
         xb[XREG ? s : 0] = unpack(swizzle(xg[Hq + k]));
+      } else if (XTM) {
+        ba = bits(swizzle(xg[k]));
+        bb = bits(swizzle(xg[Hq + k]));
       } else {
         xg[k] = swizzle(xg[k]);
         xg[Hq + k] = swizzle(xg[Hq + k]);
       }
     }
+    if constexpr (XTM) {
+      __syncwarp();
+      tmem_st(xt + s * XC, ba, bb);
+    }
+  }
   // x += f p (p of the last iteration) and, if asked, p = r + fb p, slice by slice
   auto x_and_p = [&](R f, R fb, bool newp) {
     const L lf = LN::set(f), lb = LN::set(fb);
     int o = fresh(o_first), k = fresh(k_first);
+    auto slice = [&](int s, C& x0, C& x1) {
+      const C pa = lds(PA + o), pb = lds(PB + o + oNJ + oq);
+      x0 = vaxpy(lf, pa, x0);
+      x1 = vaxpy(lf, pb, x1);
+      if (newp) {
+        sts(PA + o, vaxpy(lb, pa, ra[s]));
+        sts(PB + o + oNJ + oq, vaxpy(lb, pb, rb[s]));
+      }
+    };
+    if constexpr (XTM) {
+      static_assert(S % 2 == 0, "slices go in pairs");
+      tmem_wait_st();  // the last iteration's
+#pragma unroll
+      for (int s = 0; s < S; s += 2) {
+        B b0[2], b1[2];
+        __syncwarp();
+        tmem_ld(xt + s * XC, b0[0], b1[0]);
+        tmem_ld(xt + (s + 1) * XC, b0[1], b1[1]);
+        tmem_wait_ld();
+#pragma unroll
+        for (int e = 0; e < 2; ++e, o += oNJ)
+          if (s + e < ns) {
+            V v0, v1;
+            from_bits(b0[e], v0);
+            from_bits(b1[e], v1);
+            C x0 = unpack(v0), x1 = unpack(v1);
+            slice(s + e, x0, x1);
+            b0[e] = bits(pack(x0));
+            b1[e] = bits(pack(x1));
+          }
+        __syncwarp();
+        tmem_st(xt + s * XC, b0[0], b1[0]);
+        tmem_st(xt + (s + 1) * XC, b0[1], b1[1]);
+      }
+      return;
+    }
     if (!XREG) {
 #pragma unroll
       for (int s = 0; s < 2; ++s)
@@ -589,22 +703,14 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
     for (int s = 0; s < S; ++s, o += oNJ, k += Vq)
       if (s < ns) {
         const int e = XREG ? s : (s & 1);
-        const C pa = lds(PA + o), pb = lds(PB + o + oNJ + oq);
-        const C na = vaxpy(lf, pa, xa[e]), nb = vaxpy(lf, pb, xb[e]);
-        if (XREG) {
-          xa[e] = na;
-          xb[e] = nb;
-        } else {
-          xg[k] = pack(na);
-          xg[Hq + k] = pack(nb);
+        slice(s, xa[e], xb[e]);
+        if (!XREG) {
+          xg[k] = pack(xa[e]);
+          xg[Hq + k] = pack(xb[e]);
           if (s + 2 < S && s + 2 < ns) {
             xa[e] = unpack(xg[k + 2 * Vq]);
             xb[e] = unpack(xg[Hq + k + 2 * Vq]);
           }
-        }
-        if (newp) {
-          sts(PA + o, vaxpy(lb, pa, ra[s]));
-          sts(PB + o + oNJ + oq, vaxpy(lb, pb, rb[s]));
         }
       }
   };
@@ -867,18 +973,38 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
     ++iter;
     first = false;
   }
+  if constexpr (XTM) tmem_wait_st();
 #pragma unroll
-  for (int s = 0; s < S; ++s)
+  for (int s = 0; s < S; ++s) {
+    B ba{}, bb{};
+    if constexpr (XTM) {
+      __syncwarp();
+      tmem_ld(xt + s * XC, ba, bb);
+      tmem_wait_ld();
+    }
     if (s < ns) {
       const int k = k_first + s * Vq;
       if (XREG) {
         xg[k] = swizzle(pack(xa[XREG ? s : 0]));
         xg[Hq + k] = swizzle(pack(xb[XREG ? s : 0]));
+      } else if (XTM) {
+        V v0, v1;
+        from_bits(ba, v0);
+        from_bits(bb, v1);
+        xg[k] = swizzle(v0);
+        xg[Hq + k] = swizzle(v1);
       } else {
         xg[k] = swizzle(xg[k]);
         xg[Hq + k] = swizzle(xg[Hq + k]);
       }
     }
+  }
+  if constexpr (XTM) {
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (warp == 0) tmem_free(s_tmem, xalloc);
+  }
   if (tile == 0 && tid == 0) {
     CGScal* sc = ts.sc;
     sc->rr = rr;

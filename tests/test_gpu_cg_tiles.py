@@ -104,3 +104,23 @@ def test_fp64_tiles(shape):
         assert rel_max(host(x), x0 + ref0.x) <= 1e-13
         assert ctx.profile_read()["cg_resident_f64"]["launches"] >= 1
         assert ctx.check_guards() == 0
+
+
+@pytest.mark.parametrize("shape", [(80, 79, 62), (85, 83, 61), (97, 99, 64), (100, 101, 63)])
+def test_x_in_tensor_memory(shape):
+    """x kept in tensor memory: two and four slices of cell pairs, four and
+    eight of single cells, ragged tiles; the sum over several iterations, so
+    that every one of them has been read back and stored."""
+    need_gpu()
+    w = W.small(*shape, seed=2500 + sum(shape))
+    ol = OLat.from_params(w.lat)
+    b32 = w.b.astype(np.complex64)
+    ref = osv.cg(lambda v: of.apply_MMdag(ol, w.phi, 0.4, v, 0.3), b32.astype(np.complex128), tol=1e-30, maxit=4)
+    with ctx_for(w.lat) as ctx:
+        ctx.set_cg_variant(7)
+        x, info = ctx.solve_spcg(dev(w.phi), 0.4, dev(b32), sigma=0.3, tol=1e-30, maxit=4, allow_fail=True)
+        assert ctx.profile_read()["cg_resident_f32"]["launches"] >= 1
+        assert ctx.check_guards() == 0
+    assert info["iters"] == 4
+    # the bound of the other tests, 2e-5 an iteration
+    assert rel_max(host(x).astype(np.complex128), ref.x) <= 8e-5
