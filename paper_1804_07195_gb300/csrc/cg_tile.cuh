@@ -44,8 +44,8 @@
 // What bounds an FP32 iteration of a cooperative launch (us, 2070 MHz; in
 // brackets the design before it, which read r, x and phi from L2 row by row in
 // both halves and published p as well):
-//   6x6x16 6.4 (9.0)   12x12x32 6.8 (8.6)   36x36x64 5.6 (7.5)
-//   51x51x64 7.55 (11.6)   72x72x64 7.95 (11.8)   90x90x64 11.0   102x102x64 14.0 (16.2)
+//   6x6x16 6.4 (9.0)   12x12x32 6.8 (8.6)   36x36x64 5.5 (7.5)
+//   51x51x64 7.15 (11.6)   72x72x64 7.9 (11.8)   90x90x64 10.2   102x102x64 11.5 (16.2)
 // The two exchanges take about 2 us each (arrival and poll of one L2 word 1.4,
 // the gather or the edges 0.5), whatever the lattice. The rest is, at
 // 102x102x64, shared memory (4.3 us of wavefronts), instruction issue (4.1) and
@@ -584,6 +584,49 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
         (d.y >> 31) != 0u);
     }
   };
+  // The padding of u from the neighbours' edges in src (u, or r if `of_r`), read
+  // from L2. A thread has up to four columns, and a trip to L2 for each takes 0.6 us:
+  // 16-byte columns go by cp.async, all in flight and through no register; 8-byte
+  // ones (whose cp.async may hit a stale L1 line) FB at a time in registers. (102x102x64
+  // 12.0 -> 11.5 us an iteration, 51x51x64 7.55 -> 7.15, 75x75x64 11.8 -> 10.5; FP64
+  // 51x51x64 31.0 -> 28.5.)
+  auto fetch_padding = [&](const V* src, bool of_r) {
+    auto from = [&](unsigned y) {
+      const unsigned st = of_r ? 0u : (y >> 29) & 3u;
+      return src + (int)(y & 0x1fffffffu) + (st == 1u ? -Hq : st == 2u ? Hq : 0);
+    };
+    if constexpr (VB == 16) {
+      const unsigned base = (unsigned)__cvta_generic_to_shared(sm);
+      for (int e = e_first; e < e_end; e += e_step) {
+        const uint2 d = tab[e];
+        if (d.x != 0xffffffffu)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(base + (d.x >> 16) * VB), "l"(from(d.y)) : "memory");
+      }
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      if (wlo || whi)
+        for (int e = e_first; e < e_end; e += e_step) {
+          const uint2 d = tab[e];
+          if (d.x != 0xffffffffu && (d.y >> 31) != 0u) {
+            const int ou = (int)(d.x >> 16) * VB;
+            sts(ou, vneg_if(lds(ou), true));
+          }
+        }
+    } else {
+      constexpr int FB = INST == 4 ? 2 : 3;  // (69x69x64, four slices: 10.05 us with 2, 10.9 with 3)
+      for (int e = e_first; e < e_end; e += FB * e_step) {
+        uint2 d[FB];
+        V v[FB];
+#pragma unroll
+        for (int i = 0; i < FB; ++i) {
+          d[i] = e + i * e_step < e_end ? tab[e + i * e_step] : make_uint2(0xffffffffu, 0u);
+          if (d[i].x != 0xffffffffu) v[i] = __ldcg(from(d[i].y));
+        }
+#pragma unroll
+        for (int i = 0; i < FB; ++i)
+          if (d[i].x != 0xffffffffu) sts((int)(d[i].x >> 16) * VB, vneg_if(unpack(v[i]), (d[i].y >> 31) != 0u));
+      }
+    }
+  };
   unsigned rem_dn = 0, rem_up = 0, rem_bf = 0, rem_af = 0;  // CL: the neighbours' shared memory
   int JtD = 0, TtP = 0;  // CL: rows of the tile below, slices of the tile before
   if constexpr (CL) {
@@ -882,12 +925,7 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
     }
     T tot;
     bool ok = exchange(total(acc) + (sigma != R(0) ? sigma * total(accp) : R(0)),
-                       [&] {
-                         for_padding([&](int, int, int ou, int, int ku, bool neg) {
-                           sts(ou, vneg_if(unpack(__ldcg(Ug + ku)), neg));
-                         });
-                       },
-                       &tot);
+                       [&] { fetch_padding(Ug, false); }, &tot);
     // phases of the first slice of M
     if (ns > 0) {
       fa = PH::load(ph, k_first);
@@ -957,12 +995,7 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
     // next exchange has refilled it (the block's barrier in `exchange` orders
     // the reads of u above before these writes)
     ok = exchange(total(accr),
-                  [&] {
-                    for_padding([&](int, int, int ou, int kp, int, bool neg) {
-                      sts(ou, vneg_if(unpack(__ldcg(rg + kp)), neg));
-                    });
-                  },
-                  &tot);
+                  [&] { fetch_padding(rg, true); }, &tot);
     if (CL || tid == 0) {
       rr_prev = rr;
       if (ok)
