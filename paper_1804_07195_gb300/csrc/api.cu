@@ -391,8 +391,9 @@ hmc_status hmc_create(hmc_ctx** out, const hmc_lattice* lat, void* stream) {
   if ((e = cudaMalloc(&c->partials, sizeof(double) * kMaxRed * c->nsm * 2 * kOneItemBlocksPerSM)) != cudaSuccess)
     return bail(e);
   if ((e = cudaMallocHost(&c->sc_host, sizeof(CGScal) * 4)) != cudaSuccess) return bail(e);
-  if ((e = cudaMalloc(&c->dscal, sizeof(double) * 128)) != cudaSuccess) return bail(e);
-  if ((e = cudaMallocHost(&c->dscal_host, sizeof(double) * 128)) != cudaSuccess) return bail(e);
+  if ((e = cudaMalloc(&c->dscal, sizeof(double) * kDscal)) != cudaSuccess) return bail(e);
+  if ((e = cudaMallocHost(&c->dscal_host, sizeof(double) * (kDscal + 1))) != cudaSuccess) return bail(e);
+  c->dscal_host[kDscal] = 0.0;
   *out = c;
   return HMC_OK;
 }

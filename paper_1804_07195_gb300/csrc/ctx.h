@@ -138,6 +138,7 @@ struct ProfileState {
 
 }  // namespace hmc
 
+constexpr int kDscal = 128;
 struct hmc_ctx {
   int device = 0;
   int nsm = 0;
@@ -161,8 +162,9 @@ struct hmc_ctx {
   hmc::CGScal* sc = nullptr;       // device CG state (two: FP64 outer, FP32 inner)
   hmc::GridBar* gbar = nullptr;    // grid barrier of the persistent FP32 CG kernel
   hmc::CGScal* sc_host = nullptr;  // pinned mirror
-  double* dscal = nullptr;         // device scalar results (64 doubles)
-  double* dscal_host = nullptr;    // pinned mirror
+  double* dscal = nullptr;         // device scalar results (kDscal doubles)
+  double* dscal_host = nullptr;    // pinned mirror, then the word that read_back watches
+  unsigned read_seq = 0;
   int max_grid = 0;
   // resident-tile CG: the memory of its exchanges (stale: to be cleared before
   // the next launch), and the plans of this lattice ([cells per column - 1])

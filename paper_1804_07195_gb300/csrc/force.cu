@@ -75,9 +75,7 @@ hmc_status term_action(hmc_ctx* c, int nmass, const double* masses, const double
   HMC_TRY(mdag_launch<double>(c, c->geo, c->delta * lower_mass(masses, i), eta, xi));
   HMC_TRY(redot_launch(c, c->geo.N, src, eta, c->dscal + 100, c->tickets));
   HMC_TRY(norm2_launch(c, c->geo.N, xi, c->dscal + 101, c->tickets));
-  HMC_CUDA(c, cudaMemcpyAsync(c->dscal_host + 100, c->dscal + 100, 2 * sizeof(double),
-                              cudaMemcpyDeviceToHost, c->stream));
-  HMC_CUDA(c, cudaStreamSynchronize(c->stream));
+  HMC_TRY(read_back(c, c->dscal + 100, c->dscal_host + 100, 2 * sizeof(double)));
   *S_host = 2.0 * c->dscal_host[100] - c->dscal_host[101];
   return HMC_OK;
 }
@@ -219,8 +217,7 @@ hmc_status hmc_action(hmc_ctx* c, const double* phi, int nmass, const double* ma
   if (flags & HMC_GAUSSIAN) {
     if (!ph) return fail(c, HMC_ERR_INVALID, "the Gaussian term needs phi");
     HMC_TRY(half_sq_launch(c, c->geo.N, ph, 1.0 / (c->delta * c->lat.U), nullptr, c->dscal + 50, c->tickets));
-    HMC_CUDA(c, cudaMemcpyAsync(c->dscal_host + 50, c->dscal + 50, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    HMC_CUDA(c, cudaStreamSynchronize(c->stream));
+    HMC_TRY(read_back(c, c->dscal + 50, c->dscal_host + 50, sizeof(double)));
     total += c->dscal_host[50];
   }
   if (fermion) {

@@ -5,6 +5,7 @@
 // steps of Algorithm A.1 (Appendix A), the force of Eqs. p_dot, f_chi_i and
 // def_xi_i, the energies of Eq. hamiltonian.
 #include <algorithm>
+#include <chrono>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -1134,6 +1135,37 @@ hmc_status init0_launch(hmc_ctx* c, int N, const V2<R>* b, V2<R>* x, V2<R>* r, V
 INST(float)
 INST(double)
 #undef INST
+
+// Copies words to pinned host memory and then says so there.
+__global__ void k_publish(const unsigned long long* src, unsigned long long* dst, int words, unsigned* flag,
+                          unsigned seq) {
+  pdl_wait();
+  for (int k = threadIdx.x; k < words; k += blockDim.x) dst[k] = src[k];
+  __threadfence_system();
+  __syncthreads();
+  if (threadIdx.x == 0) asm volatile("st.release.sys.global.u32 [%0], %1;" ::"l"(flag), "r"(seq) : "memory");
+}
+
+// A solve on a small lattice waits for a scalar every few tens of us: a copy and a
+// stream synchronisation cost 5.4 us more each than a kernel behind
+// the others that writes to the host, which watches for it (12x12x32: trajectory 52.0
+// -> 48.5 ms, action 9.47 -> 8.99). A wait beyond 1 ms
+// is left to the stream's own synchronisation, and so is every error.
+hmc_status read_back(hmc_ctx* c, const void* dev, void* host, size_t bytes) {
+  static_assert(sizeof(CGScal) % 8 == 0, "whole words");
+  unsigned* const flag = (unsigned*)(c->dscal_host + kDscal);
+  const unsigned seq = ++c->read_seq;
+  launch_pdl(c, k_publish, dim3(1), 64, c->stream, (const unsigned long long*)dev, (unsigned long long*)host,
+             (int)(bytes / 8), flag, seq);
+  HMC_CUDA(c, cudaGetLastError());
+  const auto t0 = std::chrono::steady_clock::now();
+  for (unsigned spin = 1;; ++spin) {
+    if (__atomic_load_n(flag, __ATOMIC_ACQUIRE) == seq) return HMC_OK;
+    if (spin % 256 == 0 && std::chrono::steady_clock::now() - t0 > std::chrono::milliseconds(1)) break;
+  }
+  HMC_CUDA(c, cudaStreamSynchronize(c->stream));
+  return HMC_OK;
+}
 
 // Condition of the device-side CG loop: continue while the solve runs and the
 // trip count is below its bound (trips[1], so the loop ends even if the done

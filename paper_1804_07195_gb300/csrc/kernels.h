@@ -11,6 +11,10 @@ namespace hmc {
 template <typename R>
 using V2 = typename Vec2<R>::type;
 
+// Waits for the stream's work so far and copies `bytes` (a multiple of 8) of its
+// results to pinned host memory.
+hmc_status read_back(hmc_ctx* c, const void* dev, void* host, size_t bytes);
+
 // Phase tables: E = e^{i phi} (complex128; with table64) and phi rounded to float.
 hmc_status k_phase_launch(hmc_ctx* c, const double* phi, bool table64);
 

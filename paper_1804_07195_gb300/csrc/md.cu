@@ -170,9 +170,7 @@ extern "C" hmc_status hmc_md_trajectory(hmc_ctx* c, double* phi, double* pi, int
   HMC_TRY(half_sq_launch(c, (int)N, phi, inv_dU, pi, c->dscal + 54, c->tickets));
   for (int i = 0; i <= nmass; ++i)
     HMC_TRY(norm2_launch(c, (int)N, (const double2*)rho[i], c->dscal + 56 + i, c->tickets));
-  HMC_CUDA(c, cudaMemcpyAsync(c->dscal_host + 54, c->dscal + 54, sizeof(double) * (2 + nmass + 1),
-                              cudaMemcpyDeviceToHost, c->stream));
-  HMC_CUDA(c, cudaStreamSynchronize(c->stream));
+  HMC_TRY(read_back(c, c->dscal + 54, c->dscal_host + 54, sizeof(double) * (2 + nmass + 1)));
   double h0 = c->dscal_host[54] + c->dscal_host[55];
   for (int i = 0; i <= nmass; ++i) h0 += c->dscal_host[56 + i];
 
@@ -191,9 +189,7 @@ extern "C" hmc_status hmc_md_trajectory(hmc_ctx* c, double* phi, double* pi, int
     h1 += Si;
   }
   HMC_TRY(half_sq_launch(c, (int)N, phi, inv_dU, pi, c->dscal + 54, c->tickets));
-  HMC_CUDA(c, cudaMemcpyAsync(c->dscal_host + 54, c->dscal + 54, sizeof(double) * 2,
-                              cudaMemcpyDeviceToHost, c->stream));
-  HMC_CUDA(c, cudaStreamSynchronize(c->stream));
+  HMC_TRY(read_back(c, c->dscal + 54, c->dscal_host + 54, sizeof(double) * 2));
   h1 += c->dscal_host[54] + c->dscal_host[55];
   *H0 = h0;
   *H1 = h1;

@@ -330,8 +330,7 @@ hmc_status cg_core(hmc_ctx* c, double ms, double sigma, const V2<R>* b, V2<R>* x
         HMC_TRY(cg32_resident_launch(c, g, (float2*)x, (float2*)r, (float2*)u, sc));
       else
         HMC_TRY(cg32_persist_launch(c, g, (float2*)x, (float2*)r, (float2*)p, (float2*)q, (float2*)u, sc));
-      HMC_CUDA(c, cudaMemcpyAsync(sch, sc, sizeof(CGScal), cudaMemcpyDeviceToHost, c->stream));
-      HMC_CUDA(c, cudaStreamSynchronize(c->stream));
+      HMC_TRY(read_back(c, sc, sch, sizeof(CGScal)));
       // the algorithmic bytes of one FP32 CG iteration per site, whatever the
       // design keeps on chip: the operator with its dot (p and phi read, A p
       // written: 20 B, here rounded with the dot to 24 B), x and r updated
@@ -343,8 +342,7 @@ hmc_status cg_core(hmc_ctx* c, double ms, double sigma, const V2<R>* b, V2<R>* x
     if (tiles64) {
       persistent = true;
       HMC_TRY(cg64_resident_launch(c, g, (double2*)x, (double2*)r, (double2*)u, sc));
-      HMC_CUDA(c, cudaMemcpyAsync(sch, sc, sizeof(CGScal), cudaMemcpyDeviceToHost, c->stream));
-      HMC_CUDA(c, cudaStreamSynchronize(c->stream));
+      HMC_TRY(read_back(c, sc, sch, sizeof(CGScal)));
       c->prof.bytes[K_CG_RES64] += 208.0 * g.N * sch->iter;
     }
   }
@@ -438,8 +436,7 @@ hmc_status cg_core(hmc_ctx* c, double ms, double sigma, const V2<R>* b, V2<R>* x
       }
     }
     launched += (long long)per_check * kChunk;
-    HMC_CUDA(c, cudaMemcpyAsync(sch, sc, sizeof(CGScal), cudaMemcpyDeviceToHost, c->stream));
-    HMC_CUDA(c, cudaStreamSynchronize(c->stream));
+    HMC_TRY(read_back(c, sc, sch, sizeof(CGScal)));
     if (sch->done != CG_RUNNING) break;
     if (launched > (long long)maxit + 2 * kChunk) break;  // cannot happen: the device stops at maxit
     // with per-launch timing on, check after every chunk so that few launches
@@ -457,9 +454,7 @@ hmc_status cg_core(hmc_ctx* c, double ms, double sigma, const V2<R>* b, V2<R>* x
   if (want_true_res) {
     HMC_TRY(mdag_launch<R>(c, g, dm, x, u));
     HMC_TRY(resid_launch<R>(c, g, dm, u, x, b, sigma, r, nullptr, nullptr, 0.0, 0, c->dscal, tk, ddm));
-    HMC_CUDA(c, cudaMemcpyAsync(c->dscal_host, c->dscal, 2 * sizeof(double),
-                                cudaMemcpyDeviceToHost, c->stream));
-    HMC_CUDA(c, cudaStreamSynchronize(c->stream));
+    HMC_TRY(read_back(c, c->dscal, c->dscal_host, 2 * sizeof(double)));
     const double rr = c->dscal_host[0], bb = c->dscal_host[1];
     st->true_rel = bb > 0 ? std::sqrt(rr / bb) : 0.0;
     if (sizeof(R) == 8) st->applies64++; else st->applies32++;
@@ -584,8 +579,7 @@ hmc_status fgmres_core(hmc_ctx* c, double ms, double sigma, const double2* b, do
 
   // |b|
   HMC_TRY(norm2_launch(c, N, b, hdev + 40, tk));
-  HMC_CUDA(c, cudaMemcpyAsync(hhost + 40, hdev + 40, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  HMC_CUDA(c, cudaStreamSynchronize(c->stream));
+  HMC_TRY(read_back(c, hdev + 40, hhost + 40, sizeof(double)));
   const double bnorm = std::sqrt(hhost[40]);
   if (!std::isfinite(bnorm)) return fail(c, HMC_ERR_NAN, "FGMRES: right-hand side is not finite");
   if (bnorm == 0.0) {
@@ -601,8 +595,7 @@ hmc_status fgmres_core(hmc_ctx* c, double ms, double sigma, const double2* b, do
   auto true_residual = [&](double* err) -> hmc_status {
     HMC_TRY(mdag_launch<double>(c, g, dm, x, u));
     HMC_TRY(resid_launch<double>(c, g, dm, u, x, b, sigma, r, nullptr, nullptr, 0.0, 0, hdev + 40, tk));
-    HMC_CUDA(c, cudaMemcpyAsync(hhost + 40, hdev + 40, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    HMC_CUDA(c, cudaStreamSynchronize(c->stream));
+    HMC_TRY(read_back(c, hdev + 40, hhost + 40, 2 * sizeof(double)));
     st->applies64++;
     *err = std::sqrt(hhost[40]);
     return HMC_OK;
@@ -642,8 +635,7 @@ hmc_status fgmres_core(hmc_ctx* c, double ms, double sigma, const double2* b, do
       for (int i = 0; i <= j; ++i) V.v[i] = Vb + (size_t)i * N;
       HMC_TRY(mdot_launch(c, N, V, j + 1, w, hdev, tk));
       HMC_TRY(gsupd_launch(c, N, V, j + 1, hdev, w, hdev + 40, tk));
-      HMC_CUDA(c, cudaMemcpyAsync(hhost, hdev, 41 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-      HMC_CUDA(c, cudaStreamSynchronize(c->stream));
+      HMC_TRY(read_back(c, hdev, hhost, 41 * sizeof(double)));
       for (int i = 0; i <= j; ++i) H[i + j * ldh] = cd(hhost[2 * i], hhost[2 * i + 1]);
       wnorm = std::sqrt(hhost[40]);
       H[j + 1 + j * ldh] = wnorm;
@@ -719,8 +711,7 @@ hmc_status fcg_core(hmc_ctx* c, double ms, double sigma, const double2* b, doubl
   double* d = c->dscal;
   double* h = c->dscal_host;
   auto fetch = [&](int n) -> hmc_status {
-    HMC_CUDA(c, cudaMemcpyAsync(h + 80, d + 80, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    HMC_CUDA(c, cudaStreamSynchronize(c->stream));
+    HMC_TRY(read_back(c, d + 80, h + 80, n * sizeof(double)));
     return HMC_OK;
   };
   HMC_TRY(norm2_launch(c, N, b, d + 80, tk));
