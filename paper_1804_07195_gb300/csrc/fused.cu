@@ -119,6 +119,7 @@ __global__ void __launch_bounds__(fused_max_threads<R>()) k_mmdag_fused(Geo g, F
                                                                   const typename FusedPhase<R>::type::T* __restrict__ ph,
                                                                   R dm, R sigma, const V2<R>* __restrict__ p,
                                                                   V2<R>* __restrict__ out) {
+  pdl_wait();
   using PS = typename FusedPhase<R>::type;
   using PT = typename PS::T;
   constexpr int S = D + 2;  // the step's slot J = k mod S also gives k mod 2 and k mod 4
@@ -354,6 +355,7 @@ template <int D>
 __global__ void __launch_bounds__(kPairMaxThreads, 3) k_mmdag_fused_pairs(Geo g, FusedShape fs, const float2* __restrict__ ph,
                                                            float dm, float sigma, const float4* __restrict__ p,
                                                            float4* __restrict__ out) {
+  pdl_wait();
   constexpr int S = D + 2;
   static_assert(S % 2 == 0, "ring size");
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -628,12 +630,11 @@ static void fused_raw_launch(hmc_ctx* c, const Geo& g, const FusedShape& fs, R d
         pattr |= bit;
       }
       const float2* ph2 = (const float2*)c->ws[WS_PHI32];
-      if (fs.D == 2)
-        k_mmdag_fused_pairs<2><<<blocks, threads, smem, c->stream>>>(g, fs, ph2, dm, sigma, (const float4*)in,
-                                                                     (float4*)out);
-      else
-        k_mmdag_fused_pairs<6><<<blocks, threads, smem, c->stream>>>(g, fs, ph2, dm, sigma, (const float4*)in,
-                                                                     (float4*)out);
+      // (us back to back, with ordinary launches in brackets: 306x306x64 48.2 (49.2),
+      // 200x200x64 23.6 (26.7), 102x102x64 8.7 (10.3), 24x24x48 4.4 (6.1); with the next
+      // kernel's blocks let in early 47.1, 23.9, 10.3, and 150x150x64 17.7 against 14.7)
+      launch_pdl_smem(c, fs.D == 2 ? k_mmdag_fused_pairs<2> : k_mmdag_fused_pairs<6>, dim3(blocks), threads, smem,
+                      c->stream, g, fs, ph2, dm, sigma, (const float4*)in, (float4*)out);
       return;
     }
   }
@@ -643,11 +644,11 @@ static void fused_raw_launch(hmc_ctx* c, const Geo& g, const FusedShape& fs, R d
   else
     ph = (const double2*)c->ws[WS_E];
   if constexpr (sizeof(R) == 8) {
-    k_mmdag_fused<R, 2><<<blocks, threads, smem, c->stream>>>(g, fs, ph, dm, sigma, in, out);
+    launch_pdl_smem(c, k_mmdag_fused<R, 2>, dim3(blocks), threads, smem, c->stream, g, fs, ph, dm, sigma, in, out);
   } else if (fs.D == 2) {
-    k_mmdag_fused<R, 2><<<blocks, threads, smem, c->stream>>>(g, fs, ph, dm, sigma, in, out);
+    launch_pdl_smem(c, k_mmdag_fused<R, 2>, dim3(blocks), threads, smem, c->stream, g, fs, ph, dm, sigma, in, out);
   } else {
-    k_mmdag_fused<R, 6><<<blocks, threads, smem, c->stream>>>(g, fs, ph, dm, sigma, in, out);
+    launch_pdl_smem(c, k_mmdag_fused<R, 6>, dim3(blocks), threads, smem, c->stream, g, fs, ph, dm, sigma, in, out);
   }
 }
 
