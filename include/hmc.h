@@ -320,11 +320,14 @@ hmc_status hmc_md_trajectory_batched(hmc_ctx* ctx, int nchains, const hmc_chain*
  * arithmetic), whose kernel applies M M^dagger + sigma over tiles with
  * M^dagger r kept in shared memory as hmc_apply_MMdag's fused kernel does,
  * and updates x, r, p and the recurrences of w = A r and s = A p as the
- * slices arrive. The seventh runs the whole solve in one cooperative launch
- * in which each block keeps p and M^dagger p of its tile (all n cells of a
- * row, a few rows and time slices) in shared memory and exchanges the tile's
- * edges through memory between grid barriers (bounded waits, as for the
- * persistent kernel). variant: 0 = let the autotuner choose among all of
+ * slices arrive. The seventh runs the whole solve in one launch in which each
+ * block keeps p and M^dagger p of its tile (all n cells of a row, a few rows
+ * and time slices) in shared memory, r and x in registers (x of large tiles in
+ * tensor memory): a cooperative launch over all SMs, whose blocks exchange
+ * their tiles' edges through memory between grid barriers (bounded waits, as
+ * for the persistent kernel), or on lattices of up to about 100,000 sites one
+ * thread block cluster, which exchanges them through its shared memory.
+ * variant: 0 = let the autotuner choose among all of
  * them (default), 1 = grid-stride with one cell per thread, 2 = tiled only,
  * 3 = marching only, 4 = persistent, 5 = grid-stride with two cells per
  * thread, 6 = single-reduction, 7 = resident tiles (2 to 7 fall back to
