@@ -46,7 +46,8 @@ static const void* cluster_kernel32(const TilePlan& p) {
 }
 
 // us per iteration of a system on a cluster of cs blocks, from the columns of its
-// largest tile. Fitted to measured iterations; it only ranks the choices:
+// largest tile. Fitted to measured iterations (with a cluster barrier an exchange, 0.2
+// to 0.5 more than now); it only ranks the choices:
 //   12x12x32 on 1, 2, 4, 8, 16 blocks: 8.8, 4.4, 3.4, 2.9, 3.0
 //   24x24x48 on 8, 16: 6.4, 4.5;  18x18x48 on 4, 8, 16: 6.8, 4.3, 3.9
 //   36x36x48 on 16: 7.2 (over all SMs 5.8);  25x24x48 on 8, 16: 8.2, 6.8
