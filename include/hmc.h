@@ -385,14 +385,22 @@ hmc_status hmc_set_cg_fused_tile(hmc_ctx* ctx, int Ti, int Tj, int Tt, int depth
  * (in_use = 1: chosen by the tuner or pinned by variant 6). */
 hmc_status hmc_cg_fused_tile(hmc_ctx* ctx, int* Ti, int* Tj, int* Tt, int* depth, int* in_use);
 
-/* Test hook for the bounded waits of the persistent FP32 CG kernel (variant 4
- * above): from the next persistent solve on, every grid barrier waits for
- * `extra` more arrivals than the launch has blocks (with extra > 0 no barrier
- * can complete, a wait that nothing ends) and gives up after `limit_cycles`
- * SM clock cycles (0: the default, about one second). A solve whose wait gave
- * up returns HMC_ERR_TIMEOUT and the context stays usable. extra = 0 and
- * limit_cycles = 0 restore normal operation. */
+/* Test hook for the bounded waits of the CG kernels that run a whole solve
+ * (the persistent kernels, and the resident tiles over all SMs and on
+ * clusters): from the next such solve on, every wait of a block for the others
+ * is for `extra` more arrivals than there will be (with extra > 0 none can
+ * complete, a wait that nothing ends) and gives up after `limit_cycles` SM
+ * clock cycles (0: the default, about one second; on clusters at least
+ * 100,000). A solve whose wait gave up returns HMC_ERR_TIMEOUT and the context
+ * stays usable. extra = 0 and limit_cycles = 0 restore normal operation. */
 hmc_status hmc_set_wait_test(hmc_ctx* ctx, int extra, long long limit_cycles);
+
+/* Test hook: where the resident-tile CG runs. 0 (default) = as the rules of
+ * hmc_set_cg_variant and hmc_set_batched_variant say, 1 = over all SMs, never
+ * on a cluster, 2 = variant 7 on one cluster wherever the lattice fits one,
+ * 3 = nowhere: FP64 solves run three kernels per iteration, batches the
+ * cooperative launch or the graph loop. */
+hmc_status hmc_set_tile_test(hmc_ctx* ctx, int where);
 
 /* How the context runs CG iterations: 2 = each solve is one CUDA-graph launch
  * whose device-side while loop repeats captured chunks of iterations until
@@ -419,7 +427,9 @@ typedef struct {
   int waves;            /* grid = waves x resident blocks (0: one item per thread);
                            -tt: the tiled FP32 CG kernels with tt time slices
                            per tile of `threads` cells; -(1000 + tt): the
-                           marching kernels, tt slices per block */
+                           marching kernels, tt slices per block;
+                           cg_resident_f32: blocks of the last launch,
+                           negative on a cluster */
   int design;           /* FP32 CG kernels: 0 grid-stride (one cell per thread),
                            1 tiled, 2 marching, 4 grid-stride with two cells
                            per thread */

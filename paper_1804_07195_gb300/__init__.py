@@ -381,10 +381,15 @@ class Context:
         self._check(self.lib.hmc_set_graph_mode(self.h, mode))
 
     def set_wait_test(self, extra: int, limit_cycles: int = 0):
-        """Test hook: grid barriers of the persistent FP32 CG kernel wait for
-        `extra` more arrivals than there are blocks and give up after
+        """Test hook: the blocks of the CG kernels that run a whole solve wait
+        for `extra` more arrivals than there will be and give up after
         `limit_cycles` SM cycles (0: default); (0, 0) restores normal work."""
         self._check(self.lib.hmc_set_wait_test(self.h, extra, limit_cycles))
+
+    def set_tile_test(self, where: int):
+        """Test hook: the resident-tile CG runs 0 = as its rules say, 1 = over
+        all SMs, 2 = (variant 7) on one cluster, 3 = nowhere."""
+        self._check(self.lib.hmc_set_tile_test(self.h, where))
 
     def check_guards(self) -> int:
         """Number of the context's device buffers whose guard bands were

@@ -119,6 +119,7 @@ PROTOTYPES = {
     "hmc_set_cg_fused_tile": (S, [P, I, I, I, I]),
     "hmc_cg_fused_tile": (S, [P, C.POINTER(I), C.POINTER(I), C.POINTER(I), C.POINTER(I), C.POINTER(I)]),
     "hmc_set_wait_test": (S, [P, I, C.c_longlong]),
+    "hmc_set_tile_test": (S, [P, I]),
     "hmc_graph_mode": (S, [P, C.POINTER(I)]),
     "hmc_set_graph_mode": (S, [P, I]),
     "hmc_check_guards": (S, [P, C.POINTER(I)]),

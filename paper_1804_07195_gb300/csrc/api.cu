@@ -719,6 +719,14 @@ hmc_status hmc_set_wait_test(hmc_ctx* c, int extra, long long limit_cycles) {
   return HMC_OK;
 }
 
+hmc_status hmc_set_tile_test(hmc_ctx* c, int where) {
+  if (!c) return HMC_ERR_INVALID;
+  if (where < kTilesByRule || where > kTilesNone) return fail(c, HMC_ERR_INVALID, "where must be 0 to 3");
+  c->tile_where = (TilesWhere)where;
+  c->tuned32 = false;
+  return HMC_OK;
+}
+
 hmc_status hmc_check_guards(hmc_ctx* c, int* nbad) {
   if (!c || !nbad) return HMC_ERR_INVALID;
   *nbad = 0;

@@ -960,7 +960,7 @@ extern "C" hmc_status hmc_solve_batched(hmc_ctx* c, int nsys, const hmc_system* 
     // FP32 CG: every system on a cluster of its own where all of them fit one,
     // unless the graph loop is pinned or the wait test needs the bounded waits
     // of the cooperative launch
-    if (mixed && c->batch_variant != 1 && c->bar_extra == 0) {
+    if (mixed && c->batch_variant != 1 && c->bar_extra == 0 && c->tile_where != kTilesGrid && c->tile_where != kTilesNone) {
       std::vector<Geo> geos(nsys);
       std::vector<double> its(nsys);
       for (int i = 0; i < nsys; ++i) {

@@ -24,14 +24,14 @@ constexpr int kStrideSmall = 12 * 1024, kStrideLarge = 44 * 1024;
 
 template <int CW, int S, int AS>
 __global__ void __launch_bounds__(tile_max_threads<float, CW, S>(), 1)
-    k_cg32_cluster(const TileSys* __restrict__ list, const __grid_constant__ TileSys one) {
+    k_cg32_cluster(const TileSys* __restrict__ list, const __grid_constant__ TileSys one, unsigned extra, long long limit) {
   extern __shared__ float4 s_tile[];
   __shared__ TileSys ts;
   static_assert(sizeof(TileSys) % 4 == 0, "copied by words");
   const unsigned* src = list ? (const unsigned*)(list + blockIdx.x / cluster_size()) : (const unsigned*)&one;
   for (unsigned i = threadIdx.x; i < sizeof(TileSys) / 4; i += blockDim.x) ((unsigned*)&ts)[i] = src[i];
   __syncthreads();
-  cg_tile_solve<float, CW, S, true, AS>(ts, GridSync{}, (int)cluster_rank(), (char*)s_tile);
+  cg_tile_solve<float, CW, S, true, AS>(ts, GridSync{nullptr, nullptr, nullptr, extra, limit}, (int)cluster_rank(), (char*)s_tile);
 }
 
 static const void* cluster_kernel32(const TilePlan& p) {
@@ -123,6 +123,14 @@ static void cluster_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, c
   cfg->numAttrs = 1;
 }
 
+// The waits of an exchange: by the wait test for sums that nobody sends, and the
+// cycles after which a block gives up. Not below 50 us: a block that has given up
+// leaves once all have, and by then every store on its way to it must have landed.
+static void cluster_waits(const hmc_ctx* c, unsigned* extra, long long* limit) {
+  *extra = (unsigned)c->bar_extra;
+  *limit = c->bar_limit > 0 ? std::max(c->bar_limit, 100000LL) : 2000000000LL;
+}
+
 // Whether this GPU can run a cluster of the plan.
 static bool cluster_runs(const hmc_ctx* c, const TilePlan& p, int cs) {
   const void* k = cluster_kernel32(p);
@@ -171,7 +179,10 @@ hmc_status cg32_cluster_launch(hmc_ctx* c, const Geo& g, float2* x, float2* r, C
   const TilePlan& p = c->cluster_plan;
   const TileSys one = make_tile_sys(g, p, phase_of<float>(c).phi, x, r, nullptr, sc);
   const TileSys* list = nullptr;
-  void* args[] = {(void*)&list, (void*)&one};
+  unsigned extra = 0;
+  long long limit = 0;
+  cluster_waits(c, &extra, &limit);
+  void* args[] = {(void*)&list, (void*)&one, &extra, &limit};
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr;
   cluster_config(&cfg, &attr, p, 1 << c->cluster_log2, 1, c->stream);
@@ -179,6 +190,7 @@ hmc_status cg32_cluster_launch(hmc_ctx* c, const Geo& g, float2* x, float2* r, C
   HMC_TRY(launch_b(c, K_CG_RES32, 0.0, [&] { le = cudaLaunchKernelExC(&cfg, cluster_kernel32(p), args); }));
   if (le != cudaSuccess) return cuda_fail(c, le, "resident CG cluster launch");
   c->shape[K_CG_RES32].tiled = p.cw == 2 ? 4 : 0;  // reported as the design
+  c->shape[K_CG_RES32].waves = -(1 << c->cluster_log2);
   return HMC_OK;
 }
 
@@ -292,6 +304,9 @@ hmc_status cg32_cluster_batch_launch(hmc_ctx* c, const std::vector<ClusterGroup>
   if (!c->side_start) HMC_CUDA(c, cudaEventCreateWithFlags(&c->side_start, cudaEventDisableTiming));
   bool on[hmc_ctx::kSideStreams] = {};
   HMC_CUDA(c, cudaEventRecord(c->side_start, c->stream));
+  unsigned extra = 0;
+  long long limit = 0;
+  cluster_waits(c, &extra, &limit);
   int first = 0;
   hmc_status st = HMC_OK;
   for (size_t k = 0; k < groups.size() && st == HMC_OK; ++k) {
@@ -305,7 +320,7 @@ hmc_status cg32_cluster_batch_launch(hmc_ctx* c, const std::vector<ClusterGroup>
     on[i] = true;
     const TileSys* mine = list + first;
     const TileSys one{};
-    void* args[] = {(void*)&mine, (void*)&one};
+    void* args[] = {(void*)&mine, (void*)&one, &extra, &limit};
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr;
     cluster_config(&cfg, &attr, g.plan, 1 << g.log2, (int)g.sys.size(), c->side[i]);

@@ -205,6 +205,7 @@ hmc_status cg32_resident_launch(hmc_ctx* c, const Geo& g, float2* x, float2* r, 
   const TileSys ts = make_tile_sys(g, p, phase_of<float>(c).phi, x, r, u, sc);
   HMC_TRY(tile_grid_launch(c, K_CG_RES32, kfn, p, ts));
   c->shape[K_CG_RES32].tiled = p.cw == 2 ? 4 : 0;  // reported as the design
+  c->shape[K_CG_RES32].waves = p.tiles_j * p.tiles_t;
   return HMC_OK;
 }
 

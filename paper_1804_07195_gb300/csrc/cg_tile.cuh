@@ -89,12 +89,13 @@ struct TileSys {
   CGScal* sc;
 };
 
-// Exchanges of a cooperative launch.
+// Exchanges of a cooperative launch, and the limit of their waits; a cluster's
+// take the last two only.
 struct GridSync {
   double* part;    // [2][kTileMaxGroup] partials, 8 bytes each: the exchanges alternate
   unsigned* word;  // arrivals: the top bit flips when every block has arrived
   int* err;        // a block gave up
-  unsigned need;   // arrivals an exchange waits for
+  unsigned need;   // arrivals an exchange waits for; a cluster: sums it waits for beyond its own
   long long limit; // SM cycles
 };
 
@@ -787,7 +788,7 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
   const unsigned bar_off = bar0 - (unsigned)__cvta_generic_to_shared(sm);  // in any block of the cluster
   unsigned due = 0;
   if constexpr (CL) {
-    due = cluster_size() * nwarps * (unsigned)sizeof(T) + (unsigned)((2 * Tt + 2 * Jt) * nq * VB);
+    due = (cluster_size() * nwarps + gs.need) * (unsigned)sizeof(T) + (unsigned)((2 * Tt + 2 * Jt) * nq * VB);
     if (tid == 0) {
       bar_init(bar0);
       bar_init(bar0 + 8);
@@ -816,7 +817,7 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
       }
       const long long tw = clock64();
       bool late = false;
-      while (!bar_try(bar, parity) && !(late = clock64() - tw > 2000000000LL)) {
+      while (!bar_try(bar, parity) && !(late = clock64() - tw > gs.limit)) {
       }
       // the block's own writes to shared memory, and one answer for all its threads
       if (__syncthreads_or(late)) return false;
@@ -1079,8 +1080,9 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
     if (warp == 0) tmem_free(s_tmem, xalloc);
   }
   if constexpr (CL) cluster_barrier();  // no block leaves while one that gave up may still be written to
-  if (tile == 0 && tid == 0) {
-    CGScal* sc = ts.sc;
+  if (tid != 0) return;
+  CGScal* sc = ts.sc;
+  if (tile == 0) {
     sc->rr = rr;
     sc->rr_cur = rr;
     sc->rr32 = sc->rr_cur32 = (float)rr;
@@ -1089,8 +1091,10 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
     sc->beta = beta;
     sc->iter = iter;
     sc->first = 0;
-    sc->done = done ? done : CG_MAXIT;
   }
+  // the largest code of all blocks: one that gave up counts, also where the others
+  // had what they waited for and went on to the end
+  if (tile == 0 || done == CG_TIMEOUT) atomicMax(&sc->done, done ? done : CG_MAXIT);
 }
 
 }  // namespace hmc

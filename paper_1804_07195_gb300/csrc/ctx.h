@@ -127,6 +127,10 @@ struct ClusterPlans {
   double us[5];
 };
 
+// Where the resident-tile CG runs (test hook): as its rules say, always over all
+// SMs, always on one cluster (where it fits), or nowhere.
+enum TilesWhere { kTilesByRule, kTilesGrid, kTilesCluster, kTilesNone };
+
 struct ProfileState {
   bool timing = false;
   long long launches[K_COUNT] = {};
@@ -212,6 +216,7 @@ struct hmc_ctx {
   size_t bpool_host_bytes[4] = {};
   int bar_extra = 0;         // test hook: extra arrivals every grid barrier waits for
   long long bar_limit = 0;   // test hook: barrier wait limit in SM cycles (0: default)
+  hmc::TilesWhere tile_where = hmc::kTilesByRule;  // test hook: where the resident tiles run
 
   // batched FP32 CG: 0 = choose by timing, 1 = graph loop of per-iteration
   // kernels, 2 = one persistent cooperative launch per solve

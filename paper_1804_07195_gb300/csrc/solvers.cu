@@ -198,8 +198,9 @@ static hmc_status tune_cg(hmc_ctx* c, double ms, double sigma, const V2<R>* b) {
       if (designs.empty()) designs.push_back({false, false, false, false, -1});
       if (cg32_persist_ok(c, g)) designs.push_back({true, false, false, false, -1});
       if (cg1_fit) designs.push_back({false, true, false, false, -1});
-      if (cg32_resident_ok(c, g)) designs.push_back({false, false, true, false, -1});
-      if (cg32_cluster_ok(c, g)) designs.push_back({false, false, false, true, -1});
+      if (c->tile_where != kTilesNone && cg32_resident_ok(c, g)) designs.push_back({false, false, true, false, -1});
+      if ((c->tile_where == kTilesByRule || c->tile_where == kTilesCluster) && cg32_cluster_ok(c, g))
+        designs.push_back({false, false, false, true, -1});
       auto use_shapes = [&](int f) {
         for (int k = 0; k < nk; ++k) c->shape[ids[k]] = f >= 0 ? fam[f][k] : keep[k];
       };
@@ -255,12 +256,12 @@ template <typename R>
 hmc_status cg_core(hmc_ctx* c, double ms, double sigma, const V2<R>* b, V2<R>* x, bool x_zero,
                    double tol, int maxit, int sc_slot, bool want_true_res, SolveStats* st) {
   const Geo& g = c->geo;
-  // FP64 solves take the resident tiles wherever they fit (the wait test and a
-  // capture excepted), without timing: they were the faster at every size
+  // FP64 solves take the resident tiles wherever they fit (a capture excepted),
+  // without timing: they were the faster at every size
   // (us per iteration against the three kernels: 3x3x8 11.2 / 15.2, 24x24x48 11.4 /
   // 19.2, 36x36x64 18.6 / 27.4, 51x51x64 32.6 / 34.3, 64x64x64 40.3 / 41.5; with
   // eight slices a column, 66x66x64, they lost, 50.1 / 41.8, and have no instance)
-  const bool tiles64 = sizeof(R) == 8 && !c->capturing && c->bar_extra == 0 && cg64_resident_ok(c, c->geo);
+  const bool tiles64 = sizeof(R) == 8 && !c->capturing && c->tile_where != kTilesNone && cg64_resident_ok(c, c->geo);
   if (!c->capturing && !tiles64) HMC_TRY(tune_cg<R>(c, ms, sigma, b));
   const R dm = (R)(c->delta * ms);
   V2<R> *r, *p, *u;
@@ -313,13 +314,14 @@ hmc_status cg_core(hmc_ctx* c, double ms, double sigma, const V2<R>* b, V2<R>* x
   bool persistent = false;
   if constexpr (sizeof(R) == 4) {
     // the resident-tile kernel (one launch per solve) when the tuner or the
-    // pinned variant chose it: on one cluster, or over all SMs (there with the
-    // bounded waits of the wait test)
+    // pinned variant chose it: on one cluster, or over all SMs
     const bool pinned = c->cg32_variant == 7, tuned = c->cg32_variant == 0;
-    const bool cluster = !c->capturing && c->bar_extra == 0 &&
-                         ((pinned && cg32_prefer_cluster(c, g)) || (tuned && c->cluster32)) && cg32_cluster_ok(c, g) &&
+    const bool tiles = !c->capturing && c->tile_where != kTilesNone;
+    const bool by_rule = c->tile_where == kTilesCluster || (pinned && cg32_prefer_cluster(c, g));
+    const bool cluster = tiles && c->tile_where != kTilesGrid && ((pinned && by_rule) || (tuned && c->cluster32)) &&
+                         cg32_cluster_ok(c, g) &&
                          ((g.n & 1) || ((uintptr_t)x & 15u) == 0);  // pairs of cells are 16-byte accesses
-    const bool resident = !c->capturing && !cluster && (pinned || (tuned && (c->resident32 || c->cluster32))) &&
+    const bool resident = tiles && !cluster && (pinned || (tuned && (c->resident32 || c->cluster32))) &&
                           cg32_resident_ok(c, g);
     const bool whole = resident || cluster;
     persistent = whole || (!c->capturing && (c->cg32_variant == 4 || (tuned && c->persist32)) && cg32_persist_ok(c, g));
@@ -451,6 +453,7 @@ hmc_status cg_core(hmc_ctx* c, double ms, double sigma, const V2<R>* b, V2<R>* x
   st->iters += sch->iter;
   if (sizeof(R) == 8) st->applies64 += sch->iter; else st->applies32 += sch->iter;
   st->cg_done = sch->done;
+  if (sch->done == CG_TIMEOUT) c->tile_sync_stale = true;
   if (want_true_res) {
     HMC_TRY(mdag_launch<R>(c, g, dm, x, u));
     HMC_TRY(resid_launch<R>(c, g, dm, u, x, b, sigma, r, nullptr, nullptr, 0.0, 0, c->dscal, tk, ddm));
@@ -459,8 +462,7 @@ hmc_status cg_core(hmc_ctx* c, double ms, double sigma, const V2<R>* b, V2<R>* x
     st->true_rel = bb > 0 ? std::sqrt(rr / bb) : 0.0;
     if (sizeof(R) == 8) st->applies64++; else st->applies32++;
   }
-  if (sch->done == CG_TIMEOUT) c->tile_sync_stale = true;
-  if (sch->done == CG_TIMEOUT) return fail(c, HMC_ERR_TIMEOUT, "persistent CG: a grid barrier wait gave up");
+  if (sch->done == CG_TIMEOUT) return fail(c, HMC_ERR_TIMEOUT, "persistent CG: a wait between thread blocks gave up");
   if (sch->done == CG_BREAKDOWN) return fail(c, HMC_ERR_NAN, "CG breakdown: non-positive or non-finite curvature/residual");
   if (sch->done == CG_MAXIT) return fail(c, HMC_ERR_NOT_CONVERGED, "CG reached its iteration limit");
   return HMC_OK;
