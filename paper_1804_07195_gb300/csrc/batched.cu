@@ -724,6 +724,9 @@ static hmc_status batched_cg(hmc_ctx* c, BatchWs& w, cudaStream_t s, const V2<R>
       HMC_CUDA(c, cudaMemcpyAsync(w.st_host, w.st, sizeof(BState) * w.nsys, cudaMemcpyDeviceToHost, s));
       HMC_CUDA(c, cudaStreamSynchronize(s));
       for (int i = 0; i < w.nsys; ++i) c->prof.bytes[K_BATCH_CG32] += (double)w.st_host[i].cg.iter * w.hsys[i].g.N * 88.0;
+      // an x that was left half way is no correction to add
+      for (int i = 0; i < w.nsys; ++i)
+        if (w.st_host[i].cg.done == CG_TIMEOUT) return fail(c, HMC_ERR_TIMEOUT, "batched CG: a wait between thread blocks gave up");
       return HMC_OK;
     }
   }
@@ -958,9 +961,8 @@ extern "C" hmc_status hmc_solve_batched(hmc_ctx* c, int nsys, const hmc_system* 
       HMC_TRY(bmalloc(c, w, (void**)&w.rr32, sizeof(float2) * Nt));
     }
     // FP32 CG: every system on a cluster of its own where all of them fit one,
-    // unless the graph loop is pinned or the wait test needs the bounded waits
-    // of the cooperative launch
-    if (mixed && c->batch_variant != 1 && c->bar_extra == 0 && c->tile_where != kTilesGrid && c->tile_where != kTilesNone) {
+    // unless the graph loop is pinned
+    if (mixed && c->batch_variant != 1 && c->tile_where != kTilesGrid && c->tile_where != kTilesNone) {
       std::vector<Geo> geos(nsys);
       std::vector<double> its(nsys);
       for (int i = 0; i < nsys; ++i) {

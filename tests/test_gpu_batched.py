@@ -81,6 +81,7 @@ def test_persistent_batched_wait_times_out_and_context_survives():
                    "x": torch.zeros(p.nsites, dtype=torch.complex128, device="cuda")}]
     with ctx_for(p) as ctx:
         ctx.set_batched_variant(2)
+        ctx.set_tile_test(1)  # the cooperative launch, no clusters (theirs: test_gpu_tile_waits)
         ctx.set_wait_test(1, 2_000_000)
         with pytest.raises(hmc.HMCError) as e:
             ctx.solve_batched(mk(), mixed=True)

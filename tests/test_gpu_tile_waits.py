@@ -58,3 +58,23 @@ def test_fp64_tiles(shape):
         assert ctx.profile_read()["cg_resident_f64"]["launches"] == 2
     r = w.b - of.apply_MMdag(ol, w.phi, 0.3, host(x))
     assert info["status"] == 0 and np.linalg.norm(r) <= 1.0001e-10 * np.linalg.norm(w.b)
+
+
+def test_batched_clusters():
+    """A mixed batch whose systems run on clusters of different sizes."""
+    need_gpu()
+    import paper_1804_07195_gb300 as hmc
+    import torch
+    ws = [W.small(*sh, seed=2620 + k, U=3.0, beta=6.0) for k, sh in enumerate([(6, 6, 16), (24, 24, 33), (5, 3, 9)])]
+
+    def systems():
+        return [{"lattice": hmc.Lattice(w.lat.n, w.lat.m, w.lat.nt, w.lat.kappa, w.lat.U, w.lat.beta), "phi": dev(w.phi),
+                 "ms": 0.3, "b": dev(w.b), "x": torch.zeros(w.lat.nsites, dtype=torch.complex128, device="cuda")}
+                for w in ws]
+    with ctx_for(ws[0].lat) as ctx:
+        times_out(ctx, lambda: ctx.solve_batched(systems(), mixed=True))
+        sy = systems()
+        ctx.solve_batched(sy, mixed=True)
+    for w, s in zip(ws, sy):
+        r = w.b - of.apply_MMdag(OLat.from_params(w.lat), w.phi, 0.3, host(s["x"]))
+        assert np.linalg.norm(r) <= 1.0001e-10 * np.linalg.norm(w.b)
