@@ -346,7 +346,8 @@ hmc_status hmc_set_cg_variant(hmc_ctx* ctx, int variant);
  * (default) takes the clusters where they fit; otherwise it runs the first
  * inner solve of the context with 1 and the second with 2 and keeps the one
  * with the shorter time per iteration; 1 or 2 pins one. The variant in use
- * (0 = not chosen yet) is reported by hmc_batched_variant. */
+ * (of the last batch with mixed = 1; 0 = not chosen yet) is reported by
+ * hmc_batched_variant. */
 hmc_status hmc_set_batched_variant(hmc_ctx* ctx, int variant);
 hmc_status hmc_batched_variant(hmc_ctx* ctx, int* variant);
 

@@ -625,13 +625,14 @@ hmc_status hmc_set_batched_variant(hmc_ctx* c, int variant) {
   if (variant < 0 || variant > 2) return fail(c, HMC_ERR_INVALID, "variant must be 0, 1 or 2");
   c->batch_variant = variant;
   c->batch_choice = 0;
+  c->batch_clusters = false;
   c->batch_us[0] = c->batch_us[1] = 0.f;
   return HMC_OK;
 }
 
 hmc_status hmc_batched_variant(hmc_ctx* c, int* variant) {
   if (!c || !variant) return HMC_ERR_INVALID;
-  *variant = c->batch_variant ? c->batch_variant : c->batch_choice;
+  *variant = c->batch_variant ? c->batch_variant : c->batch_clusters ? 2 : c->batch_choice;
   return HMC_OK;
 }
 

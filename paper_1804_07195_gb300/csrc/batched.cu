@@ -714,7 +714,6 @@ static hmc_status batched_cg(hmc_ctx* c, BatchWs& w, cudaStream_t s, const V2<R>
   HMC_CUDA(c, cudaGetLastError());
   if constexpr (sizeof(R) == 4) {
     if (w.clusters) {
-      c->batch_choice = 2;
       cudaEvent_t a = nullptr;
       prof_begin(c, K_BATCH_CG32, &a);
       const hmc_status st = cg32_cluster_batch_launch(c, w.groups, w.tsys);
@@ -974,6 +973,7 @@ extern "C" hmc_status hmc_solve_batched(hmc_ctx* c, int nsys, const hmc_system* 
       }
       w.clusters = cg32_cluster_batch(c, geos, its, &w.groups);
     }
+    if (mixed) c->batch_clusters = w.clusters;
     if (w.clusters) {
       HMC_TRY(bmalloc(c, w, (void**)&w.tsys, sizeof(TileSys) * nsys));
       std::vector<TileSys> h;

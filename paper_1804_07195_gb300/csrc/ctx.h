@@ -218,10 +218,11 @@ struct hmc_ctx {
   long long bar_limit = 0;   // test hook: barrier wait limit in SM cycles (0: default)
   hmc::TilesWhere tile_where = hmc::kTilesByRule;  // test hook: where the resident tiles run
 
-  // batched FP32 CG: 0 = choose by timing, 1 = graph loop of per-iteration
-  // kernels, 2 = one persistent cooperative launch per solve
+  // batched FP32 CG: 0 = clusters where they fit, else by timing, 1 = graph loop
+  // of per-iteration kernels, 2 = clusters or one persistent cooperative launch
   int batch_variant = 0;
-  int batch_choice = 0;                // the variant chosen (0: not yet)
+  int batch_choice = 0;                // the variant chosen for batches that fit no clusters (0: not yet)
+  bool batch_clusters = false;         // the last mixed batch ran on clusters
   float batch_us[2] = {0.f, 0.f};      // us per iteration measured for 1 and 2
   // per-chain contexts of hmc_md_trajectory_batched (slot i: chain i of the
   // last call; recreated when a chain's lattice changes), destroyed with ctx

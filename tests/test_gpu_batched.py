@@ -92,6 +92,29 @@ def test_persistent_batched_wait_times_out_and_context_survives():
     check([(w, 0.1, 0.0, w.b)], [host(sy[0]["x"])], infos, 1e-10)
 
 
+def test_a_batch_on_clusters_leaves_the_choice_for_others_open():
+    """After a batch on clusters the first inner solve of one that runs elsewhere
+    is still a timed candidate (nothing chosen yet), and the second decides."""
+    need_gpu()
+    import paper_1804_07195_gb300 as hmc
+    w = W.small(6, 6, 16, seed=331, U=3.0, beta=6.0)
+    p = w.lat
+    x = torch.zeros(p.nsites, dtype=torch.complex128, device="cuda")
+    one = [{"lattice": hmc.Lattice(p.n, p.m, p.nt, p.kappa, p.U, p.beta), "phi": dev(w.phi), "ms": 0.1, "b": dev(w.b),
+            "x": x, "tol": 0.3}]  # one inner solve
+    with ctx_for(p) as ctx:
+        ctx.solve_batched(one, mixed=True)
+        assert ctx.batched_variant() == 2
+        ctx.set_tile_test(1)
+        ctx.solve_batched(one, mixed=True)
+        assert ctx.batched_variant() == 0
+        ctx.solve_batched(one, mixed=True)
+        assert ctx.batched_variant() in (1, 2)
+        ctx.set_tile_test(0)
+        ctx.solve_batched(one, mixed=True)
+        assert ctx.batched_variant() == 2
+
+
 @pytest.mark.parametrize("mixed", [0, 1])
 def test_uneven_small_batch(mixed):
     need_gpu()
