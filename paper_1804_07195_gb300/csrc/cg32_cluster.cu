@@ -301,7 +301,13 @@ bool cg32_cluster_batch(hmc_ctx* c, const std::vector<Geo>& geos, const std::vec
 }
 
 hmc_status cg32_cluster_batch_launch(hmc_ctx* c, const std::vector<ClusterGroup>& groups, const TileSys* list) {
+  // all that can fail for want of memory before the first launch
   if (!c->side_start) HMC_CUDA(c, cudaEventCreateWithFlags(&c->side_start, cudaEventDisableTiming));
+  for (const ClusterGroup& g : groups) {
+    const int i = g.stream;
+    if (!c->side[i]) HMC_CUDA(c, cudaStreamCreateWithFlags(&c->side[i], cudaStreamNonBlocking));
+    if (!c->side_done[i]) HMC_CUDA(c, cudaEventCreateWithFlags(&c->side_done[i], cudaEventDisableTiming));
+  }
   bool on[hmc_ctx::kSideStreams] = {};
   HMC_CUDA(c, cudaEventRecord(c->side_start, c->stream));
   unsigned extra = 0;
@@ -312,11 +318,13 @@ hmc_status cg32_cluster_batch_launch(hmc_ctx* c, const std::vector<ClusterGroup>
   for (size_t k = 0; k < groups.size() && st == HMC_OK; ++k) {
     const ClusterGroup& g = groups[k];
     const int i = g.stream;
-    if (!c->side[i]) {
-      HMC_CUDA(c, cudaStreamCreateWithFlags(&c->side[i], cudaStreamNonBlocking));
-      HMC_CUDA(c, cudaEventCreateWithFlags(&c->side_done[i], cudaEventDisableTiming));
+    if (!on[i]) {
+      const cudaError_t e = cudaStreamWaitEvent(c->side[i], c->side_start, 0);
+      if (e != cudaSuccess) {
+        st = cuda_fail(c, e, "batched CG side stream");
+        break;
+      }
     }
-    if (!on[i]) HMC_CUDA(c, cudaStreamWaitEvent(c->side[i], c->side_start, 0));
     on[i] = true;
     const TileSys* mine = list + first;
     const TileSys one{};
@@ -329,10 +337,15 @@ hmc_status cg32_cluster_batch_launch(hmc_ctx* c, const std::vector<ClusterGroup>
     c->prof.launches[K_BATCH_CG32]++;
     first += (int)g.sys.size();
   }
-  for (int i = 0; i < hmc_ctx::kSideStreams; ++i) {  // also after a failure: nothing outlives the call
+  // also after a failure: nothing outlives the call, whose buffers go back to the pool
+  for (int i = 0; i < hmc_ctx::kSideStreams; ++i) {
     if (!on[i]) continue;
-    HMC_CUDA(c, cudaEventRecord(c->side_done[i], c->side[i]));
-    HMC_CUDA(c, cudaStreamWaitEvent(c->stream, c->side_done[i], 0));
+    cudaError_t e = cudaEventRecord(c->side_done[i], c->side[i]);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, c->side_done[i], 0);
+    if (e != cudaSuccess) {
+      cudaStreamSynchronize(c->side[i]);
+      if (st == HMC_OK) st = cuda_fail(c, e, "batched CG side stream");
+    }
   }
   return st;
 }
