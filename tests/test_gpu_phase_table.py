@@ -82,9 +82,32 @@ def test_neighbour_sums():
                 for f, o in ((ctx.apply_M, of.apply_M), (ctx.apply_Mdag, of.apply_Mdag)):
                     ref = o(ol, w.phi, ms, v)
                     assert np.abs(host(f(dev(w.phi), ms, dev(v))) - ref).max() <= 4e-15 * np.abs(v).max(), (name, ms)
+        # M(-v) = -M v bit for bit: no bias towards one sign
+        for v in (vecs["plain"], vecs["spread"]):
+            for f in (ctx.apply_M, ctx.apply_Mdag):
+                assert np.array_equal(host(f(dev(w.phi), 0.0, dev(-v))), -host(f(dev(w.phi), 0.0, dev(v))))
         v = z(r)
         v[[5, 60]] = [np.nan, np.inf]
         with np.errstate(invalid="ignore"):
             ref = of.apply_M(ol, w.phi, 0.0, v)
         got = host(ctx.apply_M(dev(w.phi), 0.0, dev(v)))
         assert np.array_equal(np.isfinite(got), np.isfinite(ref))
+
+
+@pytest.mark.parametrize("fixed_point", [20, 40])
+def test_exact_sums_stay_exact(fixed_point):
+    """Entries that are small whole multiples of a power of two, most of them
+    zero, phi = 0 and a power of two as hopping: every product and sum of the
+    operator is exact in FP64, cancelling ones included, and must come out so."""
+    need_gpu()
+    w = W.small(6, 5, 8, seed=2103, U=2.0, beta=2.0)  # delta kappa = 1/4
+    ol = OLat.from_params(w.lat)
+    g = np.random.Generator(np.random.PCG64(33))
+    n = w.lat.nsites
+    zero = np.zeros(n)
+    draw = lambda: np.where(g.random(n) < 0.6, 0.0, g.integers(-3, 4, n) * 2.0 ** -(fixed_point * g.integers(0, 2, n)))
+    with ctx_for(w.lat) as ctx:
+        for _ in range(3):
+            v = draw() + 1j * draw()
+            for f, o in ((ctx.apply_M, of.apply_M), (ctx.apply_Mdag, of.apply_Mdag)):
+                assert np.array_equal(host(f(dev(zero), 0.0, dev(v))), o(ol, zero, 0.0, v))
