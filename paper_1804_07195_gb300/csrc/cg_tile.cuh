@@ -42,7 +42,7 @@
 //
 // Every sum is formed in a fixed order that is the same in every block, so
 // all blocks of a group hold the same scalars and leave together. FP32 sums
-// are float-float pairs, FP64 sums doubles.
+// are float-float pairs, FP64 sums doubles, up to alpha, beta and the stopping test.
 //
 // What bounds an FP32 iteration of a cooperative launch (us, 2070 MHz; in
 // brackets the design before it, which read r, x and phi from L2 row by row in
@@ -278,6 +278,24 @@ struct Red<float> {
     return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
   }
   static __device__ __forceinline__ float value(T a) { return a.x + a.y; }
+  static __device__ __forceinline__ T of64(double a) {
+    const float h = (float)a;
+    return make_float2(h, (float)(a - (double)h));
+  }
+  static __device__ __forceinline__ double to64(T a) { return (double)a.x + (double)a.y; }
+  static __device__ __forceinline__ bool le(T a, T b) { return (a.x - b.x) + (a.y - b.y) <= 0.f; }
+  // a / b (b > 0) from all bits of both, rounded once: the approximate quotient,
+  // off by 2^-22, and the exact rest over b. rc: about 1 / b, or 0 outside the range
+  // of that, and then the quotient of the high parts.
+  static __device__ __forceinline__ float over(T b) {
+    return b.x > 1e-30f && b.x < 1e30f ? __fdividef(1.f, b.x) : 0.f;
+  }
+  static __device__ __forceinline__ float ratio(T a, T b, float rc) {
+    if (rc == 0.f) return a.x / b.x;
+    const float q = a.x * rc;
+    return fmaf(fmaf(-q, b.x, a.x) + fmaf(-q, b.y, a.y), rc, q);
+  }
+  static __device__ __forceinline__ float ratio(T a, T b) { return ratio(a, b, over(b)); }
 };
 template <>
 struct Red<double> {
@@ -287,6 +305,11 @@ struct Red<double> {
   static __device__ __forceinline__ T add(T a, T b) { return a + b; }
   static __device__ __forceinline__ T shfl(T a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
   static __device__ __forceinline__ double value(T a) { return a; }
+  static __device__ __forceinline__ T of64(double a) { return a; }
+  static __device__ __forceinline__ double to64(T a) { return a; }
+  static __device__ __forceinline__ bool le(T a, T b) { return a <= b; }
+  static __device__ __forceinline__ int over(T) { return 0; }
+  static __device__ __forceinline__ double ratio(T a, T b, int = 0) { return a / b; }
 };
 template <typename R>
 __device__ __forceinline__ typename Red<R>::T warp_sum(typename Red<R>::T v) {
@@ -422,21 +445,16 @@ template <typename R>
 struct TileScal;
 template <>
 struct TileScal<float> {
-  static __device__ __forceinline__ void load(const CGScal* s, float& dm, float& sigma, float& rr, float& thresh) {
+  static __device__ __forceinline__ void load(const CGScal* s, float& dm, float& sigma) {
     dm = s->dm32;
     sigma = s->sigma32;
-    rr = s->rr32;
-    thresh = s->thresh32;
   }
 };
 template <>
 struct TileScal<double> {
-  static __device__ __forceinline__ void load(const CGScal* s, double& dm, double& sigma, double& rr,
-                                              double& thresh) {
+  static __device__ __forceinline__ void load(const CGScal* s, double& dm, double& sigma) {
     dm = s->dm;
     sigma = s->sigma;
-    rr = s->rr;
-    thresh = s->thresh;
   }
 };
 
@@ -655,13 +673,23 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
     TtP = min(TN, nt - tb * TN);
   }
 
-  R dm, sigma, rr, thresh;
-  TileScal<R>::load(ts.sc, dm, sigma, rr, thresh);
+  // |r|^2 (of iteration i in s_rr[i & 1]) and <p, A p> keep all bits of their sums;
+  // alpha and beta are rounded to R from these. Kept in shared memory, as registers
+  // are short: by thread 0, read behind a barrier (CL) or by thread 0 alone.
+  R dm, sigma;
+  TileScal<R>::load(ts.sc, dm, sigma);
+  __shared__ T s_rr[2], s_pap, s_thresh;
+  T rr = RT::of64(ts.sc->rr), thresh = RT::of64(ts.sc->thresh);
   const L ldm = LN::set(dm), ldk = LN::set(geo_dk(ts.g, R(0))), lndk = LN::set(-geo_dk(ts.g, R(0)));
   int iter = ts.sc->iter, done = ts.sc->done;
   const int maxit = ts.sc->maxit;
-  R rr_prev = R(1), pAp = R(0), alpha = R(0), beta = R(0);
+  R alpha = R(0), beta = R(0);
   bool first = true;
+  if (tid == 0) {
+    s_rr[iter & 1] = rr;
+    s_pap = RT::zero();
+    s_thresh = thresh;
+  }
   // exchanges so far; CL = false: its parity is the arrival word's top bit
   unsigned ep = CL ? 0u : *(const volatile unsigned*)gs.word >> 31;
 
@@ -875,14 +903,13 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
   for (;;) {
     if (CL || tid == 0) {
       if (!done) {
-        if (!isfinite(rr))
+        if (!isfinite(RT::value(rr)))
           done = CG_BREAKDOWN;
-        else if (rr <= thresh)
+        else if (RT::le(rr, thresh))
           done = CG_CONVERGED;
         else if (iter >= maxit)
           done = CG_MAXIT;
       }
-      beta = first ? R(0) : rr / rr_prev;
     }
     R fb = beta, fap = alpha;
     int stop = done;
@@ -964,6 +991,7 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
         }
     }
     T tot;
+    if constexpr (CL) rr = s_rr[iter & 1];  // (at hand when the sum arrives)
     bool ok = exchange(total(acc) + (sigma != R(0) ? sigma * total(accp) : R(0)),
                        [&] { fetch_padding(Ug, false); }, &tot);
     // phases of the first slice of M
@@ -972,9 +1000,11 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
       fbt = PH::load(ph, Hq + k_first);
     }
     if (CL || tid == 0) {
-      pAp = ok ? RT::value(tot) : R(0);
-      const bool bad = !(pAp > R(0)) || !isfinite(pAp);
-      alpha = bad ? R(0) : rr / pAp;
+      if constexpr (!CL) rr = s_rr[iter & 1];
+      if (!ok) tot = RT::zero();
+      const bool bad = !(RT::value(tot) > R(0)) || !isfinite(RT::value(tot));
+      alpha = bad ? R(0) : RT::ratio(rr, tot);
+      if (tid == 0) s_pap = tot;
       if (bad) done = ok ? CG_BREAKDOWN : CG_TIMEOUT;
     }
     R fal = alpha;
@@ -1035,14 +1065,27 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
     // the neighbours' r waits in the padding of u, which nothing reads until the
     // next exchange has refilled it (the block's barrier in `exchange` orders
     // the reads of u above before these writes)
+    decltype(RT::over(rr)) over{};
+    if constexpr (CL) {
+      rr = s_rr[iter & 1];
+      thresh = s_thresh;
+      over = RT::over(rr);
+    }
     ok = exchange(total(accr),
                   [&] { fetch_padding(rg, true); }, &tot);
     if (CL || tid == 0) {
-      rr_prev = rr;
-      if (ok)
-        rr = RT::value(tot);
-      else
+      if constexpr (!CL) {
+        rr = s_rr[iter & 1];
+        thresh = s_thresh;
+        over = RT::over(rr);
+      }
+      if (!ok) {
+        tot = rr;
         done = CG_TIMEOUT;
+      }
+      beta = RT::ratio(tot, rr, over);
+      rr = tot;
+      if (tid == 0) s_rr[(iter + 1) & 1] = rr;
     }
     ++iter;
     first = false;
@@ -1083,10 +1126,9 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
   if (tid != 0) return;
   CGScal* sc = ts.sc;
   if (tile == 0) {
-    sc->rr = rr;
-    sc->rr_cur = rr;
-    sc->rr32 = sc->rr_cur32 = (float)rr;
-    sc->pAp = pAp;
+    sc->rr = sc->rr_cur = RT::to64(s_rr[iter & 1]);
+    sc->rr32 = sc->rr_cur32 = (float)sc->rr;
+    sc->pAp = RT::to64(s_pap);
     sc->alpha = alpha;
     sc->beta = beta;
     sc->iter = iter;

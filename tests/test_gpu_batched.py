@@ -115,6 +115,37 @@ def test_a_batch_on_clusters_leaves_the_choice_for_others_open():
         assert ctx.batched_variant() == 2
 
 
+@pytest.mark.parametrize("where", [0, 1])
+def test_fp32_scalars_of_a_batch_keep_all_bits(where):
+    """x after one FP32 iteration on whole numbers, phi = 0 and a power of two as
+    hopping, so that every product and sum is exact: alpha must be |r|^2 / <p, A p>
+    rounded once to FP32 from the exact sums (more than 24 bits), on clusters and
+    in the graph loop. The shift 64 brings the residual below tol in one step."""
+    need_gpu()
+    import paper_1804_07195_gb300 as hmc
+    rng = np.random.Generator(np.random.PCG64(340))
+    systems, want = [], []
+    for sh in [(12, 12, 32), (13, 11, 20), (6, 6, 16), (24, 24, 48), (7, 30, 9)] * 2:
+        lat = hmc.Lattice(*sh, 0.5, 2.0, 0.5 * sh[2])  # delta kappa = 1/4
+        ol = OLat.from_params(W.small(*sh, seed=1, kappa=0.5, U=2.0, beta=0.5 * sh[2]).lat)
+        p = rng.integers(-9, 10, lat.nsites) + 1j * rng.integers(-9, 10, lat.nsites)
+        zero = np.zeros(lat.nsites)
+        u = of.apply_Mdag(ol, zero, 0.0, p)
+        sq = lambda v: float((v.real ** 2 + v.imag ** 2).sum())  # exact: below 2^53 of its units
+        alpha = np.float32(sq(p) / (sq(u) + 64.0 * sq(p)))
+        want.append((alpha * p.astype(np.complex64)).astype(np.complex128))
+        systems.append({"lattice": lat, "phi": dev(zero), "ms": 0.0, "sigma": 64.0, "b": dev(p), "tol": 0.25,
+                        "x": torch.zeros(lat.nsites, dtype=torch.complex128, device="cuda"), "maxit": 1})
+    with ctx_for(W.small(6, 6, 16, seed=1).lat) as ctx:
+        ctx.set_tile_test(where)
+        if where:
+            ctx.set_batched_variant(1)
+        infos = ctx.solve_batched(systems, mixed=True)
+    for s, x, info in zip(systems, want, infos):
+        assert info["iters_inner"] == 1 and info["iters_outer"] == 1
+        assert np.array_equal(host(s["x"]), x)
+
+
 @pytest.mark.parametrize("mixed", [0, 1])
 def test_uneven_small_batch(mixed):
     need_gpu()
