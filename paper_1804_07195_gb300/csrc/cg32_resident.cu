@@ -21,6 +21,19 @@ __global__ void __launch_bounds__(tile_max_threads<float, 2, S>(), 1) k_cg32_res
   cg_tile_solve<float, 2, S, false, tile_array_stride<false>()>(ts, gs, blockIdx.x, (char*)s_tile);
 }
 
+// Lattices whose tiles leave no room for the padding's table: arrays up to the whole
+// of shared memory, the table in global memory, where a thread's own entries cost it a
+// trip to L2 twice an iteration. (us per iteration, in brackets the best of the designs
+// that run it from L2: 106x106x64 13.3, 108x108x64 16.4 (19.6), 110x110x64 16.7 (20.1),
+// 99x99x64 16.7 (17.5), 105x105x64 16.9 (19.1). Pairs in columns of eight slices are the
+// slowest: 352 threads; single cells in 672 threads take 16.8 at 108x108x64.)
+constexpr int kStrideAll = 57856;
+template <int CW, int S>
+__global__ void __launch_bounds__(tile_max_threads<float, CW, S>(), 1) k_cg32_resident_large(TileSys ts, GridSync gs) {
+  extern __shared__ float4 s_tile[];
+  cg_tile_solve<float, CW, S, false, kStrideAll, true>(ts, gs, blockIdx.x, (char*)s_tile);
+}
+
 const int* tile_slices32(int cw) {
   static const int one[] = {1, 2, 4, 4 + kXInMemory, 8, 8 + kXInMemory, 0}, two[] = {1, 2, 2 + kXInMemory, 4, 4 + kXInMemory, 0};
   return cw == 2 ? two : one;
@@ -95,7 +108,7 @@ bool tile_plan_grid(const hmc_ctx* c, const Geo& g, int cw, int real, const int*
   return found;
 }
 
-TileSys make_tile_sys(const Geo& g, const TilePlan& p, const void* ph, void* x, void* r, void* U, CGScal* sc) {
+TileSys make_tile_sys(const Geo& g, const TilePlan& p, const void* ph, void* x, void* r, void* U, CGScal* sc, void* gtab) {
   TileSys ts;
   ts.g = g;
   ts.J = p.J;
@@ -110,6 +123,7 @@ TileSys make_tile_sys(const Geo& g, const TilePlan& p, const void* ph, void* x, 
   ts.x = x;
   ts.r = r;
   ts.U = U;
+  ts.gtab = (uint2*)gtab;
   ts.sc = sc;
   return ts;
 }
@@ -179,12 +193,74 @@ static const TilePlan* plan32(hmc_ctx* c, const Geo& g, int cw) {
   return p.cw > 0 ? &p : nullptr;
 }
 
-bool cg32_resident_ok(hmc_ctx* c, const Geo& g) { return plan32(c, g, 2) || plan32(c, g, 1); }
+// The same for lattices that plan32 finds no tiles for. T need not be a multiple
+// of the slices a column has. table: bytes of global memory at hand for the table.
+static const int* slices_large(int cw) {
+  static const int one[] = {8 + kXInMemory, 0}, two[] = {4 + kXInMemory, 8 + kXInMemory, 0};
+  return cw == 2 ? two : one;
+}
+static int max_threads_large(int cw, int S) {
+  if (cw == 1) return tile_max_threads<float, 1, 8 + kXInMemory>();
+  return S == 4 + kXInMemory ? tile_max_threads<float, 2, 4 + kXInMemory>() : tile_max_threads<float, 2, 8 + kXInMemory>();
+}
+static const void* kernel_large(int cw, int S) {
+  if (cw == 1) return (const void*)k_cg32_resident_large<1, 8 + kXInMemory>;
+  return S == 4 + kXInMemory ? (const void*)k_cg32_resident_large<2, 4 + kXInMemory>
+                             : (const void*)k_cg32_resident_large<2, 8 + kXInMemory>;
+}
+static bool plan_large(const hmc_ctx* c, const Geo& g, int cw, TilePlan* out) {
+  if (g.n % cw) return false;
+  const size_t cap = smem_cap(c, 1024), table = sizeof(float2) * (size_t)g.N;
+  const int nq = g.n / cw;
+  bool found = false;
+  double best = 0.0;
+  for (const int* S = slices_large(cw); *S; ++S)
+    for (int T = 1; T <= g.nt && (size_t)(T + 1) * 2 * g.n * sizeof(float2) <= (size_t)kStrideAll; ++T)
+      for (int J = 1; J <= g.m; ++J) {
+        TilePlan p;
+        p.cw = cw;
+        p.S = *S;
+        p.J = J;
+        p.T = T;
+        p.nseg = (T + tile_slices(*S) - 1) / tile_slices(*S);
+        p.tiles_j = (g.m + J - 1) / J;
+        p.tiles_t = (g.nt + T - 1) / T;
+        p.stride = kStrideAll;
+        const size_t one = (size_t)(T + 1) * (J + 1) * g.n * sizeof(float2);
+        const long long th = ((long long)nq * J * p.nseg + 31) / 32 * 32;
+        p.smem = 3 * (size_t)kStrideAll + one;
+        if (one > (size_t)kStrideAll || p.smem > cap || th > max_threads_large(cw, *S)) break;
+        const long long tiles = (long long)p.tiles_j * p.tiles_t;
+        if (tiles > std::min(c->nsm, kTileMaxGroup) || tiles * 2 * (T + J) * nq * sizeof(uint2) > table) continue;
+        p.threads = (int)th;
+        const double cost = (double)J * T * nq + 0.7 * (J + T) * nq + 8.0 * tile_slices(*S);
+        if (!found || cost < best) {
+          found = true;
+          best = cost;
+          *out = p;
+        }
+      }
+  return found;
+}
+static const TilePlan* plan32_large(hmc_ctx* c, const Geo& g, int cw) {
+  TilePlan& p = c->tile_plan32_large[cw - 1];
+  if (p.cw == 0 && !plan_large(c, g, cw, &p)) p.cw = -1;
+  return p.cw > 0 ? &p : nullptr;
+}
+
+// two cells per column where n is even and every vector is 16-byte aligned
+static const TilePlan* pick32(hmc_ctx* c, const Geo& g, bool aligned) {
+  const TilePlan* p = aligned ? plan32(c, g, 2) : nullptr;
+  if (!p) p = plan32(c, g, 1);
+  if (!p && aligned) p = plan32_large(c, g, 2);
+  return p ? p : plan32_large(c, g, 1);
+}
+
+bool cg32_resident_ok(hmc_ctx* c, const Geo& g) { return pick32(c, g, true) != nullptr; }
 
 bool cg32_prefer_cluster(hmc_ctx* c, const Geo& g) {
   if (!cg32_cluster_ok(c, g)) return false;
-  const TilePlan* p = plan32(c, g, 2);
-  if (!p) p = plan32(c, g, 1);
+  const TilePlan* p = pick32(c, g, true);
   if (!p) return true;
   // us per iteration over all SMs: two exchanges through L2, phase latency, work
   // (measured: 5.6 at 36x36x64, 7.95 at 72x72x64); cluster_us has the cluster's.
@@ -194,15 +270,13 @@ bool cg32_prefer_cluster(hmc_ctx* c, const Geo& g) {
   return c->cluster_us < 5.2 + 2.6e-3 * cols;
 }
 
-hmc_status cg32_resident_launch(hmc_ctx* c, const Geo& g, float2* x, float2* r, float2* u, CGScal* sc) {
-  // two cells per column where n is even and every vector is 16-byte aligned
+hmc_status cg32_resident_launch(hmc_ctx* c, const Geo& g, float2* x, float2* r, float2* u, float2* spare, CGScal* sc) {
   auto al16 = [](const void* v) { return ((uintptr_t)v & 15u) == 0; };
-  const TilePlan* pp = al16(x) && al16(r) && al16(u) ? plan32(c, g, 2) : nullptr;
-  if (!pp) pp = plan32(c, g, 1);
+  const TilePlan* pp = pick32(c, g, al16(x) && al16(r) && al16(u));
   if (!pp) return fail(c, HMC_ERR_INVALID, "resident CG tiles do not fit on chip");
   const TilePlan& p = *pp;
-  const void* kfn = grid_kernel32(p.cw, p.S);
-  const TileSys ts = make_tile_sys(g, p, phase_of<float>(c).phi, x, r, u, sc);
+  const void* kfn = p.stride == kStrideAll ? kernel_large(p.cw, p.S) : grid_kernel32(p.cw, p.S);
+  const TileSys ts = make_tile_sys(g, p, phase_of<float>(c).phi, x, r, u, sc, spare);
   HMC_TRY(tile_grid_launch(c, K_CG_RES32, kfn, p, ts));
   c->shape[K_CG_RES32].tiled = p.cw == 2 ? 4 : 0;  // reported as the design
   c->shape[K_CG_RES32].waves = p.tiles_j * p.tiles_t;

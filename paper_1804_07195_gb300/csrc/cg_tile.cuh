@@ -86,6 +86,7 @@ struct TileSys {
   FastDiv fq;    // division by the columns of a row, n / CW
   const void* ph;  // FP32: phi as float, in [-pi, pi]; FP64: e^{i phi}
   void *x, *r, *U;
+  uint2* gtab;   // the padding's table where shared memory has no room for it, tile after tile
   CGScal* sc;
 };
 
@@ -487,9 +488,9 @@ constexpr int tile_max_threads() {
 }
 
 // The solve of one system by the block `tile` of its group. sm: four padded
-// arrays AS bytes apart, the table of the padding (8 bytes a column) and, for CL,
-// the neighbours' r there.
-template <typename R, int CW, int INST, bool CL, int AS>
+// arrays AS bytes apart, the table of the padding (8 bytes a column; GT: in global
+// memory instead) and, for CL, the neighbours' r there.
+template <typename R, int CW, int INST, bool CL, int AS, bool GT = false>
 __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync& gs, int tile, char* sm) {
   using LN = Lane<R, CW>;
   using L = typename LN::L;
@@ -594,7 +595,7 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
   const int e_first = CL ? tid : nwarps > 1 ? tid - 32 : tid;
   const int e_step = CL ? (int)blockDim.x : nwarps > 1 ? (int)blockDim.x - 32 : 32;
   const int e_end = e_first < 0 ? e_first : lines * nq;
-  uint2* const tab = (uint2*)(sm + TAB);
+  uint2* const tab = GT ? ts.gtab + (size_t)tile * (2 * (TN + J) * nq) : (uint2*)(sm + TAB);
   for (int e = e_first; e < e_end; e += e_step) {
     const int l = (int)fdiv((uint32_t)e, ts.fq);
     int kind, ip, iu, k;

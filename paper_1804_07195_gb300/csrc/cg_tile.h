@@ -33,7 +33,8 @@ inline bool tile_allow_smem(const hmc_ctx* c, const void* k) {
   return false;
 }
 
-TileSys make_tile_sys(const Geo& g, const TilePlan& p, const void* ph, void* x, void* r, void* U, CGScal* sc);
+TileSys make_tile_sys(const Geo& g, const TilePlan& p, const void* ph, void* x, void* r, void* U, CGScal* sc,
+                      void* gtab = nullptr);
 
 // One launch of a batch: systems whose plans share a kernel instance and a
 // cluster size (2^log2 blocks). plan: the instance, with the block and the

@@ -174,7 +174,7 @@ struct hmc_ctx {
   // the next launch), and the plans of this lattice ([cells per column - 1])
   void* tile_sync = nullptr;
   bool tile_sync_stale = false;
-  hmc::TilePlan tile_plan32[2];
+  hmc::TilePlan tile_plan32[2], tile_plan32_large[2];
   hmc::TilePlan tile_plan64;
   // the same on one thread block cluster (log2 of its blocks; -2: not looked for yet, -1: none)
   int cluster_log2 = -2;

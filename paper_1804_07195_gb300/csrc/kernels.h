@@ -64,10 +64,11 @@ hmc_status set_cg1_shape(hmc_ctx* c, int Ti, int Tj, int Tt, int D);
 
 // Resident-tile FP32 CG (cg_tile.cuh): the whole solve in one cooperative
 // launch from the state k_init0 (or the residual kernel) left in sc, x and r
-// (u: the blocks' exchanged edges), with every vector of the iteration on the
-// chip; false / HMC_ERR_INVALID when the tiles do not fit there.
+// (u: the blocks' exchanged edges; spare: a vector that may be overwritten),
+// with every vector of the iteration on the chip; false / HMC_ERR_INVALID when
+// the tiles do not fit there.
 bool cg32_resident_ok(hmc_ctx* c, const Geo& g);
-hmc_status cg32_resident_launch(hmc_ctx* c, const Geo& g, float2* x, float2* r, float2* u, CGScal* sc);
+hmc_status cg32_resident_launch(hmc_ctx* c, const Geo& g, float2* x, float2* r, float2* u, float2* spare, CGScal* sc);
 // The same on one thread block cluster (small lattices).
 bool cg32_cluster_ok(hmc_ctx* c, const Geo& g);
 hmc_status cg32_cluster_launch(hmc_ctx* c, const Geo& g, float2* x, float2* r, CGScal* sc);

@@ -329,7 +329,7 @@ hmc_status cg_core(hmc_ctx* c, double ms, double sigma, const V2<R>* b, V2<R>* x
       if (cluster)
         HMC_TRY(cg32_cluster_launch(c, g, (float2*)x, (float2*)r, sc));
       else if (resident)
-        HMC_TRY(cg32_resident_launch(c, g, (float2*)x, (float2*)r, (float2*)u, sc));
+        HMC_TRY(cg32_resident_launch(c, g, (float2*)x, (float2*)r, (float2*)u, (float2*)p, sc));
       else
         HMC_TRY(cg32_persist_launch(c, g, (float2*)x, (float2*)r, (float2*)p, (float2*)q, (float2*)u, sc));
       HMC_TRY(read_back(c, sc, sch, sizeof(CGScal)));

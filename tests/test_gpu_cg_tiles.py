@@ -124,3 +124,24 @@ def test_x_in_tensor_memory(shape):
     assert info["iters"] == 4
     # the bound of the other tests, 2e-5 an iteration
     assert rel_max(host(x).astype(np.complex128), ref.x) <= 8e-5
+
+
+@pytest.mark.parametrize("shape,cols", [((106, 106, 64), 2), ((110, 108, 63), 2), ((99, 99, 64), 1), ((50, 146, 113), 2),
+                                        ((117, 75, 70), 1)])
+def test_largest_tiles(shape, cols):
+    """Tiles that leave no room for the table of their padding in shared memory
+    (it lies in global memory): pairs of four and eight slices, single cells,
+    tiles whose slices are no multiple of a column's."""
+    need_gpu()
+    w = W.small(*shape, seed=2700 + sum(shape))
+    ol = OLat.from_params(w.lat)
+    b32 = w.b.astype(np.complex64)
+    ref = osv.cg(lambda v: of.apply_MMdag(ol, w.phi, 0.4, v, 0.3), b32.astype(np.complex128), tol=1e-30, maxit=3)
+    with ctx_for(w.lat) as ctx:
+        ctx.set_cg_variant(7)
+        x, info = ctx.solve_spcg(dev(w.phi), 0.4, dev(b32), sigma=0.3, tol=1e-30, maxit=3, allow_fail=True)
+        prof = ctx.profile_read()["cg_resident_f32"]
+        assert prof["launches"] >= 1 and prof["design"] == (4 if cols == 2 else 0)
+        assert ctx.check_guards() == 0
+    assert info["iters"] == 3
+    assert rel_max(host(x).astype(np.complex128), ref.x) <= 6e-5
