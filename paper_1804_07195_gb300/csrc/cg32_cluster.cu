@@ -45,16 +45,19 @@ static const void* cluster_kernel32(const TilePlan& p) {
   return nullptr;
 }
 
-// us per iteration of a system on a cluster of cs blocks, from the columns of its
-// largest tile. Fitted to measured iterations (with a cluster barrier an exchange, 0.2
-// to 0.5 more than now); it only ranks the choices:
-//   12x12x32 on 1, 2, 4, 8, 16 blocks: 8.8, 4.4, 3.4, 2.9, 3.0
-//   24x24x48 on 8, 16: 6.4, 4.5;  18x18x48 on 4, 8, 16: 6.8, 4.3, 3.9
-//   36x36x48 on 16: 7.2 (over all SMs 5.8);  25x24x48 on 8, 16: 8.2, 6.8
-static double cluster_us(const TilePlan& p, const Geo& g, int cs) {
+// us per iteration of a system on a cluster of 2^k blocks: the cells of its largest
+// tile, and the partials every warp sends to and takes from every block, twice. It
+// only ranks the choices. Fitted to 103 measured plans (5x5x16 to 36x36x48, odd and
+// even n; rms error 7 %, 18 % at most; the fastest cluster's choice costs 0.5 % on
+// average), for instance on 1, 2, 4, 8, 16 blocks (a dash: does not fit):
+//   6x6x16 2.61, 2.36, 2.29, 2.33, 2.42   12x12x32 9.29, 4.47, 3.40, 2.74, 2.59
+//   13x13x32 -, 5.62, 4.04, 3.50, 2.85    18x18x48 -, -, 6.26, 4.11, 3.49
+//   24x24x48 -, -, -, 6.06, 4.23          25x25x48 -, -, -, 12.7, 7.24
+//   36x36x48 -, -, -, -, 6.46 (over all SMs 5.60)
+static double cluster_us(const TilePlan& p, const Geo& g, int k) {
   const double cols = (double)p.J * std::min(p.T, g.nt) * (g.n / p.cw);
-  const double slope = p.cw == 1 ? 1.5e-3 : tile_slices(p.S) <= 2 ? 1.6e-3 : 2.25e-3;
-  return (cs == 16 ? 2.85 : 2.45) + slope * cols + (p.S >= kXInMemory ? 1.2 : 0.0);
+  const double slope = (p.cw == 1 ? 1.35e-3 : 1.95e-3) + (p.S >= kXInMemory ? 1.25e-3 : 0.0);
+  return 2.0 + 0.05 * k + 0.0028 * (p.threads / 32) * (1 << k) + slope * cols;
 }
 
 // Tiles of one system for a cluster of cs blocks (cs a power of two): the split
@@ -131,31 +134,36 @@ static void cluster_waits(const hmc_ctx* c, unsigned* extra, long long* limit) {
   *limit = c->bar_limit > 0 ? std::max(c->bar_limit, 100000LL) : 2000000000LL;
 }
 
-// Whether this GPU can run a cluster of the plan.
-static bool cluster_runs(const hmc_ctx* c, const TilePlan& p, int cs) {
+// How many clusters of the plan this GPU can run at a time with an SM to each block.
+// (Blocks of small tiles can share one, but then take longer: counted that way, 100
+// systems of 4x4 to 8x8 cells take 3.8 ms instead of 3.35.)
+static int cluster_count(const hmc_ctx* c, const TilePlan& p, int cs) {
   const void* k = cluster_kernel32(p);
-  if (!k) return false;
+  if (!k) return 0;
   if (!tile_allow_smem(c, k) ||
       (cs > 8 && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
     cudaGetLastError();
-    return false;
+    return 0;
   }
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr;
-  cluster_config(&cfg, &attr, p, cs, 1, nullptr);
+  TilePlan alone = p;
+  alone.smem = std::max(p.smem, (size_t)120 * 1024);  // more than half of an SM's
+  cluster_config(&cfg, &attr, alone, cs, 1, nullptr);
   int n = 0;
   if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return 0;
   }
-  return n > 0;
+  return n;
 }
 
 static ClusterPlans cluster_plans(const hmc_ctx* c, const Geo& g) {
   ClusterPlans cp;
   for (int k = 0; k < 5; ++k) {
-    if (!plan_cluster(c, g, 1 << k, &cp.p[k]) || !cluster_runs(c, cp.p[k], 1 << k)) cp.p[k].cw = 0;
-    cp.us[k] = cp.p[k].cw ? cluster_us(cp.p[k], g, 1 << k) : 0.0;
+    cp.count[k] = plan_cluster(c, g, 1 << k, &cp.p[k]) ? cluster_count(c, cp.p[k], 1 << k) : 0;
+    if (cp.count[k] < 1) cp.p[k].cw = 0;
+    cp.us[k] = cp.p[k].cw ? cluster_us(cp.p[k], g, k) : 0.0;
   }
   return cp;
 }
@@ -206,10 +214,6 @@ bool cg32_cluster_batch(hmc_ctx* c, const std::vector<Geo>& geos, const std::vec
   if (c->batch_plans.size() > 512) c->batch_plans.clear();
   std::vector<const ClusterPlans*> cp(ns);
   std::vector<int> pick(ns);
-  // SMs that a cluster of 1, 2, 4, 8 or 16 blocks takes of this GPU: larger ones
-  // must lie in one of its groups of SMs and leave some unused (152, 76, 36, 15
-  // and 7 at a time on 152 SMs)
-  const double sms[5] = {1.0, 2.0, 4.2, 10.1, 21.7};
   for (int i = 0; i < ns; ++i) {
     const std::array<int, 3> key{geos[i].n, geos[i].m, geos[i].nt};
     auto it = c->batch_plans.find(key);
@@ -233,7 +237,8 @@ bool cg32_cluster_batch(hmc_ctx* c, const std::vector<Geo>& geos, const std::vec
   }
   std::sort(cand.begin(), cand.end());
   std::vector<int> trial(ns), order(ns);
-  double best = 0.0;
+  std::vector<double> ends, times;
+  std::vector<std::vector<int>> trials;
   const int ncand = (int)cand.size(), tries = std::min(ncand, 32);
   for (int v = 0; v < tries; ++v) {
     const double T = cand[tries == ncand ? v : (size_t)v * (ncand - 1) / (tries - 1)];
@@ -248,7 +253,10 @@ bool cg32_cluster_batch(hmc_ctx* c, const std::vector<Geo>& geos, const std::vec
     std::priority_queue<std::pair<double, double>, std::vector<std::pair<double, double>>, std::greater<>> running;
     double free = c->nsm, now = 0.0, end = 0.0;
     for (int i : order) {
-      const double need = sms[trial[i]];
+      // SMs a cluster takes of this GPU: clusters must lie in one of its groups of SMs
+      // and leave some unused (152, 76, 36, 15 and 7 of 1 to 16 blocks at a time on 152
+      // SMs)
+      const double need = (double)c->nsm / cp[i]->count[trial[i]];
       while (free < need && !running.empty()) {
         now = running.top().first;
         free += running.top().second;
@@ -259,12 +267,20 @@ bool cg32_cluster_batch(hmc_ctx* c, const std::vector<Geo>& geos, const std::vec
       free -= need;
       end = std::max(end, done);
     }
-    // of values that end together the largest T: the least SM time
-    if (v == 0 || end <= 1.01 * best) {
-      best = v == 0 ? end : std::min(best, end);
-      pick = trial;
-    }
+    ends.push_back(end);
+    times.push_back(T);
+    trials.push_back(trial);
   }
+  // Of values that end together the largest T (the least SM time), but the systems'
+  // iterations differ from what is expected: below 0.65 of the end, where there is
+  // one. (ms for 48 systems of 5x5x16 to 19x19x32, 24 of 12x12 to 24x24, 12 of 6x6 to
+  // 24x24, with the largest T, the smallest, and this one: 5.0, 4.3, 4.3; 6.1, 6.3, 6.5;
+  // 8.05, 9.1, 8.05; eight chains 115, 104, 109.)
+  const double best = *std::min_element(ends.begin(), ends.end());
+  int take = -1;
+  for (int v = 0; v < tries; ++v)
+    if (ends[v] <= 1.01 * best && (take < 0 || times[v] <= 0.65 * best)) take = v;
+  pick = trials[take];
   auto time_of = [&](int i) { return time_at(i, pick[i]); };
   // one launch per instance and cluster size, with the largest block and shared
   // memory of its systems; the systems that run longest first
@@ -296,7 +312,7 @@ bool cg32_cluster_batch(hmc_ctx* c, const std::vector<Geo>& geos, const std::vec
     g->plans.push_back(p);
   }
   for (const ClusterGroup& g : *groups)
-    if (!cluster_runs(c, g.plan, 1 << g.log2)) return false;
+    if (cluster_count(c, g.plan, 1 << g.log2) < 1) return false;
   return true;
 }
 

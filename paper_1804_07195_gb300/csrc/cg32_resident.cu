@@ -263,9 +263,10 @@ bool cg32_prefer_cluster(hmc_ctx* c, const Geo& g) {
   const TilePlan* p = pick32(c, g, true);
   if (!p) return true;
   // us per iteration over all SMs: two exchanges through L2, phase latency, work
-  // (measured: 5.6 at 36x36x64, 7.95 at 72x72x64); cluster_us has the cluster's.
-  // The line between them runs near 100,000 sites (measured: 24x24x48 4.5 us on a
-  // cluster, 6.2 over all SMs)
+  // (measured: 5.6 at 36x36x64, 7.95 at 72x72x64; 5.6 to 6.8 below 100,000 sites);
+  // cluster_us has the cluster's. The line between them runs near 70,000 sites
+  // (measured: 24x24x48 4.2 us on a cluster, 5.9 over all SMs; 25x25x48 7.2, 5.7;
+  // 36x36x32 5.6, 5.6; 30x30x64 6.7, 5.6)
   const double cols = (double)p->J * std::min(p->T, g.nt) * (g.n / p->cw) * (p->cw == 2 ? 1.0 : 0.75);
   return c->cluster_us < 5.2 + 2.6e-3 * cols;
 }

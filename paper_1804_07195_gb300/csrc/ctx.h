@@ -121,9 +121,10 @@ struct TilePlan {
 };
 
 // Plans of one lattice on a cluster of 1, 2, 4, 8 or 16 blocks (cw <= 0: none),
-// with the estimated us per iteration.
+// with the estimated us per iteration and how many run at a time.
 struct ClusterPlans {
   TilePlan p[5];
+  int count[5];
   double us[5];
 };
 
