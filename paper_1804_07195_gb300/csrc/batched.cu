@@ -207,8 +207,8 @@ struct BPhase<float> {
   }
 };
 
-// x = 0, r = p = b; |b|^2; state init with thresh = tol2[s] |b|^2 (inactive
-// systems are marked done).
+// x = 0, r = p = b (p may be NULL); |b|^2; state init with thresh = tol2[s] |b|^2
+// (inactive systems are marked done).
 template <typename R>
 __global__ void kb_init(const BSys* __restrict__ sys, const int* __restrict__ bsys, BState* bst,
                         const double* __restrict__ tol2, const V2<R>* __restrict__ b, V2<R>* __restrict__ x,
@@ -221,7 +221,7 @@ __global__ void kb_init(const BSys* __restrict__ sys, const int* __restrict__ bs
     Cx<R> bk = ld<R>(b, i);
     st(x, i, Cx<R>{(R)0, (R)0});
     st(r, i, bk);
-    st(p, i, bk);
+    if (p != nullptr) st(p, i, bk);
     acc[0] += (double)norm2(bk);
   }
   double tot[1];
@@ -954,9 +954,6 @@ extern "C" hmc_status hmc_solve_batched(hmc_ctx* c, int nsys, const hmc_system* 
       HMC_TRY(bmalloc(c, w, (void**)&w.u, sizeof(double2) * Nt));
       HMC_TRY(bmalloc(c, w, (void**)&w.r32, sizeof(float2) * Nt));
       HMC_TRY(bmalloc(c, w, (void**)&w.e32, sizeof(float2) * Nt));
-      HMC_TRY(bmalloc(c, w, (void**)&w.p32v, sizeof(float2) * Nt));
-      HMC_TRY(bmalloc(c, w, (void**)&w.q32v, sizeof(float2) * Nt));
-      HMC_TRY(bmalloc(c, w, (void**)&w.u32, sizeof(float2) * Nt));
       HMC_TRY(bmalloc(c, w, (void**)&w.rr32, sizeof(float2) * Nt));
     }
     // FP32 CG: every system on a cluster of its own where all of them fit one,
@@ -974,6 +971,11 @@ extern "C" hmc_status hmc_solve_batched(hmc_ctx* c, int nsys, const hmc_system* 
       w.clusters = cg32_cluster_batch(c, geos, its, &w.groups);
     }
     if (mixed) c->batch_clusters = w.clusters;
+    if (mixed && !w.clusters) {
+      HMC_TRY(bmalloc(c, w, (void**)&w.p32v, sizeof(float2) * Nt));
+      HMC_TRY(bmalloc(c, w, (void**)&w.q32v, sizeof(float2) * Nt));
+      HMC_TRY(bmalloc(c, w, (void**)&w.u32, sizeof(float2) * Nt));
+    }
     if (w.clusters) {
       HMC_TRY(bmalloc(c, w, (void**)&w.tsys, sizeof(TileSys) * nsys));
       std::vector<TileSys> h;

@@ -146,6 +146,30 @@ def test_fp32_scalars_of_a_batch_keep_all_bits(where):
         assert np.array_equal(host(s["x"]), x)
 
 
+def test_a_batch_on_clusters_keeps_no_direction_vectors():
+    """Device memory a mixed batch adds to its context, per site: E 16, phi 4,
+    x, b, r and u 16 each, r32, e32 and the residual 8 each, 108 in all; the
+    vectors of the other designs (24 more) are not among them."""
+    need_gpu()
+    import paper_1804_07195_gb300 as hmc
+
+    def batch(lat, count):
+        zero = torch.zeros(lat.nsites, dtype=torch.float64, device="cuda")
+        return [{"lattice": lat, "phi": zero, "ms": 2.0, "b": torch.ones(lat.nsites, dtype=torch.complex128, device="cuda"),
+                 "x": torch.empty(lat.nsites, dtype=torch.complex128, device="cuda")} for _ in range(count)]
+    lat = hmc.Lattice(36, 36, 48, 1.0, 3.0, 6.0)
+    small, large = batch(hmc.Lattice(6, 6, 16, 1.0, 3.0, 6.0), 1), batch(lat, 24)
+    with hmc.Context(lat) as ctx:
+        ctx.solve_batched(small, mixed=True)
+        ctx.solve_batched(batch(lat, 1), mixed=True)  # loads its kernels
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        ctx.solve_batched(large, mixed=True)
+        assert ctx.batched_variant() == 2 and ctx.check_guards() == 0
+        used = before - torch.cuda.mem_get_info()[0]
+    assert used <= 108 * 24 * lat.nsites + 20 * (2 << 20)  # and the allocator's 2 MB steps
+
+
 @pytest.mark.parametrize("mixed", [0, 1])
 def test_uneven_small_batch(mixed):
     need_gpu()
