@@ -430,7 +430,9 @@ typedef struct {
                            per tile of `threads` cells; -(1000 + tt): the
                            marching kernels, tt slices per block;
                            cg_resident_f32: blocks of the last launch,
-                           negative on a cluster */
+                           negative on a cluster; batch_cg_graph_*: blocks of
+                           the last persistent launch, 0 after the graph loop,
+                           minus the number of launches on clusters */
   int design;           /* FP32 CG kernels: 0 grid-stride (one cell per thread),
                            1 tiled, 2 marching, 4 grid-stride with two cells
                            per thread */

@@ -697,6 +697,7 @@ static hmc_status batched_cg_persist(hmc_ctx* c, BatchWs& w, cudaStream_t s, V2<
   double bytes = 0.0;
   for (int i = 0; i < w.nsys; ++i) bytes += (double)w.st_host[i].cg.iter * w.hsys[i].g.N * (sizeof(R) == 8 ? 192.0 : 88.0);
   c->prof.bytes[kid] += bytes;
+  c->shape[kid].waves = grid;
   *ran = true;
   return HMC_OK;
 }
@@ -719,6 +720,7 @@ static hmc_status batched_cg(hmc_ctx* c, BatchWs& w, cudaStream_t s, const V2<R>
       const hmc_status st = cg32_cluster_batch_launch(c, w.groups, w.tsys);
       prof_end(c, K_BATCH_CG32, a);
       c->prof.launches[K_BATCH_CG32]--;  // prof_begin counted one more
+      c->shape[K_BATCH_CG32].waves = -(int)w.groups.size();
       HMC_TRY(st);
       HMC_CUDA(c, cudaMemcpyAsync(w.st_host, w.st, sizeof(BState) * w.nsys, cudaMemcpyDeviceToHost, s));
       HMC_CUDA(c, cudaStreamSynchronize(s));
@@ -787,6 +789,7 @@ template <typename R>
 static hmc_status batched_cg_loop(hmc_ctx* c, BatchWs& w, cudaStream_t s, V2<R>* x, V2<R>* r, V2<R>* p, V2<R>* q,
                                   V2<R>* u, int maxit, int pre_done, int chunk, int kid, double bytes_iter,
                                   long long* iters_launched) {
+  c->shape[kid].waves = 0;
   // One graph launch for the whole batched solve: a device-side while loop
   // repeats the captured chunk until every running system is done (counted
   // in ndone) or the trip bound maxit / chunk + 2 is reached.

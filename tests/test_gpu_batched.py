@@ -36,7 +36,7 @@ def check(instances, xs, infos, tol):
         assert abs(info["true_rel_res"] - rel) <= 1e-3 * tol + 1e-14
 
 
-def run_batch_variant(instances, mixed, variant, tol=1e-10):
+def run_batch_variant(instances, mixed, variant, tol=1e-10, where=0):
     import paper_1804_07195_gb300 as hmc
     systems = []
     for w, ms, sigma, b in instances:
@@ -46,24 +46,27 @@ def run_batch_variant(instances, mixed, variant, tol=1e-10):
                         "tol": tol, "maxit": 100000})
     with ctx_for(instances[0][0].lat) as ctx:
         ctx.set_batched_variant(variant)
+        ctx.set_tile_test(where)
         infos = ctx.solve_batched(systems, mixed=mixed)
-        used = ctx.batched_variant()
+        used = ctx.batched_variant(), ctx.profile_read()["batch_cg_graph_f32"]["waves"]
     return [host(s["x"]) for s in systems], infos, used
 
 
-@pytest.mark.parametrize("variant", [1, 2])
-def test_fp32_batched_designs(variant):
-    """The two designs of the batched FP32 CG (graph loop of per-iteration
-    kernels; one persistent cooperative launch with grid barriers) under FP64
-    defect correction: every system's true residual against the oracle."""
+@pytest.mark.parametrize("variant,where", [(1, 0), (2, 0), (2, 1)])
+def test_fp32_batched_designs(variant, where):
+    """The designs of the batched FP32 CG (graph loop of per-iteration kernels;
+    thread block clusters; one persistent cooperative launch with grid barriers)
+    under FP64 defect correction: every system's true residual against the
+    oracle."""
     need_gpu()
     shapes = [(1, 1, 2), (3, 3, 8), (6, 6, 16), (2, 5, 4), (12, 12, 16), (4, 3, 10), (18, 18, 32)]
     inst = []
     for k, sh in enumerate(shapes):
         w = W.small(*sh, seed=320 + k, U=3.0, beta=6.0)
         inst.append((w, [0.0, 0.1, 0.5, 2.0][k % 4], [0.0, 0.0, 0.04][k % 3], w.b))
-    xs, infos, used = run_batch_variant(inst, 1, variant)
+    xs, infos, (used, blocks) = run_batch_variant(inst, 1, variant, where=where)
     assert used == variant
+    assert blocks == 0 if variant == 1 else (blocks < 0) == (where == 0)
     check(inst, xs, infos, 1e-10)
 
 

@@ -1,7 +1,7 @@
-"""The resident-tile FP32 CG (variant 7: one cooperative launch per solve, p
-and u = M^dagger p of every block's tile in shared memory, the neighbouring
-tiles' edge rows and slices exchanged through memory between grid barriers)
-against the oracle's textbook CG (Section 3), with one cell per thread (odd
+"""The resident-tile FP32 CG (variant 7: one launch per solve, p and u =
+M^dagger p of every block's tile in shared memory, the neighbouring tiles' edge
+rows and slices exchanged through memory between the blocks of a cooperative
+launch, or through the shared memory of a thread block cluster) against the oracle's textbook CG (Section 3), with one cell per thread (odd
 n) and two (even n): the same CG step, so x after k
 iterations matches the oracle's FP64 CG after k iterations to FP32
 rounding, on lattices with n or m of 1 to 3 (every wrap: a tile's padding
@@ -28,7 +28,8 @@ SHAPES = [(1, 1, 4), (2, 1, 4), (1, 3, 5), (3, 3, 8), (2, 5, 3), (6, 6, 16), (7,
 
 @pytest.mark.parametrize("shape", SHAPES)
 @pytest.mark.parametrize("ms,sigma", [(0.3, 0.0), (0.1, 0.2)])
-def test_resident_iterates_equal_cg(shape, ms, sigma):
+@pytest.mark.parametrize("where", [1, 2])  # over all SMs, on one cluster
+def test_resident_iterates_equal_cg(shape, ms, sigma, where):
     need_gpu()
     w = W.small(*shape, seed=1600 + sum(shape))
     ol = OLat.from_params(w.lat)
@@ -37,13 +38,14 @@ def test_resident_iterates_equal_cg(shape, ms, sigma):
     kmax = max(1, min(5, w.lat.nsites // 4))
     with ctx_for(w.lat) as ctx:
         ctx.set_cg_variant(7)
+        ctx.set_tile_test(where)
         for k in sorted({1, 2, kmax}):
             x, info = ctx.solve_spcg(dev(w.phi), ms, dev(b32), sigma=sigma, tol=1e-30, maxit=k, allow_fail=True)
             assert info["iters"] == k, (shape, k, info)
             ref = osv.cg(A, b32.astype(np.complex128), tol=1e-30, maxit=k)
             assert rel_max(host(x).astype(np.complex128), ref.x) <= 2e-5 * k, (shape, k)
         st = ctx.profile_read()["cg_resident_f32"]
-        assert st["launches"] >= 2
+        assert st["launches"] >= 2 and (st["waves"] < 0) == (where == 2)
         # two cells per thread (16-byte pairs) where n is even
         assert st["design"] == (4 if shape[0] % 2 == 0 else 0)
         # the roofline's algorithmic bytes: 96 B per site for exactly the
@@ -92,6 +94,7 @@ def test_resident_barrier_wait_times_out_and_context_survives():
     b32 = dev(w.b.astype(np.complex64))
     with ctx_for(w.lat) as ctx:
         ctx.set_cg_variant(7)
+        ctx.set_tile_test(1)  # (clusters: test_gpu_tile_waits)
         ctx.set_wait_test(1, 2_000_000)
         t = time.perf_counter()
         with pytest.raises(hmc.HMCError) as e:

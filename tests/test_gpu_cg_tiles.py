@@ -85,9 +85,8 @@ def test_batched_clusters(shapes):
 @pytest.mark.parametrize("shape", [(1, 1, 4), (2, 5, 3), (7, 5, 9), (36, 35, 40), (36, 36, 64), (51, 33, 61),
                                    (72, 40, 64), (33, 120, 64)])
 def test_fp64_tiles(shape):
-    """The FP64 CG on resident tiles (the context's tuner runs it beside the
-    three-kernel iteration and keeps the faster): x after two iterations and
-    from a starting guess against the oracle's CG."""
+    """The FP64 CG on resident tiles, which runs wherever the tiles fit: x after
+    two iterations and from a starting guess against the oracle's CG."""
     need_gpu()
     w = W.small(*shape, seed=2000 + sum(shape))
     ol = OLat.from_params(w.lat)

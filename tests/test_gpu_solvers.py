@@ -9,7 +9,7 @@ from oracle import fermion as of
 from oracle import solvers as osv
 from oracle.lattice import Lattice as OLat
 
-from gpu_util import ctx_for, dev, host, need_gpu, torch
+from gpu_util import ctx_for, dev, host, need_gpu, rel_max, torch
 
 pytestmark = pytest.mark.gpu
 
@@ -186,18 +186,22 @@ def test_fp32_cg_kernel_variants(variant, name, ms, sigma, bound):
 
 
 def test_solves_run_as_one_graph_launch_with_a_device_loop():
-    """After a solve the context reports the device-side loop graph (one graph
-    launch per CG solve), and a second solve through the cached loop graph gives
-    the same result bit for bit (FP64 CG is deterministic)."""
+    """After a solve by three kernels an iteration the context reports the
+    device-side loop graph (one graph launch per CG solve), and a second solve
+    through the cached loop graph gives the same result bit for bit (FP64 CG is
+    deterministic)."""
     need_gpu()
     w = W.workload("L6x6x16")
     with ctx_for(w.lat) as ctx:
+        ctx.set_tile_test(3)  # small lattices would run on resident tiles, without a graph
         x1, i1 = ctx.solve_cg(dev(w.phi), 0.3, dev(w.b), tol=1e-10)
         assert ctx.graph_mode() == 2
         x2, i2 = ctx.solve_cg(dev(w.phi), 0.3, dev(w.b), tol=1e-10)
         ctx.set_graph_mode(1)  # chunks with host checks: the same iterations
         assert ctx.graph_mode() == 1
         x3, i3 = ctx.solve_cg(dev(w.phi), 0.3, dev(w.b), tol=1e-10)
+        prof = ctx.profile_read()
+        assert prof["cg_resident_f64"]["launches"] == 0 and prof["cg_Mdag_f64"]["launches"] >= 3 * i1["iters"]
     assert i1["iters"] == i2["iters"] == i3["iters"]
     assert np.array_equal(host(x1), host(x2)) and np.array_equal(host(x1), host(x3))
 
@@ -260,3 +264,27 @@ def test_arnoldi_steps_against_numpy(shape, steps):
     # cond(H) < 10: the normal equations and one pass of Gram-Schmidt lose its square,
     # 100 x 2.2e-16 x 16 steps = 4e-13; five times that
     assert np.linalg.norm(host(x) - ref) <= 2e-12 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("shape", [(3, 3, 8), (7, 5, 9), (12, 12, 32), (35, 12, 21)])
+@pytest.mark.parametrize("ms,sigma", [(0.0, 0.0), (0.3, 0.0), (0.0, 0.2), (0.1, 0.2)])
+def test_fp64_three_kernel_iterates(shape, ms, sigma):
+    """The FP64 CG of three kernels an iteration (lattices whose tiles do not fit
+    the chip), with an instance for each of mass and shift zero or not: x after
+    a few iterations, from zero and from a guess, against the oracle's CG."""
+    need_gpu()
+    w = W.small(*shape, seed=2150 + sum(shape))
+    ol = OLat.from_params(w.lat)
+    A = lambda v: of.apply_MMdag(ol, w.phi, ms, v, sigma)
+    with ctx_for(w.lat) as ctx:
+        ctx.set_tile_test(3)
+        for x0 in (None, 0.1 * w.b):
+            ref = osv.cg(A, w.b if x0 is None else w.b - A(x0), tol=1e-30, maxit=4).x
+            if x0 is not None:
+                ref = x0 + ref
+            x, info = ctx.solve_cg(dev(w.phi), ms, dev(w.b), x=None if x0 is None else dev(x0), sigma=sigma, tol=1e-30,
+                                   maxit=4, allow_fail=True)
+            assert info["iters"] == 4
+            assert rel_max(host(x), ref) <= 2e-13  # 5e-14 an iteration, as for the tiles
+        prof = ctx.profile_read()
+        assert prof["cg_resident_f64"]["launches"] == 0 and prof["cg_Mdag_f64"]["launches"] >= 8
