@@ -42,7 +42,7 @@
 //
 // Every sum is formed in a fixed order that is the same in every block, so
 // all blocks of a group hold the same scalars and leave together. FP32 sums
-// are float-float pairs, FP64 sums doubles, up to alpha, beta and the stopping test.
+// are float-float pairs, FP64 sums doubles.
 //
 // What bounds an FP32 iteration of a cooperative launch (us, 2070 MHz; in
 // brackets the design before it, which read r, x and phi from L2 row by row in
@@ -279,24 +279,6 @@ struct Red<float> {
     return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
   }
   static __device__ __forceinline__ float value(T a) { return a.x + a.y; }
-  static __device__ __forceinline__ T of64(double a) {
-    const float h = (float)a;
-    return make_float2(h, (float)(a - (double)h));
-  }
-  static __device__ __forceinline__ double to64(T a) { return (double)a.x + (double)a.y; }
-  static __device__ __forceinline__ bool le(T a, T b) { return (a.x - b.x) + (a.y - b.y) <= 0.f; }
-  // a / b (b > 0) from all bits of both, rounded once: the approximate quotient,
-  // off by 2^-22, and the exact rest over b. rc: about 1 / b, or 0 outside the range
-  // of that, and then the quotient of the high parts.
-  static __device__ __forceinline__ float over(T b) {
-    return b.x > 1e-30f && b.x < 1e30f ? __fdividef(1.f, b.x) : 0.f;
-  }
-  static __device__ __forceinline__ float ratio(T a, T b, float rc) {
-    if (rc == 0.f) return a.x / b.x;
-    const float q = a.x * rc;
-    return fmaf(fmaf(-q, b.x, a.x) + fmaf(-q, b.y, a.y), rc, q);
-  }
-  static __device__ __forceinline__ float ratio(T a, T b) { return ratio(a, b, over(b)); }
 };
 template <>
 struct Red<double> {
@@ -306,11 +288,46 @@ struct Red<double> {
   static __device__ __forceinline__ T add(T a, T b) { return a + b; }
   static __device__ __forceinline__ T shfl(T a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
   static __device__ __forceinline__ double value(T a) { return a; }
-  static __device__ __forceinline__ T of64(double a) { return a; }
-  static __device__ __forceinline__ double to64(T a) { return a; }
-  static __device__ __forceinline__ bool le(T a, T b) { return a <= b; }
-  static __device__ __forceinline__ int over(T) { return 0; }
-  static __device__ __forceinline__ double ratio(T a, T b, int = 0) { return a / b; }
+};
+
+// The scalars of a solve made of the sums: of type R, or (WIDE, FP32) with all bits of
+// the sums, alpha and beta rounded once from these. Clusters hold them wide, as the
+// other batched kernels hold FP64 ones; over all SMs they are FP32, as in the other
+// FP32 CG kernels of a single system (a trajectory at 102x102x64 158.6 ms, wide 162.9).
+template <typename R, bool WIDE>
+struct Scalars {
+  using S = R;
+  static __device__ __forceinline__ S of64(double a) { return (R)a; }
+  static __device__ __forceinline__ double to64(S a) { return (double)a; }
+  static __device__ __forceinline__ S of(typename Red<R>::T a) { return Red<R>::value(a); }
+  static __device__ __forceinline__ R value(S a) { return a; }
+  static __device__ __forceinline__ bool le(S a, S b) { return a <= b; }
+  static __device__ __forceinline__ int over(S) { return 0; }
+  static __device__ __forceinline__ R ratio(S a, S b, int = 0) { return a / b; }
+};
+template <>
+struct Scalars<float, true> {
+  using S = float2;
+  static __device__ __forceinline__ S of64(double a) {
+    const float h = (float)a;
+    return make_float2(h, (float)(a - (double)h));
+  }
+  static __device__ __forceinline__ double to64(S a) { return (double)a.x + (double)a.y; }
+  static __device__ __forceinline__ S of(float2 a) { return a; }
+  static __device__ __forceinline__ float value(S a) { return a.x + a.y; }
+  static __device__ __forceinline__ bool le(S a, S b) { return (a.x - b.x) + (a.y - b.y) <= 0.f; }
+  // about 1 / b (b > 0), or 0 outside the range of that
+  static __device__ __forceinline__ float over(S b) {
+    return b.x > 1e-30f && b.x < 1e30f ? __fdividef(1.f, b.x) : 0.f;
+  }
+  // a / b: the approximate quotient, off by 2^-22, and the exact rest over b; where rc
+  // is 0 the quotient of the high parts
+  static __device__ __forceinline__ float ratio(S a, S b, float rc) {
+    if (rc == 0.f) return a.x / b.x;
+    const float q = a.x * rc;
+    return fmaf(fmaf(-q, b.x, a.x) + fmaf(-q, b.y, a.y), rc, q);
+  }
+  static __device__ __forceinline__ float ratio(S a, S b) { return ratio(a, b, over(b)); }
 };
 template <typename R>
 __device__ __forceinline__ typename Red<R>::T warp_sum(typename Red<R>::T v) {
@@ -674,13 +691,14 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
     TtP = min(TN, nt - tb * TN);
   }
 
-  // |r|^2 (of iteration i in s_rr[i & 1]) and <p, A p> keep all bits of their sums;
-  // alpha and beta are rounded to R from these. Kept in shared memory, as registers
-  // are short: by thread 0, read behind a barrier (CL) or by thread 0 alone.
+  // |r|^2 (of iteration i in s_rr[i & 1]), <p, A p> and the threshold are kept in shared
+  // memory, as registers are short: by thread 0, read behind a barrier (CL) or by
+  // thread 0 alone.
+  using SC = Scalars<R, CL>;
   R dm, sigma;
   TileScal<R>::load(ts.sc, dm, sigma);
-  __shared__ T s_rr[2], s_pap, s_thresh;
-  T rr = RT::of64(ts.sc->rr), thresh = RT::of64(ts.sc->thresh);
+  __shared__ typename SC::S s_rr[2], s_pap, s_thresh;
+  typename SC::S rr = SC::of64(ts.sc->rr), thresh = SC::of64(ts.sc->thresh);
   const L ldm = LN::set(dm), ldk = LN::set(geo_dk(ts.g, R(0))), lndk = LN::set(-geo_dk(ts.g, R(0)));
   int iter = ts.sc->iter, done = ts.sc->done;
   const int maxit = ts.sc->maxit;
@@ -688,7 +706,7 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
   bool first = true;
   if (tid == 0) {
     s_rr[iter & 1] = rr;
-    s_pap = RT::zero();
+    s_pap = SC::of64(0.0);
     s_thresh = thresh;
   }
   // exchanges so far; CL = false: its parity is the arrival word's top bit
@@ -904,9 +922,9 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
   for (;;) {
     if (CL || tid == 0) {
       if (!done) {
-        if (!isfinite(RT::value(rr)))
+        if (!isfinite(SC::value(rr)))
           done = CG_BREAKDOWN;
-        else if (RT::le(rr, thresh))
+        else if (SC::le(rr, thresh))
           done = CG_CONVERGED;
         else if (iter >= maxit)
           done = CG_MAXIT;
@@ -1002,10 +1020,10 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
     }
     if (CL || tid == 0) {
       if constexpr (!CL) rr = s_rr[iter & 1];
-      if (!ok) tot = RT::zero();
-      const bool bad = !(RT::value(tot) > R(0)) || !isfinite(RT::value(tot));
-      alpha = bad ? R(0) : RT::ratio(rr, tot);
-      if (tid == 0) s_pap = tot;
+      const typename SC::S pap = ok ? SC::of(tot) : SC::of64(0.0);
+      const bool bad = !(SC::value(pap) > R(0)) || !isfinite(SC::value(pap));
+      alpha = bad ? R(0) : SC::ratio(rr, pap);
+      if (tid == 0) s_pap = pap;
       if (bad) done = ok ? CG_BREAKDOWN : CG_TIMEOUT;
     }
     R fal = alpha;
@@ -1066,11 +1084,11 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
     // the neighbours' r waits in the padding of u, which nothing reads until the
     // next exchange has refilled it (the block's barrier in `exchange` orders
     // the reads of u above before these writes)
-    decltype(RT::over(rr)) over{};
+    decltype(SC::over(rr)) over{};
     if constexpr (CL) {
       rr = s_rr[iter & 1];
       thresh = s_thresh;
-      over = RT::over(rr);
+      over = SC::over(rr);
     }
     ok = exchange(total(accr),
                   [&] { fetch_padding(rg, true); }, &tot);
@@ -1078,14 +1096,12 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
       if constexpr (!CL) {
         rr = s_rr[iter & 1];
         thresh = s_thresh;
-        over = RT::over(rr);
+        over = SC::over(rr);
       }
-      if (!ok) {
-        tot = rr;
-        done = CG_TIMEOUT;
-      }
-      beta = RT::ratio(tot, rr, over);
-      rr = tot;
+      const typename SC::S now = ok ? SC::of(tot) : rr;
+      if (!ok) done = CG_TIMEOUT;
+      beta = SC::ratio(now, rr, over);
+      rr = now;
       if (tid == 0) s_rr[(iter + 1) & 1] = rr;
     }
     ++iter;
@@ -1127,9 +1143,9 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
   if (tid != 0) return;
   CGScal* sc = ts.sc;
   if (tile == 0) {
-    sc->rr = sc->rr_cur = RT::to64(s_rr[iter & 1]);
+    sc->rr = sc->rr_cur = SC::to64(s_rr[iter & 1]);
     sc->rr32 = sc->rr_cur32 = (float)sc->rr;
-    sc->pAp = RT::to64(s_pap);
+    sc->pAp = SC::to64(s_pap);
     sc->alpha = alpha;
     sc->beta = beta;
     sc->iter = iter;
