@@ -419,8 +419,8 @@ def main():
         roofline["note"] = ("one launch runs a whole FP32 CG solve; its algorithmic bytes are 96 B per site and "
                             "iteration (the CG step's operator with its dot, x and r updates with the norm, p "
                             "update, complex64) times the iterations the solve ran, although p and M^dagger p "
-                            "stay in shared memory and r, x in L2 (1.33M sites: the working set fits the 126 MB "
-                            "L2), hence a fraction near or above 1 of the copy peak; 'traffic' is the DRAM bytes "
+                            "stay in shared memory, r in registers and x in tensor memory (phi is read from L2), "
+                            "hence a fraction near or above 1 of the copy peak; 'traffic' is the DRAM bytes "
                             "of one launch under ncu (one 60-iteration solve on this lattice, caches flushed "
                             "first): its cold first reads of r, x, b and phi and the final writes, which do not "
                             "grow with the iterations a launch runs, so far below the algorithmic bytes")
@@ -523,8 +523,9 @@ def main():
                                  else "k_cg32_resident"], "bytes_per_site": 96.0, "sites": N,
                      "us_per_iteration": t_res * 1e6, "achieved": 96.0 * N / t_res / 1e9, "peak": hbm,
                      "unit": "GB/s", "frac": 96.0 * N / t_res / 1e9 / hbm,
-                     "method": "300 FP32 CG iterations in one launch, CUDA events around the solve; the working "
-                               "set is L2-resident (p and M^dagger p in shared memory)"}
+                     "method": "300 FP32 CG iterations in one launch, CUDA events around the solve; the vectors "
+                               "stay on the chip (p and M^dagger p in shared memory, r in registers, x in tensor "
+                               "memory), phi in L2"}
     solve["speedup_mixed_vs_fp64"] = solve["fp64_cg"]["ms"] / solve["mixed_fgmres"]["ms"]
     solve["workload"] = "102x102x64 lattice, m_s=0, phi of the step, b = rho_0, true residual 1e-10"
     solve["fgmres_a"] = args.fgmres_a
@@ -1103,8 +1104,9 @@ FUSED_STREAM_TILE = (28, 14, 22, 2, 1)
 # the translation units of the FP32 CG kernels whose DRAM traffic
 # profiles/traffic.json records, and everything they include
 PAIR_SOURCES = ("paper_1804_07195_gb300/csrc/kernels.cu", "paper_1804_07195_gb300/csrc/cg32_fused.cu",
-                "paper_1804_07195_gb300/csrc/cg32_resident.cu",
-                "paper_1804_07195_gb300/csrc/kernels.h", "paper_1804_07195_gb300/csrc/ctx.h",
+                "paper_1804_07195_gb300/csrc/cg32_resident.cu", "paper_1804_07195_gb300/csrc/cg_tile.cuh",
+                "paper_1804_07195_gb300/csrc/cg_tile.h", "paper_1804_07195_gb300/csrc/kernels.h",
+                "paper_1804_07195_gb300/csrc/ctx.h", "paper_1804_07195_gb300/csrc/phase.cuh",
                 "paper_1804_07195_gb300/csrc/common.cuh", "paper_1804_07195_gb300/csrc/operator.cuh",
                 "paper_1804_07195_gb300/csrc/launch.cuh", "include/hmc.h")
 

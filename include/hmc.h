@@ -325,7 +325,7 @@ hmc_status hmc_md_trajectory_batched(hmc_ctx* ctx, int nchains, const hmc_chain*
  * and time slices) in shared memory, r and x in registers (x of large tiles in
  * tensor memory): a cooperative launch over all SMs, whose blocks exchange
  * their tiles' edges through memory between grid barriers (bounded waits, as
- * for the persistent kernel), or on lattices of up to about 100,000 sites one
+ * for the persistent kernel), or on small lattices (up to about 80,000 sites) one
  * thread block cluster, which exchanges them through its shared memory.
  * variant: 0 = let the autotuner choose among all of
  * them (default), 1 = grid-stride with one cell per thread, 2 = tiled only,

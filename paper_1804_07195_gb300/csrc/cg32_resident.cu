@@ -13,12 +13,12 @@ namespace hmc {
 template <int S>
 __global__ void __launch_bounds__(tile_max_threads<float, 1, S>(), 1) k_cg32_resident(TileSys ts, GridSync gs) {
   extern __shared__ float4 s_tile[];
-  cg_tile_solve<float, 1, S, false, tile_array_stride<false>()>(ts, gs, blockIdx.x, (char*)s_tile);
+  cg_tile_solve<float, 1, S, false, kTileStride>(ts, gs, blockIdx.x, (char*)s_tile);
 }
 template <int S>
 __global__ void __launch_bounds__(tile_max_threads<float, 2, S>(), 1) k_cg32_resident2(TileSys ts, GridSync gs) {
   extern __shared__ float4 s_tile[];
-  cg_tile_solve<float, 2, S, false, tile_array_stride<false>()>(ts, gs, blockIdx.x, (char*)s_tile);
+  cg_tile_solve<float, 2, S, false, kTileStride>(ts, gs, blockIdx.x, (char*)s_tile);
 }
 
 // Lattices whose tiles leave no room for the padding's table: arrays up to the whole
@@ -68,7 +68,7 @@ bool tile_plan_grid(const hmc_ctx* c, const Geo& g, int cw, int real, const int*
                     TilePlan* out) {
   if (g.n % cw) return false;
   const size_t cap = smem_cap(c, real == 8 ? 7168 : 2048);  // static arrays and the driver's 1 KB
-  constexpr size_t AS = tile_array_stride<false>();
+  constexpr size_t AS = kTileStride;
   const int nq = g.n / cw;
   bool found = false;
   double best = 0.0;

@@ -9,7 +9,7 @@ namespace hmc {
 template <int S>
 __global__ void __launch_bounds__(tile_max_threads<double, 1, S>(), 1) k_cg64_resident(TileSys ts, GridSync gs) {
   extern __shared__ float4 s_tile[];
-  cg_tile_solve<double, 1, S, false, tile_array_stride<false>()>(ts, gs, blockIdx.x, (char*)s_tile);
+  cg_tile_solve<double, 1, S, false, kTileStride>(ts, gs, blockIdx.x, (char*)s_tile);
 }
 
 static const int kSlices64[] = {1, 2, 4 + kXInMemory, 0};

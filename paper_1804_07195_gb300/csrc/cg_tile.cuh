@@ -37,8 +37,8 @@
 // other blocks' shared memory (st.async), each store reporting its bytes to a
 // barrier word of the block it goes to; a block goes on when all bytes due to it
 // have arrived. (us per iteration, with a cluster barrier, which waits for every
-// block's stores and for every block, in brackets: 12x12x32 2.70 (2.89), 13x13x32 2.75
-// (3.31), 18x18x32 3.14 (3.53), 24x24x48 4.32 (4.53).) These waits are bounded too.
+// block's stores and for every block, in brackets: 12x12x32 2.61 (2.89), 13x13x32 2.85
+// (3.31), 18x18x32 3.19 (3.53), 24x24x48 4.27 (4.53).) These waits are bounded too.
 //
 // Every sum is formed in a fixed order that is the same in every block, so
 // all blocks of a group hold the same scalars and leave together. FP32 sums
@@ -47,8 +47,8 @@
 // What bounds an FP32 iteration of a cooperative launch (us, 2070 MHz; in
 // brackets the design before it, which read r, x and phi from L2 row by row in
 // both halves and published p as well):
-//   6x6x16 6.4 (9.0)   12x12x32 6.8 (8.6)   36x36x64 5.5 (7.5)
-//   51x51x64 7.15 (11.6)   72x72x64 7.9 (11.8)   90x90x64 10.2   102x102x64 11.5 (16.2)
+//   6x6x16 6.4 (9.0)   12x12x32 6.8 (8.6)   36x36x64 5.7 (7.5)
+//   51x51x64 7.1 (11.6)   72x72x64 7.9 (11.8)   90x90x64 9.9   102x102x64 11.3 (16.2)
 // The two exchanges take about 2 us each (arrival and poll of one L2 word 1.4,
 // the gather or the edges 0.5), whatever the lattice. The rest is, at
 // 102x102x64, shared memory (4.3 us of wavefronts), instruction issue (4.1) and
@@ -453,11 +453,8 @@ __device__ __forceinline__ bool bar_try(unsigned bar, unsigned parity) {
 }
 
 // Bytes from one of the four padded arrays to the next: constant, so that it is
-// an immediate of every access.
-template <bool CL>
-constexpr int tile_array_stride() {
-  return CL ? 44 * 1024 : 52 * 1024;
-}
+// an immediate of every access (over all SMs; clusters have their own).
+constexpr int kTileStride = 52 * 1024;
 
 template <typename R>
 struct TileScal;

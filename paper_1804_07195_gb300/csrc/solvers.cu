@@ -258,9 +258,11 @@ hmc_status cg_core(hmc_ctx* c, double ms, double sigma, const V2<R>* b, V2<R>* x
   const Geo& g = c->geo;
   // FP64 solves take the resident tiles wherever they fit (a capture excepted),
   // without timing: they were the faster at every size
-  // (us per iteration against the three kernels: 3x3x8 11.2 / 15.2, 24x24x48 11.4 /
-  // 19.2, 36x36x64 18.6 / 27.4, 51x51x64 32.6 / 34.3, 64x64x64 40.3 / 41.5; with
-  // eight slices a column, 66x66x64, they lost, 50.1 / 41.8, and have no instance)
+  // (us per iteration against the three kernels: 12x12x32 10.2 / 14.2, 24x24x48 11.0 /
+  // 17.5, 36x36x64 17.8 / 26.1, 51x51x64 29.1 / 32.7, 64x64x64 38.2 / 41.3; largest
+  // tiles well above the mean, 59x43x88 36.7 / 39.0, 90x40x70 37.0 / 40.6; long and flat,
+  // 17x29x400 28.7 / 35.7, 130x30x60 34.1 / 39.8; with eight slices a column, 66x66x64,
+  // they lost, 50.1 / 41.8, and have no instance)
   const bool tiles64 = sizeof(R) == 8 && !c->capturing && c->tile_where != kTilesNone && cg64_resident_ok(c, c->geo);
   if (!c->capturing && !tiles64) HMC_TRY(tune_cg<R>(c, ms, sigma, b));
   const R dm = (R)(c->delta * ms);
