@@ -1136,7 +1136,15 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (warp == 0) tmem_free(s_tmem, xalloc);
   }
-  if constexpr (CL) cluster_barrier();  // no block leaves while one that gave up may still be written to
+  if constexpr (CL) {
+    // no block leaves while it may still be written to: one that had its bytes has
+    // none on their way, one that gave up waits for all blocks' last stores to land
+    // (less than 1 us behind the barrier)
+    cluster_barrier();
+    if (done == CG_TIMEOUT)
+      for (const long long tw = clock64(); clock64() - tw < 50000LL;) {
+      }
+  }
   if (tid != 0) return;
   CGScal* sc = ts.sc;
   if (tile == 0) {
