@@ -48,9 +48,9 @@ static const void* cluster_kernel32(const TilePlan& p) {
 
 // us per iteration of a system on a cluster of 2^k blocks: the cells of its largest
 // tile, and the partials every warp sends to and takes from every block, twice. It
-// only ranks the choices. Fitted to 103 measured plans (5x5x16 to 36x36x48, odd and
-// even n; rms error 7 %, 18 % at most; the fastest cluster's choice costs 0.5 % on
-// average), for instance on 1, 2, 4, 8, 16 blocks (a dash: does not fit):
+// only ranks the choices. Fitted to 151 measured plans (4x43x20 to 36x36x48, odd and
+// even n; rms error 8 %; the cluster it ranks first is 0.2 % slower than the fastest on
+// average, 3.6 % at most), for instance on 1, 2, 4, 8, 16 blocks (a dash: does not fit):
 //   6x6x16 2.61, 2.36, 2.29, 2.33, 2.42   12x12x32 9.29, 4.47, 3.40, 2.74, 2.59
 //   13x13x32 -, 5.62, 4.04, 3.50, 2.85    18x18x48 -, -, 6.26, 4.11, 3.49
 //   24x24x48 -, -, -, 6.06, 4.23          25x25x48 -, -, -, 12.7, 7.24
@@ -58,7 +58,7 @@ static const void* cluster_kernel32(const TilePlan& p) {
 static double cluster_us(const TilePlan& p, const Geo& g, int k) {
   const double cols = (double)p.J * std::min(p.T, g.nt) * (g.n / p.cw);
   const double slope = (p.cw == 1 ? 1.35e-3 : 1.95e-3) + (p.S >= kXInMemory ? 1.25e-3 : 0.0);
-  return 2.0 + 0.05 * k + 0.0028 * (p.threads / 32) * (1 << k) + slope * cols;
+  return 1.95 + 0.07 * k + 0.0034 * (p.threads / 32) * (1 << k) + slope * cols;
 }
 
 // Tiles of one system for a cluster of cs blocks (cs a power of two): the split
