@@ -1,6 +1,6 @@
 // Resident-tile FP32 CG on thread block clusters (cg_tile.cuh): one cluster
 // solves one system, so a launch can hold any number of independent systems
-// and none waits for another. Plans, kernel instances and launches.
+// and none waits for another. Plans and launches.
 //
 // An exchange inside a cluster is a round of stores into the other blocks'
 // shared memory, each reporting its bytes to a barrier word there, and the wait
@@ -14,37 +14,12 @@
 #include <queue>
 #include <utility>
 
-#include "cg_tile.h"
+#include "cg32_cluster.cuh"
 #include "launch.cuh"
 
 namespace hmc {
 
-// Bytes between the padded arrays: the small one leaves room for several
-// blocks on an SM.
-constexpr int kStrideSmall = 12 * 1024, kStrideLarge = 44 * 1024;
-
-template <int CW, int S, int AS>
-__global__ void __launch_bounds__(tile_max_threads<float, CW, S>(), 1)
-    k_cg32_cluster(const TileSys* __restrict__ list, const __grid_constant__ TileSys one, unsigned extra, long long limit) {
-  extern __shared__ float4 s_tile[];
-  __shared__ TileSys ts;
-  static_assert(sizeof(TileSys) % 4 == 0, "copied by words");
-  const unsigned* src = list ? (const unsigned*)(list + blockIdx.x / cluster_size()) : (const unsigned*)&one;
-  for (unsigned i = threadIdx.x; i < sizeof(TileSys) / 4; i += blockDim.x) ((unsigned*)&ts)[i] = src[i];
-  __syncthreads();
-  cg_tile_solve<float, CW, S, true, AS>(ts, GridSync{nullptr, nullptr, nullptr, extra, limit}, (int)cluster_rank(), (char*)s_tile);
-}
-
-static const void* cluster_kernel32(const TilePlan& p) {
-#define HMC_CASE(cw_, s_)                                                          \
-  if (p.cw == cw_ && p.S == s_)                                                    \
-    return p.stride == kStrideSmall ? (const void*)k_cg32_cluster<cw_, s_, kStrideSmall> \
-                                    : (const void*)k_cg32_cluster<cw_, s_, kStrideLarge>;
-  HMC_CASE(1, 1) HMC_CASE(1, 2) HMC_CASE(1, 4) HMC_CASE(1, 8) HMC_CASE(1, 8 + kXInMemory)
-  HMC_CASE(2, 1) HMC_CASE(2, 2) HMC_CASE(2, 4) HMC_CASE(2, 4 + kXInMemory)
-#undef HMC_CASE
-  return nullptr;
-}
+static const void* cluster_kernel(const TilePlan& p, bool batch) { return batch ? cluster_kernel_batch(p) : cluster_kernel_of<false>(p); }
 
 // us per iteration of a system on a cluster of 2^k blocks: the cells of its largest
 // tile, and the partials every warp sends to and takes from every block, twice. It
@@ -138,8 +113,8 @@ static void cluster_waits(const hmc_ctx* c, unsigned* extra, long long* limit) {
 // How many clusters of the plan this GPU can run at a time with an SM to each block.
 // (Blocks of small tiles can share one, but then take longer: counted that way, 100
 // systems of 4x4 to 8x8 cells take 3.8 ms instead of 3.35.)
-static int cluster_count(const hmc_ctx* c, const TilePlan& p, int cs) {
-  const void* k = cluster_kernel32(p);
+static int cluster_count(const hmc_ctx* c, const TilePlan& p, int cs, bool batch) {
+  const void* k = cluster_kernel(p, batch);
   if (!k) return 0;
   if (!tile_allow_smem(c, k) ||
       (cs > 8 && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
@@ -159,10 +134,10 @@ static int cluster_count(const hmc_ctx* c, const TilePlan& p, int cs) {
   return n;
 }
 
-static ClusterPlans cluster_plans(const hmc_ctx* c, const Geo& g) {
+static ClusterPlans cluster_plans(const hmc_ctx* c, const Geo& g, bool batch) {
   ClusterPlans cp;
   for (int k = 0; k < 5; ++k) {
-    cp.count[k] = plan_cluster(c, g, 1 << k, &cp.p[k]) ? cluster_count(c, cp.p[k], 1 << k) : 0;
+    cp.count[k] = plan_cluster(c, g, 1 << k, &cp.p[k]) ? cluster_count(c, cp.p[k], 1 << k, batch) : 0;
     if (cp.count[k] < 1) cp.p[k].cw = 0;
     cp.us[k] = cp.p[k].cw ? cluster_us(cp.p[k], g, k) : 0.0;
   }
@@ -171,7 +146,7 @@ static ClusterPlans cluster_plans(const hmc_ctx* c, const Geo& g) {
 
 bool cg32_cluster_ok(hmc_ctx* c, const Geo& g) {
   if (c->cluster_log2 == -2) {
-    const ClusterPlans cp = cluster_plans(c, g);
+    const ClusterPlans cp = cluster_plans(c, g, false);
     c->cluster_log2 = -1;
     for (int k = 0; k < 5; ++k)
       if (cp.p[k].cw && (c->cluster_log2 < 0 || cp.us[k] < cp.us[c->cluster_log2])) c->cluster_log2 = k;
@@ -196,7 +171,7 @@ hmc_status cg32_cluster_launch(hmc_ctx* c, const Geo& g, float2* x, float2* r, C
   cudaLaunchAttribute attr;
   cluster_config(&cfg, &attr, p, 1 << c->cluster_log2, 1, c->stream);
   cudaError_t le = cudaSuccess;
-  HMC_TRY(launch_b(c, K_CG_RES32, 0.0, [&] { le = cudaLaunchKernelExC(&cfg, cluster_kernel32(p), args); }));
+  HMC_TRY(launch_b(c, K_CG_RES32, 0.0, [&] { le = cudaLaunchKernelExC(&cfg, cluster_kernel(p, false), args); }));
   if (le != cudaSuccess) return cuda_fail(c, le, "resident CG cluster launch");
   c->shape[K_CG_RES32].tiled = p.cw == 2 ? 4 : 0;  // reported as the design
   c->shape[K_CG_RES32].waves = -(1 << c->cluster_log2);
@@ -218,7 +193,7 @@ bool cg32_cluster_batch(hmc_ctx* c, const std::vector<Geo>& geos, const std::vec
   for (int i = 0; i < ns; ++i) {
     const std::array<int, 3> key{geos[i].n, geos[i].m, geos[i].nt};
     auto it = c->batch_plans.find(key);
-    if (it == c->batch_plans.end()) it = c->batch_plans.emplace(key, cluster_plans(c, geos[i])).first;
+    if (it == c->batch_plans.end()) it = c->batch_plans.emplace(key, cluster_plans(c, geos[i], true)).first;
     cp[i] = &it->second;
   }
   // For a time T every system takes the smallest cluster (the least SM time)
@@ -313,7 +288,7 @@ bool cg32_cluster_batch(hmc_ctx* c, const std::vector<Geo>& geos, const std::vec
     g->plans.push_back(p);
   }
   for (const ClusterGroup& g : *groups)
-    if (cluster_count(c, g.plan, 1 << g.log2) < 1) return false;
+    if (cluster_count(c, g.plan, 1 << g.log2, true) < 1) return false;
   return true;
 }
 
@@ -349,7 +324,7 @@ hmc_status cg32_cluster_batch_launch(hmc_ctx* c, const std::vector<ClusterGroup>
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr;
     cluster_config(&cfg, &attr, g.plan, 1 << g.log2, (int)g.sys.size(), c->side[i]);
-    const cudaError_t e = cudaLaunchKernelExC(&cfg, cluster_kernel32(g.plan), args);
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, cluster_kernel(g.plan, true), args);
     if (e != cudaSuccess) st = cuda_fail(c, e, "batched CG cluster launch");
     c->prof.launches[K_BATCH_CG32]++;
     first += (int)g.sys.size();

@@ -291,9 +291,10 @@ struct Red<double> {
 };
 
 // The scalars of a solve made of the sums: of type R, or (WIDE, FP32) with all bits of
-// the sums, alpha and beta rounded once from these. Clusters hold them wide, as the
-// other batched kernels hold FP64 ones; over all SMs they are FP32, as in the other
-// FP32 CG kernels of a single system (a trajectory at 102x102x64 158.6 ms, wide 162.9).
+// the sums, alpha and beta rounded once from these. Batches hold them wide, as the
+// other batched kernels hold FP64 ones; solves of a single system have FP32 scalars, as
+// in its other FP32 CG kernels (wide ones cost 0.1 us of 2.6 to 4.4 an iteration on
+// clusters of odd n, and at 102x102x64 4 ms of a trajectory's 159).
 template <typename R, bool WIDE>
 struct Scalars {
   using S = R;
@@ -503,8 +504,8 @@ constexpr int tile_max_threads() {
 
 // The solve of one system by the block `tile` of its group. sm: four padded
 // arrays AS bytes apart, the table of the padding (8 bytes a column; GT: in global
-// memory instead) and, for CL, the neighbours' r there.
-template <typename R, int CW, int INST, bool CL, int AS, bool GT = false>
+// memory instead) and, for CL, the neighbours' r there. WIDE: the scalars (Scalars).
+template <typename R, int CW, int INST, bool CL, int AS, bool GT = false, bool WIDE = false>
 __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync& gs, int tile, char* sm) {
   using LN = Lane<R, CW>;
   using L = typename LN::L;
@@ -691,7 +692,7 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
   // |r|^2 (of iteration i in s_rr[i & 1]), <p, A p> and the threshold are kept in shared
   // memory, as registers are short: by thread 0, read behind a barrier (CL) or by
   // thread 0 alone.
-  using SC = Scalars<R, CL>;
+  using SC = Scalars<R, WIDE>;
   R dm, sigma;
   TileScal<R>::load(ts.sc, dm, sigma);
   __shared__ typename SC::S s_rr[2], s_pap, s_thresh;
@@ -846,8 +847,8 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
     cluster_barrier();
   }
 
-  // Sum over the group. CL: in every thread. Otherwise in warp 0; the other
-  // warps run `edges` meanwhile.
+  // Sum over the group. CL: in every thread, which runs `edges` while the sums are on
+  // their way. Otherwise in warp 0; the other warps run `edges` meanwhile.
   auto exchange = [&](R loc, auto&& edges, T* out) -> bool {
     ++ep;
     if constexpr (CL) {
@@ -859,6 +860,7 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
         const unsigned a = (unsigned)__cvta_generic_to_shared(slots + me * nwarps + warp);
         st_remote(mapa(a, lane), wsum, mapa(bar, lane));
       }
+      edges();
       const long long tw = clock64();
       bool late = false;
       while (!bar_try(bar, parity) && !(late = clock64() - tw > gs.limit)) {
@@ -1007,9 +1009,12 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
         }
     }
     T tot;
-    if constexpr (CL) rr = s_rr[iter & 1];  // (at hand when the sum arrives)
-    bool ok = exchange(total(acc) + (sigma != R(0) ? sigma * total(accp) : R(0)),
-                       [&] { fetch_padding(Ug, false); }, &tot);
+    bool ok = exchange(total(acc) + (sigma != R(0) ? sigma * total(accp) : R(0)), [&] {
+      if constexpr (CL)
+        rr = s_rr[iter & 1];
+      else
+        fetch_padding(Ug, false);
+    }, &tot);
     // phases of the first slice of M
     if (ns > 0) {
       fa = PH::load(ph, k_first);
@@ -1082,13 +1087,15 @@ __device__ __forceinline__ void cg_tile_solve(const TileSys& ts, const GridSync&
     // next exchange has refilled it (the block's barrier in `exchange` orders
     // the reads of u above before these writes)
     decltype(SC::over(rr)) over{};
-    if constexpr (CL) {
-      rr = s_rr[iter & 1];
-      thresh = s_thresh;
-      over = SC::over(rr);
-    }
-    ok = exchange(total(accr),
-                  [&] { fetch_padding(rg, true); }, &tot);
+    ok = exchange(total(accr), [&] {
+      if constexpr (CL) {
+        rr = s_rr[iter & 1];
+        thresh = s_thresh;
+        over = SC::over(rr);
+      } else {
+        fetch_padding(rg, true);
+      }
+    }, &tot);
     if (CL || tid == 0) {
       if constexpr (!CL) {
         rr = s_rr[iter & 1];

@@ -56,11 +56,13 @@ def test_one_cluster(shape, cols):
 
 
 @pytest.mark.parametrize("shapes", [[(24, 24, 33), (7, 5, 9), (36, 36, 48), (25, 3, 17), (6, 6, 16), (1, 2, 3)],
-                                    [(64, 64, 40), (6, 6, 16), (9, 4, 12)]])
+                                    [(64, 64, 40), (6, 6, 16), (9, 4, 12)],
+                                    [(25, 25, 48)] * 10 + [(24, 24, 32)] * 12 + [(13, 13, 32)] * 12])
 def test_batched_clusters(shapes):
-    """A mixed batch with every system on a cluster of its own (first list), and
-    one with a lattice that fits no cluster (the cooperative kernels take the
-    whole batch): each system's true residual by the oracle's operator."""
+    """A mixed batch with every system on a cluster of its own (first list), one
+    with a lattice that fits no cluster (the cooperative kernels take the whole
+    batch), and one of more systems than there is room for at a time (small
+    clusters, long columns): each system's true residual by the oracle's operator."""
     need_gpu()
     import paper_1804_07195_gb300 as hmc
     import torch
